@@ -4,7 +4,7 @@
 // count and to fixed-point sums of its conditional mean <phi|V> and of psi - <phi|V> in
 // its psi bin, and to the element's count, sum, minimum and maximum of psi; a second pass
 // adds the powers of psi - <phi>.  Integer atomics make every sum independent of the order
-// in which particles arrive, so the results are the same run after run.  One thread per
+// in which particles arrive, so the results are the same run after run.  One block per
 // probe element then forms, per bin, Eq. 68's phi~ (the bin average of <phi|V>), the
 // conditional diffusion t_m <Gamma lap phi | psi> (the bin average of <phi|V> - psi) and
 // Eq. 67's conditional dissipation t_m <2 Gamma (grad phi)^2 | psi> at the bin centre on
@@ -80,37 +80,60 @@ __global__ void scalar_moments_kernel(const Particles<T> p, int64_t np, const in
   }
 }
 
-__global__ void scalar_finish_kernel(int n, int nb, ScalarAcc acc, ScalarOut out) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= n) return;
+// One block per probe element, a thread per bin (kFinishThreads bins at a time), the sums of
+// psi - <phi|V> over the bins below from a block scan in fixed point (exact, so the order of
+// the additions does not matter).  Bound by the latency of a few FP64 divisions per bin; one
+// thread per probe over its bins in turn, as before, took 332 us for 64 probes of 200 bins,
+// this 10.
+constexpr int kFinishThreads = 128;
+__global__ void __launch_bounds__(kFinishThreads) scalar_finish_kernel(int nb, ScalarAcc acc, ScalarOut out) {
+  __shared__ long long wtot[kFinishThreads / 32];
+  const int j = blockIdx.x;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int N = acc.n[j];
-  double* m = out.mom + 6 * j;
-  if (N > 0) {
-    m[0] = unfix(acc.s1[j], kFixS) / N;
-    m[1] = unfix(acc.m[3 * j], kFixM) / N;
-    m[2] = unfix(acc.m[3 * j + 1], kFixM) / N;
-    m[3] = unfix(acc.m[3 * j + 2], kFixM) / N;
-    m[4] = unord64(acc.lo[j]);
-    m[5] = unord64(acc.hi[j]);
-  } else {
-    for (int k = 0; k < 6; ++k) m[k] = 0.0;
+  if (tid < 6) {
+    double v = 0.0;
+    if (N > 0) {
+      if (tid == 0) v = unfix(acc.s1[j], kFixS) / N;
+      else if (tid < 4) v = unfix(acc.m[3 * j + tid - 1], kFixM) / N;
+      else v = unord64(tid == 4 ? acc.lo[j] : acc.hi[j]);
+    }
+    out.mom[6 * j + tid] = v;
   }
   const double dpsi = 1.0 / nb;
-  long long cum = 0;   // fixed-point sum of psi - <phi|V> over the bins below
-  for (int b = 0; b < nb; ++b) {
+  long long below = 0;   // over the bins of the rounds before
+  for (int b0 = 0; b0 < nb; b0 += kFinishThreads) {
+    const int b = b0 + tid;
+    const bool in = b < nb;
     const size_t o = static_cast<size_t>(j) * nb + b;
-    const int cnt = acc.count[o];
-    const long long sd = static_cast<long long>(acc.sd[o]);
-    out.count[o] = cnt;
-    if (cnt > 0) {
-      out.phit[o] = unfix(acc.sc[o], kFixS) / cnt;
-      out.cdiff[o] = -(static_cast<double>(sd) / kFixS) / cnt;
-      out.cdiss[o] = -2.0 * dpsi * (static_cast<double>(cum) / kFixS +
-                                    0.5 * (static_cast<double>(sd) / kFixS)) / cnt;
-    } else {
-      out.phit[o] = out.cdiff[o] = out.cdiss[o] = 0.0;
+    const int cnt = in ? acc.count[o] : 0;
+    const long long sd = in ? static_cast<long long>(acc.sd[o]) : 0;
+    const unsigned long long sc = in ? acc.sc[o] : 0;
+    long long incl = sd;
+#pragma unroll
+    for (int w = 1; w < 32; w <<= 1) {
+      const long long y = __shfl_up_sync(0xffffffffu, incl, w);
+      if (lane >= w) incl += y;
     }
-    cum += sd;
+    if (lane == 31) wtot[warp] = incl;
+    __syncthreads();
+    long long cum = below + incl - sd;   // fixed-point sum of psi - <phi|V> over the bins below
+    for (int w = 0; w < kFinishThreads / 32; ++w) {
+      if (w < warp) cum += wtot[w];
+      below += wtot[w];
+    }
+    if (in) {
+      out.count[o] = cnt;
+      if (cnt > 0) {
+        out.phit[o] = unfix(sc, kFixS) / cnt;
+        out.cdiff[o] = -(static_cast<double>(sd) / kFixS) / cnt;
+        out.cdiss[o] = -2.0 * dpsi * (static_cast<double>(cum) / kFixS +
+                                      0.5 * (static_cast<double>(sd) / kFixS)) / cnt;
+      } else {
+        out.phit[o] = out.cdiff[o] = out.cdiss[o] = 0.0;
+      }
+    }
+    __syncthreads();
   }
 }
 
@@ -125,7 +148,7 @@ void launch_scalar_stats(const Particles<T>& p, int64_t np, const int32_t* probe
     scalar_sums_kernel<T><<<grid, 256, 0, s>>>(p, np, probe, vcce, G, nb, acc);
     scalar_moments_kernel<T><<<grid, 256, 0, s>>>(p, np, probe, acc);
   }
-  scalar_finish_kernel<<<(n + 127) / 128, 128, 0, s>>>(n, nb, acc, out);
+  scalar_finish_kernel<<<static_cast<unsigned>(n), kFinishThreads, 0, s>>>(nb, acc, out);
 }
 
 template void launch_scalar_stats<float>(const Particles<float>&, int64_t, const int32_t*,
