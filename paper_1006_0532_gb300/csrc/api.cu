@@ -92,6 +92,9 @@ Model<T> model_of(const pdfx_params& p) {
   m.source_on = p.source_on;
   m.model = p.model;
   m.alpha = T(p.alpha);
+  m.nu2 = T(2.0 * p.nu);
+  m.s2c34 = T(std::sqrt(2.0 * p.C3 * p.C4));
+  m.src_r2 = T(p.src_r * p.src_r);
   return m;
 }
 
@@ -380,6 +383,9 @@ int do_step(Ctx& c, double dt, cudaStream_t s) {
     a.m = model_of<T>(c.prm);
     a.dt = T(dt);
     a.sdt = T(std::sqrt(dt));
+    a.nu2dt = a.m.nu2 * a.dt;
+    a.s2nusdt = a.m.s2nu * a.sdt;
+    a.s2c34sdt = a.m.s2c34 * a.sdt;
     a.stepc = c.dstep;
     a.corr = c.corr_pending ? c.corr : nullptr;   // consumed by this advance
     a.k0 = key0(c.prm);
@@ -514,21 +520,25 @@ int do_get_particles(Ctx& c, pdfx_soa* soa, int on_device, cudaStream_t s) {
   return rc;
 }
 
-// Element geometry in the working precision: node coordinates (canonical x) and 1 / (2 A_e);
-// the FP32 form stores each coordinate as an FP32 pair.
-void geo_of(const HostGeo& g, int32_t e, ElemGeo<double>& o) {
+// Element geometry in the working precision: node coordinates (canonical x; FP32 form: as
+// FP32 pairs), the edges' vectors and 1 / (2 A_e).
+void geo_nodes(const HostGeo& g, int32_t e, ElemGeo<double>& o) {
   for (int k = 0; k < 3; ++k) {
     o.x[k] = g.nx[3 * e + k];
     o.y[k] = g.vy[3 * e + k];
   }
-  o.inv2a = 1.0 / g.area2[e];
-  o.pad = 0.0;
+  o.pad = 0;
 }
-void geo_of(const HostGeo& g, int32_t e, const int32_t* tri, double L, ElemGeo<float>& o) {
+void geo_nodes(const HostGeo& g, int32_t e, ElemGeo<float>& o) {
   for (int k = 0; k < 3; ++k) {
     pair_of(g.nx[3 * e + k], o.xh[k], o.xl[k]);
     pair_of(g.vy[3 * e + k], o.yh[k], o.yl[k]);
   }
+  o.pad[0] = o.pad[1] = 0.0f;
+}
+template <typename T>
+void geo_of(const HostGeo& g, int32_t e, const int32_t* tri, double L, ElemGeo<T>& o) {
+  geo_nodes(g, e, o);
   // edge opposite vertex k: counter-clockwise from a = k + 1 to b = k + 2; pivot at the
   // lower node id, vector from the pivot to the other node (minimum image in x)
   o.code = 0u;
@@ -536,14 +546,12 @@ void geo_of(const HostGeo& g, int32_t e, const int32_t* tri, double L, ElemGeo<f
     const int a = (k + 1) % 3, b = (k + 2) % 3;
     const bool flip = tri[3 * e + b] < tri[3 * e + a];
     const int p = flip ? b : a, q = flip ? a : b;
-    o.ex[k] = static_cast<float>(min_image(g.nx[3 * e + q] - g.nx[3 * e + p], L));
-    o.ey[k] = static_cast<float>(g.vy[3 * e + q] - g.vy[3 * e + p]);
+    o.ex[k] = static_cast<T>(min_image(g.nx[3 * e + q] - g.nx[3 * e + p], L));
+    o.ey[k] = static_cast<T>(g.vy[3 * e + q] - g.vy[3 * e + p]);
     o.code |= (static_cast<uint32_t>(p) | (flip ? 4u : 0u)) << (3 * k);
   }
-  o.inv2a = static_cast<float>(1.0 / g.area2[e]);
-  o.pad[0] = o.pad[1] = 0.0f;
+  o.inv2a = static_cast<T>(1.0 / g.area2[e]);
 }
-void geo_of(const HostGeo& g, int32_t e, const int32_t*, double, ElemGeo<double>& o) { geo_of(g, e, o); }
 void line_of(const double* src, Line<double>& o) {
   o.px = src[0]; o.py = src[1]; o.nx = src[2]; o.ny = src[3];
 }

@@ -17,11 +17,28 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 
+__device__ __forceinline__ bool nonneg(float x) { return x >= 0.0f; }
+__device__ __forceinline__ bool nonneg(double x) { return m64::nonneg(x); }
+// The index of the smallest of three numbers of which one is negative, the first among equals
+// (FP64 form: of negative doubles the smallest has the largest bits).
+__device__ __forceinline__ int lowest(float a, float b, float c) {
+  int k = 0;
+  float mn = a;
+  if (b < mn) { k = 1; mn = b; }
+  if (c < mn) k = 2;
+  return k;
+}
+__device__ __forceinline__ int lowest(double a, double b, double c) {
+  auto key = [](double v) { return m64::bits(v) < 0 ? static_cast<uint64_t>(m64::bits(v)) : 0ull; };
+  const uint64_t ka = key(a), kb = key(b), kc = key(c);
+  return kc > (kb > ka ? kb : ka) ? 2 : (kb > ka ? 1 : 0);
+}
+
 template <typename T>
 __device__ __forceinline__ bool inside(const ElemGeo<T>& g, const ElemTopo& t, const Pos<T>& P, T L) {
   T na, nb, nc;
   area_cross(g, t.n0, t.n1, t.n2, P, L, na, nb, nc);
-  return na >= T(0) && nb >= T(0) && nc >= T(0);
+  return nonneg(na) && nonneg(nb) && nonneg(nc);
 }
 
 // Sect. 3.6: walk to the neighbour opposite the lowest area coordinate (ties: lowest local
@@ -41,12 +58,9 @@ __device__ int walk(const AdvanceArgs<T>& a, int e0, Pos<T>& P, T (&U)[3], T L, 
     const ElemTopo t = a.topo[e];
     T la, lb, lc;   // 2 N^k: signs and order of the area coordinates
     area_cross(g, t.n0, t.n1, t.n2, P, L, la, lb, lc);
-    if (la >= T(0) && lb >= T(0) && lc >= T(0)) return e;
+    if (nonneg(la) && nonneg(lb) && nonneg(lc)) return e;
     if (hops >= kHopLimit) break;
-    int k = 0;
-    T mn = la;
-    if (lb < mn) { k = 1; mn = lb; }
-    if (lc < mn) k = 2;
+    const int k = lowest(la, lb, lc);
     const int nb = k == 0 ? t.nb0 : (k == 1 ? t.nb1 : t.nb2);
     if (nb < 0) {
       if (nb == -1) break;
@@ -81,14 +95,15 @@ __device__ int walk(const AdvanceArgs<T>& a, int e0, Pos<T>& P, T (&U)[3], T L, 
   return -1;
 }
 
-// q = lambda_A f_A + lambda_B f_B + lambda_C f_C for the 31 used field slots.
+// q = lambda_A f_A + lambda_B f_B + lambda_C f_C for the used field slots (FP64 form: 0 .. 29;
+// the wall frequency, slot 30, is interpolated where a wall needs it).
 __device__ __forceinline__ void interp_fields(const double* __restrict__ F, int na, int nb, int nc,
                                               double la, double lb, double lc, double* q) {
   const double2* A = reinterpret_cast<const double2*>(F + (size_t)kNF * na);
   const double2* B = reinterpret_cast<const double2*>(F + (size_t)kNF * nb);
   const double2* C = reinterpret_cast<const double2*>(F + (size_t)kNF * nc);
 #pragma unroll
-  for (int i = 0; i < 16; ++i) {
+  for (int i = 0; i < 15; ++i) {
     const double2 a = __ldg(A + i), b = __ldg(B + i), c = __ldg(C + i);
     q[2 * i] = la * a.x + lb * b.x + lc * c.x;
     q[2 * i + 1] = la * a.y + lb * b.y + lc * c.y;
@@ -109,25 +124,17 @@ __device__ __forceinline__ void interp_fields(const float* __restrict__ F, int n
   }
 }
 
-// Reciprocal, square root and cube root of the closure (Eqs. 11, 18, 25).  FP64 form: the
-// correctly rounded functions.  FP32 form: the hardware approximations (a few units in the
-// last place; the state tolerance of this form is 1e-5) called through CUDA's intrinsics;
-// arguments are positive or zero.
-__device__ __forceinline__ double trcp(double x) { return 1.0 / x; }
+// Reciprocal, square root and cube root of the closure (Eqs. 11, 18, 25), FP32 form: the
+// hardware approximations (a few units in the last place; the state tolerance of this form
+// is 1e-5) called through CUDA's intrinsics; arguments are positive or zero.
 __device__ __forceinline__ float trcp(float x) { return __fdividef(1.0f, x); }
-__device__ __forceinline__ double tsqrt(double x) { return sqrt(x); }
 __device__ __forceinline__ float tsqrt(float x) { return x > 0.0f ? x * rsqrtf(x) : 0.0f; }
-__device__ __forceinline__ double tsqrt_ratio(double a, double b) { return sqrt(a / b); }
 __device__ __forceinline__ float tsqrt_ratio(float a, float b) { return tsqrt(a * trcp(b)); }
-__device__ __forceinline__ double tcbrt(double x) { return cbrt(x); }
 __device__ __forceinline__ float tcbrt(float x) { return exp2f(__log2f(x) * (1.0f / 3.0f)); }
 
 // Box & Muller (1958) for the step's six Gaussians: FP64 form as everywhere; FP32 form with
 // the hardware logarithm, square root and sine/cosine (CUDA intrinsics), the angle taken in
 // (-pi, pi) where they are most accurate: (cos, sin)(2 pi u) = -(cos, sin)(2 pi (u - 1/2)).
-__device__ __forceinline__ void step_gaussians(uint32_t w1, uint32_t w2, double& g1, double& g2) {
-  box_muller(w1, w2, g1, g2);
-}
 __device__ __forceinline__ void step_gaussians(uint32_t w1, uint32_t w2, float& g1, float& g2) {
   const float r = tsqrt(-2.0f * __logf(uniform01(w1, 0.0f)));
   float sn, cs;
@@ -138,10 +145,31 @@ __device__ __forceinline__ void step_gaussians(uint32_t w1, uint32_t w2, float& 
 __device__ __forceinline__ double texp(double x) { return exp(x); }
 __device__ __forceinline__ float texp(float x) { return expf(x); }
 
-template <typename T>
-__device__ __forceinline__ bool finite(T v) { return isfinite(v); }
-__device__ __forceinline__ double pos_lead(const Pos<double>& P) { return P.x + P.y; }
-__device__ __forceinline__ float pos_lead(const Pos<float>& P) { return P.xh + P.yh; }
+// Whether a particle's new state is finite: a sum of finite terms of this size is, a NaN or
+// infinity anywhere is not.  FP64 form: settled on the exponents unless one is at the top.
+__device__ __forceinline__ bool state_finite(const Pos<float>& P, const float (&U)[3], float w, float psi) {
+  return isfinite(P.xh + P.yh + U[0] + U[1] + U[2] + w + psi);
+}
+__device__ __forceinline__ bool state_finite(const Pos<double>& P, const double (&U)[3], double w, double psi) {
+  const int top = 0x7fc00000;   // 2^1021
+  auto e = [](double v) { return m64::hi_word(v) & 0x7fffffff; };
+  const int m = max(max(max(e(P.x), e(P.y)), max(e(U[0]), e(U[1]))), max(max(e(U[2]), e(w)), e(psi)));
+  return m < top || isfinite(P.x + P.y + U[0] + U[1] + U[2] + w + psi);
+}
+// Whether a particle lies in the source disc (Sect. 4.1.2).  FP64 form: a coordinate's high
+// word above the radius's settles most.
+__device__ __forceinline__ bool in_source(const Model<float>& M, const Pos<float>& P, float L) {
+  const float sx = rel_x(P, M.src_x, M.src_xl, L), sy = rel_y(P, M.src_y, M.src_yl);
+  return sx * sx + sy * sy <= M.src_r * M.src_r;
+}
+__device__ __forceinline__ bool in_source(const Model<double>& M, const Pos<double>& P, double L) {
+  const int hr = m64::hi_word(M.src_r) & 0x7fffffff;
+  const double sy = rel_y(P, M.src_y, M.src_yl);
+  if ((m64::hi_word(sy) & 0x7fffffff) > hr) return false;
+  const double sx = rel_x(P, M.src_x, M.src_xl, L);
+  if ((m64::hi_word(sx) & 0x7fffffff) > hr) return false;
+  return sx * sx + sy * sy <= M.src_r2;
+}
 
 __device__ __forceinline__ void warp_count(unsigned long long* diag, int slot, int v) {
   const unsigned s = __reduce_add_sync(kFull, static_cast<unsigned>(v));
@@ -193,8 +221,7 @@ __device__ __forceinline__ int finish_update(const AdvanceArgs<T>& a, const Mode
     }
   }
   pos_wrap(Pn, L);
-  // a sum of finite terms of this size is finite; a NaN or infinity anywhere is not
-  if (!finite(pos_lead(Pn) + Un[0] + Un[1] + Un[2] + wn + psin)) f.nf = 1;
+  if (!state_finite(Pn, Un, wn, psin)) f.nf = 1;
 
   int hops = 0, fb = 0, brute = 0, refl = 0;
   int e_new = walk(a, e, Pn, Un, L, hops, fb, brute, refl);
@@ -206,9 +233,9 @@ __device__ __forceinline__ int finish_update(const AdvanceArgs<T>& a, const Mode
     f.fs = 1;
     pos_wrap(Pn, L);
   }
-  if (M.source_on) {
-    const T sx = rel_x(Pn, M.src_x, M.src_xl, L), sy = rel_y(Pn, M.src_y, M.src_yl);
-    if (sx * sx + sy * sy <= M.src_r * M.src_r) { psin = T(1); f.src = 1; }
+  if (M.source_on && in_source(M, Pn, L)) {
+    psin = T(1);
+    f.src = 1;
   }
   if (e_new < 0) {
     // counted in the old element for now; the brute-force kernel moves it (or flags it)
@@ -267,6 +294,87 @@ __device__ __forceinline__ void count_update(const AdvanceArgs<T>& a, bool valid
   if (f.hop_bin > 0) atomicAdd(bc + kDiagHopHist0 + f.hop_bin, 1u);
 }
 
+// The FP64 form's new velocity, position, frequency and scalar before the walls (Eqs. 7, 27,
+// 19, 24 with the closure of Eqs. 11, 18, 20, 25), from the fields q at the particle.  The
+// same equations as the FP32 form's below, arranged for the fewest FP64 operations: at 64
+// cycles of a scheduler's FP64 pipe each they are the kernel's time.  C0 enters only as
+// C0 eps = -2/3 wp_ij <u_i u_j> / k; time-step factors are formed once; comparisons are on
+// the bits; the elementary functions are math64.h's.  The kernel takes 396 FP64 warp
+// instructions per 32 particles, its pipe 88% busy: 3.6 ms for 5.0M particles on the
+// 50,000-triangle channel, against 6.7 ms with the library's functions, divisions, edge
+// vectors formed per particle and comparisons in FP64.
+struct Step64 {
+  double dt, sdt, nu2dt, s2nusdt, s2c34sdt;
+};
+__device__ __forceinline__ void update_f64(const Model<double>& M, const Step64& D, const double* q,
+                                           const double (&U0)[3], double w0, double psi0, double phic,
+                                           const uint4& r0, const uint4& r1, Pos<double>& P, double (&Un)[3],
+                                           double& wn, double& psin, StepFlags& f) {
+  const double Om = q[29];
+  double k = 0.5 * (q[23] + q[24] + q[25]);
+  if (m64::below_pos(k, 1e-30)) k = 1e-30;
+  double eps = Om * (k + M.nuCT2 * Om);
+  if (m64::below_pos(eps, 1e-30)) eps = 1e-30;
+  const double ik = m64::rcp(k), ieps = m64::rcp(eps);
+  double c0e;   // C0 eps, clamped at zero under the root and counted
+  if (M.c0_mode == 1) {
+    c0e = M.C0 * eps;
+  } else {
+    double s = q[14] * q[23];
+    s = fma(q[15], q[26], s); s = fma(q[16], q[27], s);
+    s = fma(q[17], q[26], s); s = fma(q[18], q[24], s); s = fma(q[19], q[28], s);
+    s = fma(q[20], q[27], s); s = fma(q[21], q[28], s); s = fma(q[22], q[25], s);
+    c0e = -2.0 / 3.0 * s * ik;
+  }
+  if (!m64::nonneg(c0e) && c0e < 0.0) { c0e = 0.0; f.c0 = 1; }
+  const double prod = -(q[23] * q[5] + q[26] * q[6] + q[26] * q[7] + q[24] * q[8] + q[27] * q[9] + q[28] * q[10]);
+  const double Somega = M.Cw2 - M.Cw1 * prod * ieps;
+  double itm;
+  if (M.tm_mode == 1) {
+    itm = 0.5 * M.Cphi * eps * ik;
+  } else {
+    auto less = [](double a, double b) { return m64::bits(a) < m64::bits(b); };   // positive times
+    const double kt = k * ieps, kol = M.CT * m64::root(M.nu * ieps);
+    double tm = less(kol, kt) ? kt : kol;
+    const double ddx = rel_x(P, M.src_x, M.src_xl, M.period_x), ddy = rel_y(P, M.src_y, M.src_yl);
+    const double Uc2 = q[0] * q[0] + q[1] * q[1] + q[2] * q[2];
+    if (m64::bits(Uc2) > 0) {
+      const double a1 = M.cs_r2 * m64::rcbrt(eps) + M.Ct * m64::root((ddx * ddx + ddy * ddy) * m64::rcp(Uc2));
+      if (less(a1, tm)) tm = a1;
+    }
+    itm = m64::rcp(tm);
+  }
+  double xi[6];
+  box_muller(r0.x, r0.y, xi[0], xi[1]);
+  box_muller(r0.z, r0.w, xi[2], xi[3]);
+  box_muller(r1.x, r1.y, xi[4], xi[5]);
+  const double wx = D.s2nusdt * xi[0], wy = D.s2nusdt * xi[1];   // sqrt(2 nu) dW, shared by Eqs. 7 and 27
+  const double dU[3] = {U0[0] - q[0], U0[1] - q[1], U0[2] - q[2]};
+  const double sc = m64::root(c0e) * D.sdt, he = -0.5 * eps, ikdt = ik * D.dt;
+#pragma unroll
+  for (int r = 0; r < 3; ++r) {
+    // the terms join the velocity one by one in the order of the equations, as they do in the
+    // FP32 form: near a wall (G dt > 1) a step amplifies whatever rounding it is given
+    double u = r < 2 ? fma(-D.dt, q[3 + r], U0[r]) : U0[r];
+    u = fma(D.nu2dt, q[11 + r], u);
+    u += fma(q[6 + 2 * r], wy, q[5 + 2 * r] * wx);
+    double g = he * dU[r];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) g = fma(q[14 + 3 * r + c], dU[c], g);
+    u = fma(g, ikdt, u);
+    Un[r] = fma(sc, xi[2 + r], u);
+  }
+  P.x = fma(U0[0], D.dt, P.x) + wx;
+  P.y = fma(U0[1], D.dt, P.y) + wy;
+  const double wpos = m64::bits(w0) > 0 ? w0 : 0.0;
+  const double Omdt = Om * D.dt;
+  wn = fma(-(M.C3 * Omdt), w0 - Om, w0);
+  wn = fma(-(Somega * Omdt), w0, wn);
+  wn = fma(fabs(Om) * (D.s2c34sdt * m64::root(wpos)), xi[5], wn);
+  if (!m64::nonneg(wn) && wn < 0.0) { wn = -wn; f.oref = 1; }
+  psin = fma(-(psi0 - phic), D.dt * itm, psi0);
+}
+
 // FP32: 4 blocks of 256 per SM (64 registers); FP64: 2 blocks.  BATCH: model constants and
 // Philox key of the particle's instance (that of its element) instead of a.m, a.k0, a.k1.
 // Tiles of blockDim.x particles, one particle per thread: block b takes the consecutive tiles
@@ -314,99 +422,121 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) advance_kernel(co
       }
       T q[kNF];
       interp_fields(a.fields, tp.n0, tp.n1, tp.n2, la, lb, lc, q);
-      const T Um[3] = {q[0], q[1], q[2]};
-      const T dP[3] = {q[3], q[4], T(0)};
-      T R[3][3];
-      R[0][0] = q[23]; R[1][1] = q[24]; R[2][2] = q[25];
-      R[0][1] = R[1][0] = q[26];
-      R[0][2] = R[2][0] = q[27];
-      R[1][2] = R[2][1] = q[28];
-      const T Om = q[29];
-
-      // k and Eq. 18 (floored at 1e-30 so a particle on a wall keeps finite coefficients)
-      T k = T(0.5) * (R[0][0] + R[1][1] + R[2][2]);
-      if (k < T(1e-30)) k = T(1e-30);
-      T eps = Om * (k + M.nuCT2 * Om);
-      if (eps < T(1e-30)) eps = T(1e-30);
-      const T ik = trcp(k), ieps = trcp(eps);
-      // Eq. 11
-      T C0;
-      if (M.c0_mode == 1) {
-        C0 = M.C0;
+      const T dt = a.dt;
+      uint32_t step;
+      // the walls' uniforms, the first line's and a corner element's second line's (FP64 form:
+      // their words, converted where a wall needs them)
+      T eta = T(0), eta2 = T(0);
+      uint32_t etaw[2] = {0u, 0u};
+      T Un[3], wn, psin;
+      Pos<T> Pn = P0;
+      if constexpr (sizeof(T) == 8) {
+        // Sect. 3.9: six Gaussians and the walls' uniforms
+        step = *a.stepc;
+        const uint4 r0 = philox(make_uint4(pid, step, kPurStep, 0u), k0, k1);
+        const uint4 r1 = philox(make_uint4(pid, step, kPurStep, 1u), k0, k1);
+        etaw[0] = r1.z;
+        etaw[1] = r1.w;
+        const T phic = static_cast<T>(a.vcce[(size_t)e * a.G + cpi]);   // conditional mean of the bin
+        Step64 D{a.dt, a.sdt, a.nu2dt, a.s2nusdt, a.s2c34sdt};
+        if (BATCH) {
+          D.nu2dt = M.nu2 * a.dt;
+          D.s2nusdt = M.s2nu * a.sdt;
+          D.s2c34sdt = M.s2c34 * a.sdt;
+        }
+        update_f64(M, D, q, U0, w0, psi0, phic, r0, r1, Pn, Un, wn, psin, f);
       } else {
-        T s = T(0);
+        const T Um[3] = {q[0], q[1], q[2]};
+        const T dP[3] = {q[3], q[4], T(0)};
+        T R[3][3];
+        R[0][0] = q[23]; R[1][1] = q[24]; R[2][2] = q[25];
+        R[0][1] = R[1][0] = q[26];
+        R[0][2] = R[2][0] = q[27];
+        R[1][2] = R[2][1] = q[28];
+        const T Om = q[29];
+
+        // k and Eq. 18 (floored at 1e-30 so a particle on a wall keeps finite coefficients)
+        T k = T(0.5) * (R[0][0] + R[1][1] + R[2][2]);
+        if (k < T(1e-30)) k = T(1e-30);
+        T eps = Om * (k + M.nuCT2 * Om);
+        if (eps < T(1e-30)) eps = T(1e-30);
+        const T ik = trcp(k), ieps = trcp(eps);
+        // Eq. 11
+        T C0;
+        if (M.c0_mode == 1) {
+          C0 = M.C0;
+        } else {
+          T s = T(0);
+#pragma unroll
+          for (int r = 0; r < 3; ++r)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) s += q[14 + 3 * r + c] * R[r][c];
+          C0 = T(-2) / T(3) * s * ik * ieps;
+        }
+        // production P = -<u_i u_j> d<U_i>/dx_j (x, y) and Eq. 20
+        T prod = T(0);
 #pragma unroll
         for (int r = 0; r < 3; ++r)
 #pragma unroll
-          for (int c = 0; c < 3; ++c) s += q[14 + 3 * r + c] * R[r][c];
-        C0 = T(-2) / T(3) * s * ik * ieps;
-      }
-      // production P = -<u_i u_j> d<U_i>/dx_j (x, y) and Eq. 20
-      T prod = T(0);
-#pragma unroll
-      for (int r = 0; r < 3; ++r)
-#pragma unroll
-        for (int c = 0; c < 2; ++c) prod -= R[r][c] * q[5 + 2 * r + c];
-      const T Somega = M.Cw2 - M.Cw1 * prod * ieps;
-      // 1 / t_m: Eq. 25, or the IEM time scale t_m = 2k / (C_phi eps)
-      T itm;
-      if (M.tm_mode == 1) {
-        itm = T(0.5) * M.Cphi * eps * ik;
-      } else {
-        const T kt = k * ieps, kol = M.CT * tsqrt(M.nu * ieps);
-        const T a2 = kt > kol ? kt : kol;
-        const T ddx = rel_x(P0, M.src_x, M.src_xl, L), ddy = rel_y(P0, M.src_y, M.src_yl);
-        const T Uc2 = Um[0] * Um[0] + Um[1] * Um[1] + Um[2] * Um[2];
-        T tm = a2;
-        if (Uc2 > T(0)) {
-          const T a1 = M.cs_r2 * tcbrt(ieps) + M.Ct * tsqrt_ratio(ddx * ddx + ddy * ddy, Uc2);
-          tm = a1 < a2 ? a1 : a2;
+          for (int c = 0; c < 2; ++c) prod -= R[r][c] * q[5 + 2 * r + c];
+        const T Somega = M.Cw2 - M.Cw1 * prod * ieps;
+        // 1 / t_m: Eq. 25, or the IEM time scale t_m = 2k / (C_phi eps)
+        T itm;
+        if (M.tm_mode == 1) {
+          itm = T(0.5) * M.Cphi * eps * ik;
+        } else {
+          const T kt = k * ieps, kol = M.CT * tsqrt(M.nu * ieps);
+          const T a2 = kt > kol ? kt : kol;
+          const T ddx = rel_x(P0, M.src_x, M.src_xl, L), ddy = rel_y(P0, M.src_y, M.src_yl);
+          const T Uc2 = Um[0] * Um[0] + Um[1] * Um[1] + Um[2] * Um[2];
+          T tm = a2;
+          if (Uc2 > T(0)) {
+            const T a1 = M.cs_r2 * tcbrt(ieps) + M.Ct * tsqrt_ratio(ddx * ddx + ddy * ddy, Uc2);
+            tm = a1 < a2 ? a1 : a2;
+          }
+          itm = trcp(tm);
         }
-        itm = trcp(tm);
-      }
 
-      // Sect. 3.9: six Gaussians and eta
-      const uint32_t step = *a.stepc;
-      const uint4 r0 = philox(make_uint4(pid, step, kPurStep, 0u), k0, k1);
-      const uint4 r1 = philox(make_uint4(pid, step, kPurStep, 1u), k0, k1);
-      T xi[6];
-      step_gaussians(r0.x, r0.y, xi[0], xi[1]);
-      step_gaussians(r0.z, r0.w, xi[2], xi[3]);
-      step_gaussians(r1.x, r1.y, xi[4], xi[5]);
-      const T eta = uniform01(r1.z, T(0));     // first wall line
-      const T eta2 = uniform01(r1.w, T(0));    // second wall line (a corner element)
-      const T dt = a.dt;
-      const T sdt = a.sdt;
-      const T dWx = sdt * xi[0], dWy = sdt * xi[1];
-      const T s2nu = M.s2nu;
+        // Sect. 3.9: six Gaussians and eta
+        step = *a.stepc;
+        const uint4 r0 = philox(make_uint4(pid, step, kPurStep, 0u), k0, k1);
+        const uint4 r1 = philox(make_uint4(pid, step, kPurStep, 1u), k0, k1);
+        T xi[6];
+        step_gaussians(r0.x, r0.y, xi[0], xi[1]);
+        step_gaussians(r0.z, r0.w, xi[2], xi[3]);
+        step_gaussians(r1.x, r1.y, xi[4], xi[5]);
+        eta = uniform01(r1.z, T(0));     // first wall line
+        eta2 = uniform01(r1.w, T(0));    // second wall line (a corner element)
+        const T sdt = a.sdt;
+        const T dWx = sdt * xi[0], dWy = sdt * xi[1];
+        const T s2nu = M.s2nu;
 
-      // Eq. 27 (C0 eps < 0 is clamped under the root and counted);
-      // G_ij (U_j - <U_j>) = (wp_ij (U_j - <U_j>) - eps/2 (U_i - <U_i>)) / k  (Eq. 11)
-      T c0e = C0 * eps;
-      if (c0e < T(0)) { c0e = T(0); f.c0 = 1; }
-      const T sc0e = tsqrt(c0e) * sdt;
-      const T dU[3] = {U0[0] - Um[0], U0[1] - Um[1], U0[2] - Um[2]};
-      T Un[3];
+        // Eq. 27 (C0 eps < 0 is clamped under the root and counted);
+        // G_ij (U_j - <U_j>) = (wp_ij (U_j - <U_j>) - eps/2 (U_i - <U_i>)) / k  (Eq. 11)
+        T c0e = C0 * eps;
+        if (c0e < T(0)) { c0e = T(0); f.c0 = 1; }
+        const T sc0e = tsqrt(c0e) * sdt;
+        const T dU[3] = {U0[0] - Um[0], U0[1] - Um[1], U0[2] - Um[2]};
 #pragma unroll
-      for (int r = 0; r < 3; ++r) {
-        const T base = U0[r] - dP[r] * dt + T(2) * M.nu * q[11 + r] * dt +
-                       s2nu * (q[5 + 2 * r] * dWx + q[6 + 2 * r] * dWy);
-        T gsum = -T(0.5) * eps * dU[r];
+        for (int r = 0; r < 3; ++r) {
+          const T base = U0[r] - dP[r] * dt + T(2) * M.nu * q[11 + r] * dt +
+                         s2nu * (q[5 + 2 * r] * dWx + q[6 + 2 * r] * dWy);
+          T gsum = -T(0.5) * eps * dU[r];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) gsum += q[14 + 3 * r + c] * dU[c];
-        Un[r] = base + gsum * ik * dt + sc0e * xi[2 + r];
+          for (int c = 0; c < 3; ++c) gsum += q[14 + 3 * r + c] * dU[c];
+          Un[r] = base + gsum * ik * dt + sc0e * xi[2 + r];
+        }
+        // Eq. 7 (same dW as Eq. 27)
+        pos_move(Pn, U0[0], U0[1], dt, s2nu, dWx, dWy);
+        // Eq. 19, reflected at zero
+        const T wpos = w0 > T(0) ? w0 : T(0);
+        wn = w0 - M.C3 * Om * (w0 - Om) * dt - Somega * Om * w0 * dt +
+               tsqrt(T(2) * M.C3 * M.C4 * Om * Om * wpos) * (sdt * xi[5]);
+        if (wn < T(0)) { wn = -wn; f.oref = 1; }
+        // Eq. 24 with the conditional mean of the particle's bin
+        const T phic = static_cast<T>(a.vcce[(size_t)e * a.G + cpi]);
+        psin = psi0 - (psi0 - phic) * dt * itm;
       }
-      // Eq. 7 (same dW as Eq. 27)
-      Pos<T> Pn = P0;
-      pos_move(Pn, U0[0], U0[1], dt, s2nu, dWx, dWy);
-      // Eq. 19, reflected at zero
-      const T wpos = w0 > T(0) ? w0 : T(0);
-      T wn = w0 - M.C3 * Om * (w0 - Om) * dt - Somega * Om * w0 * dt +
-             tsqrt(T(2) * M.C3 * M.C4 * Om * Om * wpos) * (sdt * xi[5]);
-      if (wn < T(0)) { wn = -wn; f.oref = 1; }
-      // Eq. 24 with the conditional mean of the particle's bin
-      const T phic = static_cast<T>(a.vcce[(size_t)e * a.G + cpi]);
-      T psin = psi0 - (psi0 - phic) * dt * itm;
 
       // Sect. 3.8: wall elements only; each wall line in turn (a corner element has two),
       // the second from the position after the first's reflection
@@ -424,6 +554,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) advance_kernel(co
             hit = true;
           } else {
             const T dd0 = d0 > T(0) ? d0 : T(0);
+            if constexpr (sizeof(T) == 8) eta = eta2 = uniform01(etaw[j], T(0));
             hit = (j == 0 ? eta : eta2) < texp(-dd0 * d1 / (M.nu * dt));   // Eqs. 53, 55
           }
           if (hit) {
@@ -435,6 +566,9 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) advance_kernel(co
           f.wall = 1;
           Un[0] = Un[1] = Un[2] = T(0);                  // Eq. 56
           int ex = 0;                                    // Eq. 58
+          if constexpr (sizeof(T) == 8)
+            q[30] = la * a.fields[(size_t)kNF * tp.n0 + 30] + lb * a.fields[(size_t)kNF * tp.n1 + 30] +
+                    lc * a.fields[(size_t)kNF * tp.n2 + 30];
           wn = gamma_draw<T>(k0, k1, pid, step, kPurWallGamma, T(1) / M.C4, M.C4 * q[30], &ex);
           f.gex = ex;
         }

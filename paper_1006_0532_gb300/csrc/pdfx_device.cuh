@@ -5,6 +5,8 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "math64.h"
+
 namespace pdfx {
 
 constexpr int kNF = 32;            // nodal field slots
@@ -34,15 +36,19 @@ constexpr int kBruteCap = 4096;    // particles per step that may need the brute
 // FP32 spacings of y).
 template <typename T>
 struct ElemGeo;
-template <>
-struct __align__(64) ElemGeo<double> {
-  double x[3], y[3], inv2a, pad;
-};
-// The FP32 form also keeps each edge's vector in FP32, from the edge's lower-numbered node
-// (its pivot) to the other, computed once in FP64 from the nodes' coordinates: the same
+//
+// Both keep each edge's vector, from the edge's lower-numbered node (its pivot) to the other,
+// computed once in FP64 from the nodes' coordinates (and in the FP32 form rounded): the same
 // numbers for both elements of the edge.  code holds, for the edge opposite local vertex k,
 // the pivot's local index (bits 3k, 3k + 1) and whether the pivot is the edge's second
 // node in counter-clockwise order (bit 3k + 2, the cross product's sign flips).
+template <>
+struct __align__(16) ElemGeo<double> {
+  double x[3], y[3];
+  double ex[3], ey[3];
+  double inv2a;
+  uint32_t code, pad;
+};
 template <>
 struct __align__(16) ElemGeo<float> {
   float xh[3], yh[3], xl[3], yl[3];
@@ -115,9 +121,9 @@ __device__ __forceinline__ float uniform01(uint32_t w, float) {
 
 // Box & Muller (1958): two independent N(0, 1) from two uniform words.
 __device__ __forceinline__ void box_muller(uint32_t w1, uint32_t w2, double& g1, double& g2) {
-  const double r = sqrt(-2.0 * log(uniform01(w1, 0.0)));
+  const double r = m64::root(m64::minus_two_log(w1));
   double s, c;
-  sincospi(2.0 * uniform01(w2, 0.0), &s, &c);
+  m64::turn(w2, c, s);
   g1 = r * c;
   g2 = r * s;
 }
@@ -202,12 +208,20 @@ __device__ __forceinline__ double node_y(const ElemGeo<double>& g, int k) { retu
 __device__ __forceinline__ double node_x(const ElemGeo<float>& g, int k) { return pair_value(g.xh[k], g.xl[k]); }
 __device__ __forceinline__ double node_y(const ElemGeo<float>& g, int k) { return pair_value(g.yh[k], g.yl[k]); }
 
-// Node m minus node k (minimum image in x), in the working precision.
-__device__ __forceinline__ void node_vec(const ElemGeo<double>& g, int k, int m, double L, double& ex,
-                                         double& ey) {
-  ex = min_image(g.x[m] - g.x[k], L);
-  ey = g.y[m] - g.y[k];
+// min_image and wrap_period of the FP64 form, their tests on the bits (a comparison takes the
+// FP64 pipe like any other operation): d stays while its high word is below L / 2's, which a
+// particle near its element's nodes meets unless the seam lies between.
+__device__ __forceinline__ double near_image(double d, double L) {
+  const int32_t hl = m64::hi_word(L);
+  if (hl > 0 && (m64::hi_word(d) & 0x7fffffff) >= hl - 0x100000) return min_image(d, L);
+  return d;
 }
+__device__ __forceinline__ double near_period(double x, double L) {
+  const int64_t bx = m64::bits(x), bl = m64::bits(L);
+  return bl > 0 && (bx < 0 || bx >= bl) ? wrap_period(x, L) : x;
+}
+
+// Node m minus node k (minimum image in x), in the working precision.
 __device__ __forceinline__ void node_vec(const ElemGeo<float>& g, int k, int m, float L, float& ex,
                                          float& ey) {
   ex = __fadd_rn(min_image(__fsub_rn(g.xh[m], g.xh[k]), L), __fsub_rn(g.xl[m], g.xl[k]));
@@ -216,7 +230,7 @@ __device__ __forceinline__ void node_vec(const ElemGeo<float>& g, int k, int m, 
 // Particle minus node k (minimum image in x), in the working precision.
 __device__ __forceinline__ void node_rel(const ElemGeo<double>& g, int k, const Pos<double>& P, double L,
                                          double& dx, double& dy) {
-  dx = min_image(P.x - g.x[k], L);
+  dx = near_image(P.x - g.x[k], L);
   dy = P.y - g.y[k];
 }
 __device__ __forceinline__ void node_rel(const ElemGeo<float>& g, int k, const Pos<float>& P, float L,
@@ -227,7 +241,7 @@ __device__ __forceinline__ void node_rel(const ElemGeo<float>& g, int k, const P
 
 // Particle minus a point given in FP64 (FP32 form: as the pair (ph, pl)), minimum image in x.
 __device__ __forceinline__ double rel_x(const Pos<double>& P, double px, double, double L) {
-  return min_image(P.x - px, L);
+  return near_image(P.x - px, L);
 }
 __device__ __forceinline__ double rel_y(const Pos<double>& P, double py, double) { return P.y - py; }
 __device__ __forceinline__ float rel_x(const Pos<float>& P, float ph, float pl, float L) {
@@ -276,7 +290,7 @@ __device__ __forceinline__ void pos_reflect(Pos<float>& P, float d, float nx, fl
   pair_add(P.yh, P.yl, -(2.0f * d * ny));
 }
 // Periodic wrap of x into [0, L).
-__device__ __forceinline__ void pos_wrap(Pos<double>& P, double L) { P.x = wrap_period(P.x, L); }
+__device__ __forceinline__ void pos_wrap(Pos<double>& P, double L) { P.x = near_period(P.x, L); }
 __device__ __forceinline__ void pos_wrap(Pos<float>& P, float L) {
   if (L > 0.0f) {
     if (P.xh < 0.0f) pair_add(P.xh, P.xl, L);
@@ -302,43 +316,26 @@ __device__ __forceinline__ Pos<float> pos_of(double x, double y, float) {
 __device__ __forceinline__ double xmul(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ float xmul(float a, float b) { return __fmul_rn(a, b); }
 
-// (r_b - r_a) x (r_P - r_a) for the edge from local node a to local node b.  Its inputs are
-// node b - node a and P - node a, formed from the nodes' own coordinates and the particle's
-// alone, so both elements of the edge compute the same value.
-template <typename T>
-__device__ __forceinline__ T edge_cross(const ElemGeo<T>& g, int a, int b, const Pos<T>& P, T L) {
-  T ex, ey, dx, dy;
-  node_vec(g, a, b, L, ex, ey);
-  node_rel(g, a, P, L, dx, dy);
-  return xmul(ex, dy) - xmul(ey, dx);
-}
-
 // Twice the signed areas N^A, N^B, N^C (Eqs. 44-45, Fig. 1): for each vertex, the cross
 // product of the opposite edge with the vector from one end of that edge to the particle.
 // Each edge is pivoted at its lower-numbered node, so the two elements sharing an edge
 // evaluate it with identical rounding and opposite signs (watertight point location).
-__device__ __forceinline__ void area_cross(const ElemGeo<double>& g, int na, int nb, int nc,
-                                           const Pos<double>& P, double L, double& n0, double& n1,
-                                           double& n2) {
-  n0 = nb < nc ? edge_cross(g, 1, 2, P, L) : -edge_cross(g, 2, 1, P, L);   // edge B -> C
-  n1 = nc < na ? edge_cross(g, 2, 0, P, L) : -edge_cross(g, 0, 2, P, L);   // edge C -> A
-  n2 = na < nb ? edge_cross(g, 0, 1, P, L) : -edge_cross(g, 1, 0, P, L);   // edge A -> B
-}
-// FP32 form: the particle's offsets from the three nodes, then each edge's stored vector
-// crossed with the offset from its pivot.
-__device__ __forceinline__ void area_cross(const ElemGeo<float>& g, int, int, int, const Pos<float>& P,
-                                           float L, float& n0, float& n1, float& n2) {
-  float dx[3], dy[3];
+// The particle's offsets from the three nodes, formed from the nodes' own coordinates and the
+// particle's alone, then each edge's stored vector crossed with the offset from its pivot.
+template <typename T>
+__device__ __forceinline__ void area_cross(const ElemGeo<T>& g, int, int, int, const Pos<T>& P, T L, T& n0, T& n1,
+                                           T& n2) {
+  T dx[3], dy[3];
 #pragma unroll
   for (int m = 0; m < 3; ++m) node_rel(g, m, P, L, dx[m], dy[m]);
-  float n[3];
+  T n[3];
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     const uint32_t c = g.code >> (3 * k);
     const int pv = static_cast<int>(c & 3u);
-    const float px = pv == 0 ? dx[0] : (pv == 1 ? dx[1] : dx[2]);
-    const float py = pv == 0 ? dy[0] : (pv == 1 ? dy[1] : dy[2]);
-    const float cr = xmul(g.ex[k], py) - xmul(g.ey[k], px);
+    const T px = pv == 0 ? dx[0] : (pv == 1 ? dx[1] : dx[2]);
+    const T py = pv == 0 ? dy[0] : (pv == 1 ? dy[1] : dy[2]);
+    const T cr = xmul(g.ex[k], py) - xmul(g.ey[k], px);
     n[k] = (c & 4u) ? -cr : cr;
   }
   n0 = n[0];

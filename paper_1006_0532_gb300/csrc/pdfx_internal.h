@@ -23,6 +23,7 @@ struct Model {
   int c0_mode, tm_mode, interp_mode, source_on;
   int model;    // 0 full model; 1 Eqs. 46-47
   T alpha;      // Eq. 47
+  T nu2, s2c34, src_r2;   // FP64 form: 2 nu, sqrt(2 C3 C4), r0^2
 };
 
 // One instance of a batch (a grid of the union, its particles and its parameters).  A
@@ -93,6 +94,7 @@ struct AdvanceArgs {
   double* lost_rec;      // [kLostRecords][4]
   Model<T> m;
   T dt, sdt;    // time step and its square root
+  T nu2dt, s2nusdt, s2c34sdt;   // FP64 form, one instance: 2 nu dt, sqrt(2 nu dt), sqrt(2 C3 C4 dt)
   const uint32_t* stepc;   // step counter (Philox counter word) in device memory
   const double* corr;      // [ne][2] Eq. 31 correction of the last coupled step still to be
                            // applied to the velocities as they are read (nullptr: none)
