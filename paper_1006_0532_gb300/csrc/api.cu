@@ -351,7 +351,7 @@ int run_statistics(Ctx& c, bool counts_ready, bool allow_moves, bool force_resor
 }
 
 template <typename T>
-int do_step(Ctx& c, double dt, cudaStream_t s) {
+int do_step(Ctx& c, double dt, cudaStream_t s, bool coupled = false) {
   c.last_dt = dt;
   Particles<T> p = carve<T>(c.pbuf[c.cur], c.np);
   PDFX_CUDA(cudaMemsetAsync(c.plan.cnt, 0, sizeof(int32_t) * c.ne, s));
@@ -388,6 +388,7 @@ int do_step(Ctx& c, double dt, cudaStream_t s) {
     a.s2c34sdt = a.m.s2c34 * a.sdt;
     a.stepc = c.dstep;
     a.corr = c.corr_pending ? c.corr : nullptr;   // consumed by this advance
+    a.coupled = coupled ? 1 : 0;
     a.k0 = key0(c.prm);
     a.k1 = key1(c.prm);
     a.inst = c.K > 1 ? static_cast<const InstDev<T>*>(c.inst) : nullptr;
@@ -1240,7 +1241,7 @@ int do_coupled_step(Ctx& c, double dt, double Cp, double tol, int32_t max_iter, 
   const EWork w = ework(c);
   int32_t iw = 0, ip = 0;
   PDFX_TRY(update_wp_dev<T>(c, w, tol, max_iter, &iw, s));
-  PDFX_TRY(do_step<T>(c, dt, s));   // prediction (Eq. 27 and the other equations), control, statistics
+  PDFX_TRY(do_step<T>(c, dt, s, true));   // prediction (Eq. 27 and the other equations), control, statistics
   T* fields = static_cast<T*>(c.fields);
   launch_pressure_rhs<T>(c.fem, c.ne_off, c.ne_list, c.nmom, kNS, 1, c.P, fields, c.prm.nu, dt, Cp, w.prs,
                          w.src, w.flux, s);

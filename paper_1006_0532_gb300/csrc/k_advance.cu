@@ -124,17 +124,25 @@ __device__ __forceinline__ void interp_fields(const float* __restrict__ F, int n
   }
 }
 
-// Reciprocal, square root and cube root of the closure (Eqs. 11, 18, 25), FP32 form: the
-// hardware approximations (a few units in the last place; the state tolerance of this form
-// is 1e-5) called through CUDA's intrinsics; arguments are positive or zero.
+// Reciprocal, square root and cube root of the closure (Eqs. 11, 18, 25).  FP64 form (coupled
+// steps; update_f64 has its own): the correctly rounded functions.  FP32 form: the hardware
+// approximations (a few units in the last place; the state tolerance of this form is 1e-5)
+// called through CUDA's intrinsics; arguments are positive or zero.
+__device__ __forceinline__ double trcp(double x) { return 1.0 / x; }
 __device__ __forceinline__ float trcp(float x) { return __fdividef(1.0f, x); }
+__device__ __forceinline__ double tsqrt(double x) { return sqrt(x); }
 __device__ __forceinline__ float tsqrt(float x) { return x > 0.0f ? x * rsqrtf(x) : 0.0f; }
+__device__ __forceinline__ double tsqrt_ratio(double a, double b) { return sqrt(a / b); }
 __device__ __forceinline__ float tsqrt_ratio(float a, float b) { return tsqrt(a * trcp(b)); }
+__device__ __forceinline__ double tcbrt(double x) { return cbrt(x); }
 __device__ __forceinline__ float tcbrt(float x) { return exp2f(__log2f(x) * (1.0f / 3.0f)); }
 
 // Box & Muller (1958) for the step's six Gaussians: FP64 form as everywhere; FP32 form with
 // the hardware logarithm, square root and sine/cosine (CUDA intrinsics), the angle taken in
 // (-pi, pi) where they are most accurate: (cos, sin)(2 pi u) = -(cos, sin)(2 pi (u - 1/2)).
+__device__ __forceinline__ void step_gaussians(uint32_t w1, uint32_t w2, double& g1, double& g2) {
+  box_muller(w1, w2, g1, g2);
+}
 __device__ __forceinline__ void step_gaussians(uint32_t w1, uint32_t w2, float& g1, float& g2) {
   const float r = tsqrt(-2.0f * __logf(uniform01(w1, 0.0f)));
   float sn, cs;
@@ -303,9 +311,23 @@ __device__ __forceinline__ void count_update(const AdvanceArgs<T>& a, bool valid
 // instructions per 32 particles, its pipe 88% busy: 3.6 ms for 5.0M particles on the
 // 50,000-triangle channel, against 6.7 ms with the library's functions, divisions, edge
 // vectors formed per particle and comparisons in FP64.
+//
+// A coupled step does not take it (PLAIN): its pressure solve stops at the caller's tolerance
+// after some thousand conjugate-gradient iterations, which carry a change of the load's last
+// bits up to the size of that tolerance (1e-6 of P at tolerance 1e-6 on a graded grid), so
+// the particles it sees keep the arithmetic of the equations as written.  The advance is a
+// tenth of a coupled FP64 step.
 struct Step64 {
   double dt, sdt, nu2dt, s2nusdt, s2c34sdt;
 };
+// Box & Muller (1958) with math64.h's functions.
+__device__ __forceinline__ void gaussian_pair(uint32_t w1, uint32_t w2, double& g1, double& g2) {
+  const double r = m64::root(m64::minus_two_log(w1));
+  double c, s;
+  m64::turn(w2, c, s);
+  g1 = r * c;
+  g2 = r * s;
+}
 __device__ __forceinline__ void update_f64(const Model<double>& M, const Step64& D, const double* q,
                                            const double (&U0)[3], double w0, double psi0, double phic,
                                            const uint4& r0, const uint4& r1, Pos<double>& P, double (&Un)[3],
@@ -345,9 +367,9 @@ __device__ __forceinline__ void update_f64(const Model<double>& M, const Step64&
     itm = m64::rcp(tm);
   }
   double xi[6];
-  box_muller(r0.x, r0.y, xi[0], xi[1]);
-  box_muller(r0.z, r0.w, xi[2], xi[3]);
-  box_muller(r1.x, r1.y, xi[4], xi[5]);
+  gaussian_pair(r0.x, r0.y, xi[0], xi[1]);
+  gaussian_pair(r0.z, r0.w, xi[2], xi[3]);
+  gaussian_pair(r1.x, r1.y, xi[4], xi[5]);
   const double wx = D.s2nusdt * xi[0], wy = D.s2nusdt * xi[1];   // sqrt(2 nu) dW, shared by Eqs. 7 and 27
   const double dU[3] = {U0[0] - q[0], U0[1] - q[1], U0[2] - q[2]};
   const double sc = m64::root(c0e) * D.sdt, he = -0.5 * eps, ikdt = ik * D.dt;
@@ -381,7 +403,7 @@ __device__ __forceinline__ void update_f64(const Model<double>& M, const Step64&
 // [b per, (b + 1) per), per = ceil(tiles / gridDim.x), so that its particles, stored by
 // element, reuse one another's element, geometry and nodal-field lines in L1; the block's
 // counters are flushed once, after its last tile.
-template <typename T, bool BATCH>
+template <typename T, bool BATCH, bool PLAIN = false>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) advance_kernel(const AdvanceArgs<T> a) {
   __shared__ unsigned bc[kDiagCount];
   block_counts_clear(bc);
@@ -430,7 +452,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) advance_kernel(co
       uint32_t etaw[2] = {0u, 0u};
       T Un[3], wn, psin;
       Pos<T> Pn = P0;
-      if constexpr (sizeof(T) == 8) {
+      if constexpr (sizeof(T) == 8 && !PLAIN) {
         // Sect. 3.9: six Gaussians and the walls' uniforms
         step = *a.stepc;
         const uint4 r0 = philox(make_uint4(pid, step, kPurStep, 0u), k0, k1);
@@ -554,7 +576,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) advance_kernel(co
             hit = true;
           } else {
             const T dd0 = d0 > T(0) ? d0 : T(0);
-            if constexpr (sizeof(T) == 8) eta = eta2 = uniform01(etaw[j], T(0));
+            if constexpr (sizeof(T) == 8 && !PLAIN) eta = eta2 = uniform01(etaw[j], T(0));
             hit = (j == 0 ? eta : eta2) < texp(-dd0 * d1 / (M.nu * dt));   // Eqs. 53, 55
           }
           if (hit) {
@@ -865,6 +887,7 @@ void launch_advance(const AdvanceArgs<T>& a, int num_sms, int block, cudaStream_
     brute_search_kernel<T, true><<<bgrid, 256, 0, s>>>(a);
   } else {
     if (a.m.model == 1) simple_advance_kernel<T, false><<<grid, block, 0, s>>>(a);
+    else if (sizeof(T) == 8 && a.coupled) advance_kernel<T, false, sizeof(T) == 8><<<agrid, block, 0, s>>>(a);
     else advance_kernel<T, false><<<agrid, block, 0, s>>>(a);
     brute_search_kernel<T, false><<<bgrid, 256, 0, s>>>(a);
   }

@@ -121,9 +121,9 @@ __device__ __forceinline__ float uniform01(uint32_t w, float) {
 
 // Box & Muller (1958): two independent N(0, 1) from two uniform words.
 __device__ __forceinline__ void box_muller(uint32_t w1, uint32_t w2, double& g1, double& g2) {
-  const double r = m64::root(m64::minus_two_log(w1));
+  const double r = sqrt(-2.0 * log(uniform01(w1, 0.0)));
   double s, c;
-  m64::turn(w2, c, s);
+  sincospi(2.0 * uniform01(w2, 0.0), &s, &c);
   g1 = r * c;
   g2 = r * s;
 }

@@ -98,6 +98,7 @@ struct AdvanceArgs {
   const uint32_t* stepc;   // step counter (Philox counter word) in device memory
   const double* corr;      // [ne][2] Eq. 31 correction of the last coupled step still to be
                            // applied to the velocities as they are read (nullptr: none)
+  int coupled;             // a step of the coupled loop
   uint32_t k0, k1;
   // batches: per-instance parameters (m, k0, k1 above are unused) and element -> instance
   const InstDev<T>* inst;
