@@ -1,9 +1,9 @@
-// Per-element statistics and conditional means for elements of up to 768 particles, one
-// thread block per entry of the plan's tile lists (three size classes, launched as parallel
-// stream branches), and of 769..1024 from the plan's large-element list; larger elements go
-// through the block kernel in k_stats.cu.  The chunk-sort tile below serves every class of
-// Fox's projection; the bucket-rank tile further down every class of the hierarchical
-// bins.
+// Per-element statistics and conditional means for elements of up to 768 particles from the
+// plan's tile lists (three size classes, launched as parallel stream branches), and of
+// 769..1024 from the plan's large-element list; larger elements go through the block kernel
+// in k_stats.cu.  The chunk-sort tile below serves every class of Fox's projection; for the
+// hierarchical bins the class up to the split takes the warp tile at the end, the others the
+// bucket-rank tile (a block per element) or, for FP64 sums, the warp tile.
 //
 // Sect. 3.5 / Appendix A: the element's particles are sorted by (u, id); the level-1 groups
 // (positions with equal floor(g1 p / N)) are sorted by (v, id), the level-2 groups by
@@ -822,6 +822,69 @@ __device__ __forceinline__ int tile_element(const StatsArgs<T>& a, int b, int& m
   return CLS == 2 ? a.tiles_mid[b] : a.tiles[b];
 }
 
+// Effective bins (reading of Sect. 3.5): g_l = max(1, min(b_l, n / (g_1..g_{l-1} min_per_bin))).
+template <typename T>
+__device__ __forceinline__ void effective_bins(const StatsArgs<T>& a, int n, int (&g)[3]) {
+  int Gp = 1;
+#pragma unroll
+  for (int l = 0; l < 3; ++l) {
+    const int capl = n / (Gp * a.min_per_bin);
+    int gl = a.bins[l] < capl ? a.bins[l] : capl;
+    if (gl < 1) gl = 1;
+    g[l] = gl;
+    Gp *= gl;
+  }
+}
+
+// The 13 outputs of an element from its twelve sums and the shift values, in FP64, one per
+// lane of a warp, and its effective bins.
+template <typename T>
+__device__ __forceinline__ void write_moments(const StatsArgs<T>& a, const double* mh, const double* ml,
+                                              const double* msh, int e, int n, const int (&g)[3], int lane) {
+  if (lane < kNS) {
+    const double inv = recip_n(n);
+    const int ix = mom_nib(kMomX, lane), iy = mom_nib(kMomY, lane);
+    const int iz = mom_nib(kMomZ, lane), iw = mom_nib(kMomW, lane);
+    double v = ix < 15 ? msh[ix] : 0.0;
+    if (iy < 15) v += (mh[iy] + ml[iy]) * inv;
+    if (iz < 15) {
+      const double z = (mh[iz] + ml[iz]) * inv;
+      const double wv = (mh[iw] + ml[iw]) * inv;
+      v -= z * wv;
+    }
+    if (lane == 0) v = static_cast<double>(n);
+    else if (n == 0) v = 0.0;
+    a.emom[static_cast<size_t>(kNS) * e + lane] = v;
+  }
+  if (lane < 3) a.gbin[3 * e + lane] = g[lane];
+}
+
+// Appendix A bins: conditional scalar means over the final order's bins, by THREADS threads.
+template <int THREADS, typename T, typename I>
+__device__ __forceinline__ void write_bins(const StatsArgs<T>& a, const T* psi, const I* ord, int e, int n, int G,
+                                           int tid) {
+  double* vc = a.vcce + static_cast<size_t>(a.G) * e;
+  const float invGb = 1.0f / static_cast<float>(G);
+  for (int i = tid; i < a.G; i += THREADS) {
+    double mval = 0.0;
+    if (i < G && n > 0) {
+      const int b0 = group_start(i, n, G, invGb), b1 = group_start(i + 1, n, G, invGb);
+      if (sizeof(T) == 4 && a.acc64) {
+        double sum = 0.0;
+#pragma unroll 1
+        for (int p = b0; p < b1; ++p) sum += static_cast<double>(psi[ord[p]]);
+        mval = sum / static_cast<double>(b1 - b0);
+      } else {
+        Acc<T> sum;
+#pragma unroll 1
+        for (int p = b0; p < b1; ++p) sum.add(psi[ord[p]]);
+        mval = static_cast<double>(sum.value() / static_cast<T>(b1 - b0));
+      }
+    }
+    vc[i] = mval;
+  }
+}
+
 // ---------------------------------------------------------------------------------------
 // Hierarchical bins by per-level bucket ranks (the default conditioning, Sect. 3.5 and
 // Appendix A).  A level needs each particle's rank by (key, id) inside its group of the
@@ -1330,19 +1393,8 @@ __device__ void element_rank_tile(const StatsArgs<T>& a, RankTile<T, CAP, THREAD
       }
     }
   }
-  // effective bins (reading of Sect. 3.5): g_l = max(1, min(b_l, n / (g_1..g_{l-1} min_per_bin)))
   int g[3];
-  {
-    int Gp = 1;
-#pragma unroll
-    for (int l = 0; l < 3; ++l) {
-      const int capl = n / (Gp * a.min_per_bin);
-      int gl = a.bins[l] < capl ? a.bins[l] : capl;
-      if (gl < 1) gl = 1;
-      g[l] = gl;
-      Gp *= gl;
-    }
-  }
+  effective_bins(a, n, g);
   // the prior per level, by one thread in FP32 (FP64 arithmetic runs at a small fraction of
   // the FP32 rate on this GPU); any monotone bucket mapping gives the same ranks
   if (threadIdx.x == 0) {
@@ -1384,45 +1436,8 @@ __device__ void element_rank_tile(const StatsArgs<T>& a, RankTile<T, CAP, THREAD
   // moments in the final order, then the 13 outputs in FP64 (one per lane of warp 0)
   if (sizeof(T) == 4 && a.acc64) rank_moments<double>(t, n);
   else rank_moments<T>(t, n);
-  if (warp == 0) {
-    if (lane < kNS) {
-      const double inv = recip_n(n);
-      const int ix = mom_nib(kMomX, lane), iy = mom_nib(kMomY, lane);
-      const int iz = mom_nib(kMomZ, lane), iw = mom_nib(kMomW, lane);
-      double v = ix < 15 ? t.x_m.msh[ix] : 0.0;
-      if (iy < 15) v += (t.x_m.mh[iy] + t.x_m.ml[iy]) * inv;
-      if (iz < 15) {
-        const double z = (t.x_m.mh[iz] + t.x_m.ml[iz]) * inv;
-        const double wv = (t.x_m.mh[iw] + t.x_m.ml[iw]) * inv;
-        v -= z * wv;
-      }
-      if (lane == 0) v = static_cast<double>(n);
-      else if (n == 0) v = 0.0;
-      a.emom[static_cast<size_t>(kNS) * e + lane] = v;
-    }
-    if (lane < 3) a.gbin[3 * e + lane] = g[lane];
-  }
-  // Appendix A bins: conditional scalar means over the final order's bins
-  double* vc = a.vcce + static_cast<size_t>(a.G) * e;
-  const float invGb = 1.0f / static_cast<float>(G);
-  for (int i = threadIdx.x; i < a.G; i += THREADS) {
-    double mval = 0.0;
-    if (i < G && n > 0) {
-      const int b0 = group_start(i, n, G, invGb), b1 = group_start(i + 1, n, G, invGb);
-      if (sizeof(T) == 4 && a.acc64) {
-        double sum = 0.0;
-#pragma unroll 1
-        for (int p = b0; p < b1; ++p) sum += static_cast<double>(t.psi[t.ord[p]]);
-        mval = sum / static_cast<double>(b1 - b0);
-      } else {
-        Acc<T> sum;
-#pragma unroll 1
-        for (int p = b0; p < b1; ++p) sum.add(t.psi[t.ord[p]]);
-        mval = static_cast<double>(sum.value() / static_cast<T>(b1 - b0));
-      }
-    }
-    vc[i] = mval;
-  }
+  if (warp == 0) write_moments(a, t.x_m.mh, t.x_m.ml, t.x_m.msh, e, n, g, lane);
+  write_bins<THREADS>(a, t.psi, t.ord, e, n, G, threadIdx.x);
   // conditioning pointers (and the element-ordered copy of the state every few steps)
   const float inv_n = n > 0 ? 1.0f / static_cast<float>(n) : 0.0f;
   if (a.resort) {
@@ -1455,11 +1470,418 @@ __device__ void element_rank_tile(const StatsArgs<T>& a, RankTile<T, CAP, THREAD
   }
 }
 
-// Residency: the FP32 tiles fit 12 blocks of 128 threads up to 256 particles (11 KB each),
-// 10 up to 512 (22 KB) or 7 of 192 up to 768 (32 KB) per SM, the FP64 tiles fewer; the
-// register cap matches.
+// ---------------------------------------------------------------------------------------
+// A warp per element of up to 256 particles (the class up to the split; where the moment sums
+// are FP64 also of 257..512): no block barrier,
+// and every level an exact sort in registers.  Lane l holds the places l R .. l R + R - 1
+// (R = 4, 8 or 16).  A level's key is one 32-bit word: the value mapped linearly onto the upper
+// bits from the element's smallest to its largest (FP32 rounding, subtraction and scaling are
+// monotone, so the word never decreases with the value), and the particle's index.  Words are
+// distinct, so a bitonic network of minima and maxima sorts them and carries the index along.
+// Equal mapped values are put in the order of (value, particle id) afterwards by odd-even
+// exchanges, which a ballot skips where there are none.  The result is the order of a full
+// sort by (value, id) within the groups, as the other tiles find it; moment sums, bins and
+// pointers are taken from it in the same arithmetic and order.
+// Bound by instruction issue (75% active).  A block of 128 threads per element with bucket
+// levels, as the larger classes have, took 7,800 warp instructions for an element of 100
+// particles, most of them barriers', tables' and partly filled warps'; this takes about a
+// third.  The statistics stage of 200,000 such elements: 1,971 -> 691 us (with the classes
+// above launched over their lists), of 50,000 in FP64 1,183 -> 631 us.
+// ---------------------------------------------------------------------------------------
+template <int CAP> struct WarpIndex { using type = uint16_t; };
+template <> struct WarpIndex<256> { using type = uint8_t; };
+
+template <typename T, int CAP>
+struct WarpTile {
+  using Index = typename WarpIndex<CAP>::type;
+  double mh[12], ml[12], msh[5];    // moment sums (value/error pairs) and shift values
+  T u[CAP], v[CAP], w[CAP], om[CAP], psi[CAP];
+  uint32_t pid[CAP];
+  int32_t slot[CAP];
+  Index ord[CAP];                   // position -> particle in the final order
+};
+
+// Smallest and largest of the lanes' values.
+__device__ __forceinline__ float warp_min(float x) {
+  float r;
+  asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float warp_max(float x) {
+  float r;
+  asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
+  return r;
+}
+
+// Ascending bitonic sort of the words at places lane R + r within each segment of `seg`
+// places (a power of two from R to 32 R).  A phase whose direction depends on the lane
+// complements the words of its descending lanes, so that every stage ascends.
+template <int R>
+__device__ __forceinline__ void warp_sort_words(uint32_t (&k)[R], int seg, int lane) {
+  uint32_t flip = 0;
+#pragma unroll
+  for (int kk = 2; kk <= 32 * R; kk <<= 1) {
+    if (kk > R && kk > seg) break;
+    if (kk >= R) {
+      const uint32_t f = (kk < seg && (lane & (kk / R))) ? ~0u : 0u;
+#pragma unroll
+      for (int r = 0; r < R; ++r) k[r] ^= flip ^ f;
+      flip = f;
+    }
+#pragma unroll
+    for (int j = kk >> 1; j > 0; j >>= 1) {
+      if (j >= R) {
+        const bool low = (lane & (j / R)) == 0;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          const uint32_t o = __shfl_xor_sync(kFull, k[r], j / R);
+          k[r] = low ? min(k[r], o) : max(k[r], o);
+        }
+      } else {
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          if (r & j) continue;
+          const uint32_t x = k[r], y = k[r | j];
+          const bool up = kk >= R || (r & kk) == 0;
+          k[r] = up ? min(x, y) : max(x, y);
+          k[r | j] = up ? max(x, y) : min(x, y);
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < R; ++r) k[r] ^= flip;
+}
+
+// Runs of equal mapped value (equal words above the index) into the order of (value, id), by
+// odd-even exchanges of neighbouring places within segments of `seg` places.
+template <int R, int kIdx, typename T>
+__device__ __forceinline__ void warp_order_ties(uint32_t (&k)[R], const T* val, const uint32_t* pid, int seg, int lane) {
+  constexpr uint32_t kIdxMask = (1u << kIdx) - 1u;
+  auto swapped = [&](uint32_t a, uint32_t b) {   // b belongs before a
+    if ((a >> kIdx) != (b >> kIdx) || b == 0xffffffffu) return false;
+    const uint32_t i = a & kIdxMask, j = b & kIdxMask;
+    return rank_before(val[j], pid[j], val[i], pid[i]);
+  };
+  const bool first = (lane * R) % seg == 0, last = (lane * R + R) % seg == 0;   // at a segment's ends
+  for (int pass = 0; pass < 32 * R; ++pass) {
+    bool moved = false;
+    if (pass & 1) {
+      const uint32_t below = __shfl_up_sync(kFull, k[R - 1], 1), above = __shfl_down_sync(kFull, k[0], 1);
+      const bool up = !first && swapped(below, k[0]), dn = !last && swapped(k[R - 1], above);
+      if (up) k[0] = below;
+      if (dn) k[R - 1] = above;
+      moved = up | dn;
+    }
+#pragma unroll
+    for (int r = 0; r + 1 < R; ++r) {
+      if ((r & 1) != (pass & 1)) continue;
+      if (swapped(k[r], k[r + 1])) {
+        const uint32_t o = k[r];
+        k[r] = k[r + 1];
+        k[r + 1] = o;
+        moved = true;
+      }
+    }
+    // an odd pass without an exchange follows an even one that left its pairs in order
+    if (!__any_sync(kFull, moved) && (pass & 1)) break;
+  }
+}
+
+// The levels of one element of n <= 32 R particles (a whole warp): the final order in t.ord.
+//
+// A level's groups get segments of equal size, a power of two of at least R and the largest
+// group, while these fit the 32 R places: the sort then ends at the segment's size (4 x 4 x 4
+// bins of up to 128 particles: 28 stages for the first level, 15 and 6 for the others).
+// Otherwise the places are the positions and the group leads the word.
+template <int R, typename T, int CAP>
+__device__ __forceinline__ void warp_levels(WarpTile<T, CAP>& t, int n, const int (&g)[3], int lane) {
+  constexpr int kIdx = R == 4 ? 7 : R == 8 ? 8 : 9;   // bits of the particle's index
+  constexpr uint32_t kIdxMask = (1u << kIdx) - 1u;
+  static_assert(32 * R == (1 << kIdx), "index bits");
+  using Index = typename WarpTile<T, CAP>::Index;
+  const float inv_n = 1.0f / static_cast<float>(n);
+  int last = 0;
+  for (int l = 1; l < 3; ++l)
+    if (g[l] > 1) last = l;
+  int Gprev = 1;
+#pragma unroll 1
+  for (int l = 0; l <= last; ++l) {
+    if (l > 0 && g[l] <= 1) continue;
+    const T* val = l == 0 ? t.u : (l == 1 ? t.v : t.w);
+    const float invG = 1.0f / static_cast<float>(Gprev);
+    const int M = fdiv(n + Gprev - 1, invG);   // largest group
+    int seg = R;
+    while (seg < M) seg <<= 1;
+    const bool split = Gprev * seg <= 32 * R;
+    if (!split) seg = 32 * R;
+    const int lseg = 31 - __clz(seg);
+    const int gbits = split || Gprev == 1 ? 0 : 32 - __clz(Gprev - 1);
+    // places -> particles, from the order of the level before
+    uint32_t k[R];
+    if (l == 0) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int i = lane * R + r;   // the whole element lies in the first segment
+        k[r] = i < n ? static_cast<uint32_t>(i) : 0xffffffffu;
+      }
+    } else {
+      // the segment of this lane's first place (R places never straddle one)
+      const int s = split ? (lane * R) >> lseg : 0;
+      const int gs = split && s < Gprev ? group_start(s, n, Gprev, invG) : 0;
+      const int ge = split ? (s < Gprev ? group_start(s + 1, n, Gprev, invG) : 0) : n;
+      const int p0 = gs + lane * R - (s << lseg);
+#pragma unroll
+      for (int r = 0; r < R; ++r) k[r] = p0 + r < ge ? static_cast<uint32_t>(t.ord[p0 + r]) : 0xffffffffu;
+      __syncwarp();
+    }
+    float x[R];
+    float lo = INFINITY, hi = -INFINITY;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      x[r] = 0.0f;
+      if (k[r] != 0xffffffffu) {
+        x[r] = bucket_key(val[k[r]]);
+        lo = fminf(lo, x[r]);
+        hi = fmaxf(hi, x[r]);
+      }
+    }
+    lo = warp_min(lo);
+    const float span = warp_max(hi) - lo;
+    const int qbits = 32 - kIdx - gbits;
+    const float top = static_cast<float>(1u << qbits);
+    const float scale = span > 0.0f ? __fdividef(top, span) : 0.0f;
+    const uint32_t qmax = (1u << qbits) - 2u;   // a word of ones is padding
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      // NaN (a non-finite state) maps to zero, infinities to the ends
+      const uint32_t q = min(__float2uint_rz((x[r] - lo) * scale), qmax);
+      uint32_t word = (q << kIdx) | k[r];
+      if (gbits) word |= static_cast<uint32_t>(fdiv(Gprev * (lane * R + r), inv_n)) << (32 - gbits);
+      k[r] = k[r] == 0xffffffffu ? k[r] : word;
+    }
+    warp_sort_words<R>(k, seg, lane);
+    // equal mapped values next to one another (R places never straddle a segment)
+    const uint32_t above = __shfl_down_sync(kFull, k[0], 1);
+    bool tie = (lane * R + R) % seg != 0 && (k[R - 1] >> kIdx) == (above >> kIdx) && above != 0xffffffffu;
+#pragma unroll
+    for (int r = 0; r + 1 < R; ++r) tie |= (k[r] >> kIdx) == (k[r + 1] >> kIdx) && k[r + 1] != 0xffffffffu;
+    if (__any_sync(kFull, tie)) warp_order_ties<R, kIdx>(k, val, t.pid, seg, lane);
+    // the order so far, by position
+    {
+      const int s = split ? (lane * R) >> lseg : 0;
+      const int gs = split && s < Gprev ? group_start(s, n, Gprev, invG) : 0;
+      const int p0 = gs + lane * R - (s << lseg);
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+        if (k[r] != 0xffffffffu) t.ord[p0 + r] = static_cast<Index>(k[r] & kIdxMask);
+    }
+    __syncwarp();
+    Gprev *= g[l];
+  }
+}
+
+// One level of the moment sums' tree over the lanes, N sums in and N / 2 (rounded up) out: a
+// lane sends its partner (lane ^ o) the half it gives up and joins the other half's value of
+// both, the lower lane's first, as Acc::warp_pair does for one sum in every lane.
+template <int N, typename A>
+__device__ __forceinline__ void pair_level(A (&h)[12], A (&l)[12], int o, int lane) {
+  constexpr int H = (N + 1) / 2;
+  const bool low = (lane & o) == 0;
+#pragma unroll
+  for (int s = 0; s < H; ++s) {
+    const int t = N > 1 ? (s + H < N ? s + H : N - 1) : 0;   // the upper half's sum at this place
+    const A mh = low ? h[s] : h[t], ml = low ? l[s] : l[t];
+    const A gh = low ? h[t] : h[s], gl = low ? l[t] : l[s];
+    const A oh = __shfl_xor_sync(kFull, gh, o);
+    const A ah = low ? mh : oh, bh = low ? oh : mh;
+    if (sizeof(A) == 4) {
+      const A ol = __shfl_xor_sync(kFull, gl, o);
+      const A al = low ? ml : ol, bl = low ? ol : ml;
+      const A sh = ah + bh;
+      const A bb = sh - ah;
+      const A se = (ah - (sh - bb)) + (bh - bb);
+      const A lw = se + (al + bl);
+      h[s] = sh + lw;
+      l[s] = lw - (h[s] - sh);
+    } else {
+      h[s] = ah + bh;
+    }
+  }
+}
+
+// The twelve moment sums of rank_moments by one warp: lane l takes positions l, l + 32, ...
+template <typename A, typename T, int CAP>
+__device__ __forceinline__ void warp_moments(WarpTile<T, CAP>& t, int n, int lane) {
+  A sa[5] = {A(0), A(0), A(0), A(0), A(0)};
+  const T* const val[5] = {t.u, t.v, t.w, t.om, t.psi};
+  if (n > 0) {
+    const int q0 = t.ord[0];
+#pragma unroll
+    for (int c = 0; c < 5; ++c) sa[c] = A(val[c][q0]);
+  }
+  Acc<A> m[12];
+#pragma unroll 1
+  for (int p = lane; p < n; p += 32) {
+    const int q = t.ord[p];
+    A d[5];
+#pragma unroll
+    for (int c = 0; c < 5; ++c) {
+      d[c] = A(val[c][q]) - sa[c];
+      m[c].add(d[c]);
+    }
+    m[5].add(xmul(d[0], d[0])); m[6].add(xmul(d[1], d[1])); m[7].add(xmul(d[2], d[2]));
+    m[8].add(xmul(d[0], d[1])); m[9].add(xmul(d[0], d[2])); m[10].add(xmul(d[1], d[2]));
+    m[11].add(xmul(d[4], d[4]));
+  }
+  A h[12], l[12];
+#pragma unroll
+  for (int c = 0; c < 12; ++c) {
+    h[c] = m[c].s;
+    l[c] = -Acc<A>::err(m[c]);
+  }
+  pair_level<12>(h, l, 16, lane);
+  pair_level<6>(h, l, 8, lane);
+  pair_level<3>(h, l, 4, lane);
+  pair_level<2>(h, l, 2, lane);
+  pair_level<1>(h, l, 1, lane);
+  // the lane's sum: bit 4 of the lane chose six, bit 3 three of them, bits 2 and 1 one
+  const int c = (lane & 16 ? 6 : 0) + (lane & 8 ? 3 : 0) + (lane & 4 ? 2 : 0) + (lane & 2 ? 1 : 0);
+  if (!(lane & 1) && (lane & 6) != 6) {
+    t.mh[c] = h[0];
+    t.ml[c] = sizeof(A) == 4 ? l[0] : A(0);
+  }
+  if (lane < 5) t.msh[lane] = lane == 0 ? sa[0] : lane == 1 ? sa[1] : lane == 2 ? sa[2] : lane == 3 ? sa[3] : sa[4];
+  __syncwarp();
+}
+
+// One element of N <= CAP particles by a warp (hierarchical bins).
+template <typename T, int CAP>
+__device__ void element_warp_tile(const StatsArgs<T>& a, WarpTile<T, CAP>& t, int e, int N, int moves) {
+  const int lane = threadIdx.x & 31;
+  const unsigned below = (1u << lane) - 1u;
+  // gather: the element's list minus particles moved out, plus those moved in
+  const int32_t o = a.off[e], c = a.cnt[e];
+  int n = 0;
+  if (!moves) {
+    n = c;
+  } else {
+    const int32_t gn = a.gain[e], g0 = a.goff[e];
+    for (int j0 = 0; j0 < c + gn; j0 += 32) {   // lanes of one round may hold both kinds
+      const int j = j0 + lane;
+      int32_t q = -1;
+      if (j < c) {
+        q = a.idx[o + j];
+        if (a.p.elem[q] != e) q = -1;
+      } else if (j < c + gn) {
+        q = a.movers[g0 + j - c];
+        if (q >= a.np) q = -1;
+      }
+      const unsigned keep = __ballot_sync(kFull, q >= 0);
+      const int at = n + __popc(keep & below);
+      if (q >= 0 && at < CAP) t.slot[at] = q;
+      n += __popc(keep);
+    }
+  }
+  if (n != N && lane == 0) atomicCAS(a.err, 0, PDFX_ERR_CAPACITY);
+  n = min(min(n, N), CAP);
+  __syncwarp();
+  // stage the values and ids, four particles' loads in flight together
+#pragma unroll 1
+  for (int j0 = lane; j0 - lane < n; j0 += 128) {
+    int32_t q[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int j = j0 + 32 * k;
+      q[k] = j < n ? (moves ? t.slot[j] : __ldg(a.idx + o + j)) : -1;
+    }
+    T vu[4], vv[4], vw[4], vo[4], vp[4];
+    uint32_t vi[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (q[k] >= 0) {
+        vu[k] = __ldg(a.p.u + q[k]);
+        vv[k] = __ldg(a.p.v + q[k]);
+        vw[k] = __ldg(a.p.w + q[k]);
+        vo[k] = __ldg(a.p.om + q[k]);
+        vp[k] = __ldg(a.p.psi + q[k]);
+        vi[k] = __ldg(a.p.pid + q[k]);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int j = j0 + 32 * k;
+      if (q[k] >= 0) {
+        t.slot[j] = q[k];
+        t.u[j] = vu[k];
+        t.v[j] = vv[k];
+        t.w[j] = vw[k];
+        t.om[j] = vo[k];
+        t.psi[j] = vp[k];
+        t.pid[j] = vi[k];
+      }
+    }
+  }
+  __syncwarp();
+  int g[3];
+  effective_bins(a, n, g);
+  if (CAP > 256 && n > 256) warp_levels<CAP >= 512 ? 16 : 8>(t, n, g, lane);
+  else if (n > 128) warp_levels<8>(t, n, g, lane);
+  else if (n > 0) warp_levels<4>(t, n, g, lane);
+  __syncwarp();
+  if (sizeof(T) == 4 && a.acc64) warp_moments<double>(t, n, lane);
+  else warp_moments<T>(t, n, lane);
+  write_moments(a, t.mh, t.ml, t.msh, e, n, g, lane);
+  const int G = g[0] * g[1] * g[2];
+  write_bins<32>(a, t.psi, t.ord, e, n, G, lane);
+  // conditioning pointers (and the element-ordered copy of the state every few steps)
+  const float inv_n = n > 0 ? 1.0f / static_cast<float>(n) : 0.0f;
+  if (a.resort) {
+    const int32_t fo = a.foff[e];
+    for (int p = lane; p < n; p += 32) {
+      const int32_t d = fo + p;
+      if (d >= a.np) break;
+      const int j = t.ord[p];
+      store_pos(a.out, d, load_pos(a.p, t.slot[j]));
+      a.out.u[d] = t.u[j];
+      a.out.v[d] = t.v[j];
+      a.out.w[d] = t.w[j];
+      a.out.om[d] = t.om[j];
+      a.out.psi[d] = t.psi[j];
+      a.out.pid[d] = t.pid[j];
+      a.out.elem[d] = e;
+      a.out.cp[d] = static_cast<uint8_t>(fdiv(G * p, inv_n));
+    }
+  } else {
+    for (int p = lane; p < n; p += 32) a.p.cp[t.slot[t.ord[p]]] = static_cast<uint8_t>(fdiv(G * p, inv_n));
+  }
+}
+
+template <typename T, int CAP, int WARPS, int CLS>
+__global__ void __launch_bounds__(32 * WARPS) warp_tile_kernel(const StatsArgs<T> a) {
+  extern __shared__ __align__(16) unsigned char warp_smem[];
+  const int warp = threadIdx.x >> 5;
+  const int b = static_cast<int>(blockIdx.x) * WARPS + warp;
+  if (b >= a.ne) return;
+  int moves = 0;
+  const int e = tile_element<CLS>(a, b, moves);
+  if (e < 0) return;
+  const int N = moves ? a.fin[e] : a.cnt[e];
+  element_warp_tile<T, CAP>(a, reinterpret_cast<WarpTile<T, CAP>*>(warp_smem)[warp], e, min(N, CAP), moves);
+}
+template <typename T, int CAP, int WARPS>
+constexpr int warp_tile_smem() { return static_cast<int>(sizeof(WarpTile<T, CAP>)) * WARPS; }
+template <typename T, int CAP, int WARPS, int CLS>
+void launch_warp_tile(const StatsArgs<T>& a, cudaStream_t s) {
+  warp_tile_kernel<T, CAP, WARPS, CLS>
+      <<<static_cast<unsigned>((a.ne + WARPS - 1) / WARPS), 32 * WARPS, warp_tile_smem<T, CAP, WARPS>(), s>>>(a);
+}
+
+// Residency: the FP32 bucket-rank tiles fit 10 blocks of 128 threads up to 512 particles
+// (22 KB) or 7 of 192 up to 768 (32 KB) per SM, the FP64 tiles fewer; the register cap
+// matches.
 template <typename T, int CAP, int THREADS, int CLS>
-__global__ void __launch_bounds__(THREADS, (sizeof(T) == 4 ? (CAP == 256 ? 1536 : THREADS == 192 ? 1344 : 1280) : 1024) / THREADS)
+__global__ void __launch_bounds__(THREADS, (sizeof(T) == 4 ? (THREADS == 192 ? 1344 : 1280) : 1024) / THREADS)
     rank_tile_kernel(const StatsArgs<T> a) {
   extern __shared__ __align__(16) unsigned char rank_smem[];
   RankTile<T, CAP, THREADS>& t = *reinterpret_cast<RankTile<T, CAP, THREADS>*>(rank_smem);
@@ -1468,6 +1890,35 @@ __global__ void __launch_bounds__(THREADS, (sizeof(T) == 4 ? (CAP == 256 ? 1536 
   if (e < 0) return;
   const int N = moves ? a.fin[e] : a.cnt[e];
   element_rank_tile<T, CAP, THREADS>(a, t, e, min(N, CAP), moves);
+}
+// The same over the class's entries, gridDim.x apart, for a class that few elements should
+// belong to: a block per element of the grid then mostly launches blocks that return (100 us
+// for 200,000 elements).  Entries in turn cost a block more than entries of its own (11% to
+// 24% measured on a full class).
+template <typename T, int CAP, int THREADS, int CLS>
+__global__ void __launch_bounds__(THREADS, (sizeof(T) == 4 ? 1024 : 768) / THREADS)
+    rank_list_kernel(const StatsArgs<T> a) {
+  static_assert(CLS != 0, "the class of the step counter takes a block per entry");
+  extern __shared__ __align__(16) unsigned char rank_smem[];
+  RankTile<T, CAP, THREADS>& t = *reinterpret_cast<RankTile<T, CAP, THREADS>*>(rank_smem);
+  for (int inst = 0; inst < a.K; ++inst) {
+    const int32_t* sc = a.scal + 16 * inst;
+    const int eb = a.ielem ? a.ielem[inst] : 0, ee = a.ielem ? a.ielem[inst + 1] : a.ne;
+    const int moves = sc[0] > 0, count = CLS == 1 ? sc[7] : sc[8];
+    for (int b = blockIdx.x; b < count; b += gridDim.x) {
+      const int e = CLS == 1 ? a.tiles[ee - 1 - b] : a.tiles_mid[eb + b];
+      const int N = moves ? a.fin[e] : a.cnt[e];
+      element_rank_tile<T, CAP, THREADS>(a, t, e, min(N, CAP), moves);
+      __syncthreads();   // done with the shared memory
+    }
+  }
+}
+// few: 0, or the blocks of the list kernel.
+template <typename T, int CAP, int THREADS, int CLS>
+void launch_rank_tile(const StatsArgs<T>& a, int few, cudaStream_t s) {
+  constexpr int smem = static_cast<int>(sizeof(RankTile<T, CAP, THREADS>));
+  if (few > 0 && few < a.ne) rank_list_kernel<T, CAP, THREADS, CLS><<<static_cast<unsigned>(few), THREADS, smem, s>>>(a);
+  else rank_tile_kernel<T, CAP, THREADS, CLS><<<static_cast<unsigned>(a.ne), THREADS, smem, s>>>(a);
 }
 
 // The plan's large-element lists (every instance's), entries of up to kTileBig particles, on
@@ -1518,33 +1969,44 @@ void launch_stats_tiles_impl(const StatsArgs<T>& a, int num_sms, cudaStream_t s_
   if (a.ne <= 0) return;
   static_assert(kSmallCap == 768 && kTileMid == 512 && kTileSplit == 256,
                 "tile classes cover the small-element capacity");
-  // hierarchical bins: bucket ranks in every class, up to the split (at most 256
-  // particles) on a tile of 256 (4 warps), then up to 512 (4 warps) and 513..768 (6
-  // warps).  Fox's projection: chunk sorts in every class (groups of at most 32 positions
-  // are sorted by one warp in registers; the largest class in a tile of 1,024).
+  // hierarchical bins: a warp per element up to the split (at most 256 particles), then bucket
+  // ranks up to 512 (4 warps) and 513..768 (6 warps).  Fox's projection: chunk sorts in every
+  // class (groups of at most 32 positions are sorted by one warp in registers; the largest
+  // class in a tile of 1,024).
   const unsigned grid = static_cast<unsigned>(a.ne);
   if (a.cond_mode == 1) {
     stats_tile_kernel<T, 1024, 256, 1, true><<<grid, 256, 0, s_large>>>(a);
     stats_tile_kernel<T, 256, 128, 0, true><<<grid, 128, 0, s_small>>>(a);
     stats_tile_kernel<T, 512, 128, 2, true><<<grid, 128, 0, s_mid>>>(a);
   } else {
-    constexpr size_t small = sizeof(RankTile<T, 256, 128>), mid = sizeof(RankTile<T, 512, 128>);
-    constexpr size_t large = sizeof(RankTile<T, 768, 192>), big = sizeof(RankTile<T, kTileBig, 256>);
+    constexpr size_t big = sizeof(RankTile<T, kTileBig, 256>);
     static_assert(big <= 227 * 1024, "rank tile exceeds shared memory");
     if (first_use_on_device(rank_configured<T>)) {
-      cudaFuncSetAttribute(rank_tile_kernel<T, 256, 128, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(small));
-      cudaFuncSetAttribute(rank_tile_kernel<T, 512, 128, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(mid));
-      cudaFuncSetAttribute(rank_tile_kernel<T, 768, 192, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(large));
-      cudaFuncSetAttribute(rank_big_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(big));
+      auto allow = [](const void* f, size_t bytes) {
+        cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
+      };
+      allow(reinterpret_cast<const void*>(rank_big_kernel<T>), big);
+      allow(reinterpret_cast<const void*>(rank_tile_kernel<T, 768, 192, 1>), sizeof(RankTile<T, 768, 192>));
+      allow(reinterpret_cast<const void*>(rank_list_kernel<T, 768, 192, 1>), sizeof(RankTile<T, 768, 192>));
+      allow(reinterpret_cast<const void*>(rank_tile_kernel<T, 512, 128, 2>), sizeof(RankTile<T, 512, 128>));
+      allow(reinterpret_cast<const void*>(rank_list_kernel<T, 512, 128, 2>), sizeof(RankTile<T, 512, 128>));
+      allow(reinterpret_cast<const void*>(warp_tile_kernel<T, 256, 4, 0>), warp_tile_smem<T, 256, 4>());
+      allow(reinterpret_cast<const void*>(warp_tile_kernel<T, 512, 2, 2>), warp_tile_smem<T, 512, 2>());
     }
-    rank_tile_kernel<T, 768, 192, 1><<<grid, 192, large, s_large>>>(a);
+    // the classes above the mean count by a factor of two and more hold few elements
+    const int64_t mean = a.np / a.ne;
+    const int few = 8 * (num_sms > 0 ? num_sms : 1);
+    launch_rank_tile<T, 768, 192, 1>(a, mean <= 256 ? few : 0, s_large);
     // 769..1024 from the large-element list: 4 blocks per SM
     rank_big_kernel<T><<<static_cast<unsigned>(4 * (num_sms > 0 ? num_sms : 1)), 256, big, s_large>>>(a);
-    rank_tile_kernel<T, 256, 128, 0><<<grid, 128, small, s_small>>>(a);
-    rank_tile_kernel<T, 512, 128, 2><<<grid, 128, mid, s_mid>>>(a);
+    launch_warp_tile<T, 256, 4, 0>(a, s_small);
+    // 257..512: a block per element with bucket levels in the FP32 form; where the moment sums
+    // are FP64 a warp per element, whose register sort leaves the FP64 pipe the shorter wait
+    // (8,100 elements of 300 and 500 particles: FP64 form 350 and 530 us -> 292 and 408, FP64
+    // accumulation 326 and 464 -> 244 and 363; FP32 form 216 -> 359 us for 12,100 of 350, its
+    // 15 resident warps too few)
+    if (mean > 128 && (sizeof(T) == 8 || a.acc64)) launch_warp_tile<T, 512, 2, 2>(a, s_mid);
+    else launch_rank_tile<T, 512, 128, 2>(a, mean <= 128 ? few : 0, s_mid);
   }
 }
 
