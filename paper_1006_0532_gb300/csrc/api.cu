@@ -493,11 +493,11 @@ int do_get_particles(Ctx& c, pdfx_soa* soa, int on_device, cudaStream_t s) {
   apply_pending_correction<T>(c, s);
   Particles<T> p = carve<T>(c.pbuf[c.cur], c.np);
   const size_t n = static_cast<size_t>(c.np);
+  int32_t* const scratch = c.plan.idx;   // the element lists of the last pass, no longer needed
   if (on_device) {
-    launch_gather_by_pid<T>(p, c.np, c.K > 1 ? c.einst : nullptr, c.K > 1 ? c.ip0 : nullptr,
-                            soa->x, soa->y, soa->u, soa->v, soa->w, soa->om, soa->psi, soa->elem,
-                            soa->cp, s);
-    c.launches++;
+    c.launches += launch_gather_by_pid<T>(p, c.np, c.K > 1 ? c.einst : nullptr, c.K > 1 ? c.ip0 : nullptr, scratch,
+                                          soa->x, soa->y, soa->u, soa->v, soa->w, soa->om, soa->psi, soa->elem,
+                                          soa->cp, s);
     return cerr(cudaGetLastError());
   }
   if (n == 0) return PDFX_OK;
@@ -505,10 +505,9 @@ int do_get_particles(Ctx& c, pdfx_soa* soa, int on_device, cudaStream_t s) {
   if (!tmp) return PDFX_ERR_ALLOC;
   int32_t* tel = reinterpret_cast<int32_t*>(tmp + 7 * n);
   uint8_t* tcp = reinterpret_cast<uint8_t*>(tel + n);
-  launch_gather_by_pid<T>(p, c.np, c.K > 1 ? c.einst : nullptr, c.K > 1 ? c.ip0 : nullptr, tmp,
-                          tmp + n, tmp + 2 * n, tmp + 3 * n, tmp + 4 * n, tmp + 5 * n, tmp + 6 * n,
-                          tel, tcp, s);
-  c.launches++;
+  c.launches += launch_gather_by_pid<T>(p, c.np, c.K > 1 ? c.einst : nullptr, c.K > 1 ? c.ip0 : nullptr, scratch, tmp,
+                                        tmp + n, tmp + 2 * n, tmp + 3 * n, tmp + 4 * n, tmp + 5 * n, tmp + 6 * n,
+                                        tel, tcp, s);
   double* dst[7] = {soa->x, soa->y, soa->u, soa->v, soa->w, soa->om, soa->psi};
   int rc = PDFX_OK;
   for (int k = 0; k < 7 && rc == PDFX_OK; ++k)

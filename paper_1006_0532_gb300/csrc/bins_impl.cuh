@@ -1993,9 +1993,10 @@ void launch_stats_tiles_impl(const StatsArgs<T>& a, int num_sms, cudaStream_t s_
       allow(reinterpret_cast<const void*>(warp_tile_kernel<T, 256, 4, 0>), warp_tile_smem<T, 256, 4>());
       allow(reinterpret_cast<const void*>(warp_tile_kernel<T, 512, 2, 2>), warp_tile_smem<T, 512, 2>());
     }
-    // the classes above the mean count by a factor of two and more hold few elements
+    // the classes above the mean count by a factor of two and more hold few elements: over
+    // their lists where blocks that return would take 10 us and more (0.5 ns each)
     const int64_t mean = a.np / a.ne;
-    const int few = 8 * (num_sms > 0 ? num_sms : 1);
+    const int few = a.ne >= 20000 ? 8 * (num_sms > 0 ? num_sms : 1) : 0;
     launch_rank_tile<T, 768, 192, 1>(a, mean <= 256 ? few : 0, s_large);
     // 769..1024 from the large-element list: 4 blocks per SM
     rank_big_kernel<T><<<static_cast<unsigned>(4 * (num_sms > 0 ? num_sms : 1)), 256, big, s_large>>>(a);

@@ -831,6 +831,36 @@ __global__ void gather_by_pid_kernel(Particles<T> p, int64_t np, const int32_t* 
   if (cp) cp[id] = p.cp[i];
 }
 
+// The same in two passes for many particles: each slot leaves its number at its caller's
+// index, then each index fetches its particle, so that the 61 B of output per particle are
+// written in order.  The particles of an index range lie in a few elements' slots (ids are
+// given element by element and particles stay near), so the scattered reads, 4 B each, meet
+// lines the block holds; scattered 8 B writes (the single pass) do not coalesce.
+__global__ void slot_of_index_kernel(const uint32_t* __restrict__ pid, const int32_t* __restrict__ elem, int64_t np,
+                                     const int32_t* einst, const int64_t* ip0, int32_t* __restrict__ slot) {
+  const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (i < np) slot[(einst ? ip0[einst[elem[i]]] : 0) + pid[i]] = static_cast<int32_t>(i);
+}
+template <typename T>
+__global__ void gather_slots_kernel(Particles<T> p, int64_t np, const int32_t* __restrict__ slot, double* x, double* y,
+                                    double* u, double* v, double* w, double* om, double* psi, int32_t* elem,
+                                    uint8_t* cp) {
+  const int64_t id = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (id >= np) return;
+  const int32_t i = slot[id];
+  if (i < 0 || i >= np) return;
+  const Pos<T> P = load_pos(p, i);
+  if (x) __stcs(x + id, pos_x(P));
+  if (y) __stcs(y + id, pos_y(P));
+  if (u) __stcs(u + id, static_cast<double>(p.u[i]));
+  if (v) __stcs(v + id, static_cast<double>(p.v[i]));
+  if (w) __stcs(w + id, static_cast<double>(p.w[i]));
+  if (om) __stcs(om + id, static_cast<double>(p.om[i]));
+  if (psi) __stcs(psi + id, static_cast<double>(p.psi[i]));
+  if (elem) __stcs(elem + id, p.elem[i]);
+  if (cp) cp[id] = p.cp[i];
+}
+
 template <typename T>
 __global__ void load_state_kernel(Particles<T> p, int64_t np, const int32_t* einst,
                                   const int64_t* ip0, const double* x, const double* y,
@@ -917,12 +947,20 @@ void launch_count(const int32_t* elem, int64_t np, int32_t ne, int32_t* cnt, uns
 }
 
 template <typename T>
-void launch_gather_by_pid(Particles<T> p, int64_t np, const int32_t* einst, const int64_t* ip0,
-                          double* x, double* y, double* u, double* v, double* w, double* om,
-                          double* psi, int32_t* elem, uint8_t* cp, cudaStream_t s) {
-  if (np <= 0) return;
+int launch_gather_by_pid(Particles<T> p, int64_t np, const int32_t* einst, const int64_t* ip0, int32_t* slot,
+                         double* x, double* y, double* u, double* v, double* w, double* om,
+                         double* psi, int32_t* elem, uint8_t* cp, cudaStream_t s) {
+  if (np <= 0) return 0;
+  // two passes from a million particles on, where the writes leave the L2 (25M in the FP32 form:
+  // 994 -> 694 us, 20M in small elements 573 -> 533); below, one launch less
+  if (np >= (int64_t(1) << 20)) {
+    slot_of_index_kernel<<<blocks_for(np, 256), 256, 0, s>>>(p.pid, p.elem, np, einst, ip0, slot);
+    gather_slots_kernel<T><<<blocks_for(np, 256), 256, 0, s>>>(p, np, slot, x, y, u, v, w, om, psi, elem, cp);
+    return 2;
+  }
   gather_by_pid_kernel<T><<<blocks_for(np, 256), 256, 0, s>>>(p, np, einst, ip0, x, y, u, v, w, om,
                                                               psi, elem, cp);
+  return 1;
 }
 
 template <typename T>
@@ -948,9 +986,9 @@ void launch_convert_fields(const double* in, float* out, int64_t n, cudaStream_t
   template void launch_init_batch<T>(Particles<T>, int64_t, int, const InstDev<T>*,            \
                                      const int64_t*, const ElemGeo<T>*, const ElemTopo*,       \
                                      const T*, unsigned long long*, cudaStream_t);             \
-  template void launch_gather_by_pid<T>(Particles<T>, int64_t, const int32_t*, const int64_t*, \
-                                        double*, double*, double*, double*, double*, double*,  \
-                                        double*, int32_t*, uint8_t*, cudaStream_t);            \
+  template int launch_gather_by_pid<T>(Particles<T>, int64_t, const int32_t*, const int64_t*,  \
+                                       int32_t*, double*, double*, double*, double*, double*,  \
+                                       double*, double*, int32_t*, uint8_t*, cudaStream_t);    \
   template void launch_load_state<T>(Particles<T>, int64_t, const int32_t*, const int64_t*,    \
                                      const double*, const double*, const double*,              \
                                      const double*, const double*, const double*,              \

@@ -470,11 +470,11 @@ void launch_scalar_stats(const Particles<T>& p, int64_t np, const int32_t* probe
                          int G, int n, int nb, const ScalarAcc& acc, const ScalarOut& out,
                          int num_sms, cudaStream_t s);   // k_scalar.cu
 // Particle order of the caller's arrays: by (instance, id), i.e. index p0_k + id (einst and
-// ip0 nullptr: one instance, index = id).
+// ip0 nullptr: one instance, index = id).  slot: scratch [np].  Returns the kernels launched.
 template <typename T>
-void launch_gather_by_pid(Particles<T> p, int64_t np, const int32_t* einst, const int64_t* ip0,
-                          double* x, double* y, double* u, double* v, double* w, double* om,
-                          double* psi, int32_t* elem, uint8_t* cp, cudaStream_t s);
+int launch_gather_by_pid(Particles<T> p, int64_t np, const int32_t* einst, const int64_t* ip0, int32_t* slot,
+                         double* x, double* y, double* u, double* v, double* w, double* om,
+                         double* psi, int32_t* elem, uint8_t* cp, cudaStream_t s);
 template <typename T>
 void launch_load_state(Particles<T> p, int64_t np, const int32_t* einst, const int64_t* ip0,
                        const double* x, const double* y, const double* u, const double* v,
