@@ -266,18 +266,29 @@ int ensure_particles(Ctx& c, int64_t np) {
   return PDFX_OK;
 }
 
+// Counts per element at zero before an advance or a count: the statistics pass before left
+// them so (its node average clears them), unless there was none or it was cut short.
+int clear_counts(Ctx& c, cudaStream_t s) {
+  const bool clear = c.counts_clear;
+  c.counts_clear = false;
+  if (clear) return PDFX_OK;
+  PDFX_CUDA(cudaMemsetAsync(c.err + 1, 0, sizeof(int), s));   // the brute-force list's length
+  return cerr(cudaMemsetAsync(c.plan.cnt, 0, sizeof(int32_t) * c.ne, s));
+}
+
 // Statistics and conditional means of the current state (after advance or a new state).
 template <typename T>
 int run_statistics(Ctx& c, bool counts_ready, bool allow_moves, bool force_resort, cudaStream_t s) {
   Particles<T> p = carve<T>(c.pbuf[c.cur], c.np);
   if (!counts_ready) {
-    PDFX_CUDA(cudaMemsetAsync(c.plan.cnt, 0, sizeof(int32_t) * c.ne, s));
+    PDFX_TRY(clear_counts(c, s));
     launch_count(p.elem, c.np, c.ne, c.plan.cnt, c.diag, c.err, s);
     c.launches++;
   }
   {
     StageTimer t(c, 1, s);
     c.plan.tile_split = c.tile_split;
+    c.plan.brute_count = c.err + 1;
     c.launches += launch_plan(c.plan, c.ne, c.K, c.prm.minnpel, allow_moves ? 1 : 0, s);
   }
   {
@@ -331,10 +342,7 @@ int run_statistics(Ctx& c, bool counts_ready, bool allow_moves, bool force_resor
     a.fox_bins = c.prm.fox_bins;
     a.diag = c.diag;
     a.err = c.err;
-    launch_stats<T>(a, c.num_sms, s, &c.side);
-    // three tile classes, the large-element kernel and (hierarchical bins) the bucket-rank
-    // tile over the large-element list
-    c.launches += a.cond_mode == 1 ? 4 : 5;
+    c.launches += launch_stats<T>(a, c.num_sms, s, &c.side);
   }
   if (resort) {
     c.cur = 1 - c.cur;
@@ -344,17 +352,19 @@ int run_statistics(Ctx& c, bool counts_ready, bool allow_moves, bool force_resor
   }
   {
     StageTimer t(c, 5, s);
-    launch_node_average(c.emom, c.ne_off, c.ne_list, c.nn, c.nmom, s);
+    launch_node_average(c.emom, c.ne_off, c.ne_list, c.nn, c.nmom, c.plan.cnt, c.ne, s);
     c.launches++;
   }
-  return cerr(cudaGetLastError());
+  const int rc = cerr(cudaGetLastError());
+  c.counts_clear = rc == PDFX_OK;
+  return rc;
 }
 
 template <typename T>
 int do_step(Ctx& c, double dt, cudaStream_t s, bool coupled = false) {
   c.last_dt = dt;
   Particles<T> p = carve<T>(c.pbuf[c.cur], c.np);
-  PDFX_CUDA(cudaMemsetAsync(c.plan.cnt, 0, sizeof(int32_t) * c.ne, s));
+  PDFX_TRY(clear_counts(c, s));
   {
     StageTimer t(c, 0, s);
     AdvanceArgs<T> a{};
@@ -829,6 +839,7 @@ int set_grid(Ctx& c, int32_t nn, const double* xy, int32_t ne, const int32_t* tr
   c.h_area2 = g.area2;
   c.fem_ready = false;   // the Eulerian calls rebuild their FEM data for this grid
   c.corr_pending = false;
+  c.counts_clear = false;
   c.have_grid = true;
   c.have_fields = false;
   return PDFX_OK;
@@ -1253,7 +1264,7 @@ int do_coupled_step(Ctx& c, double dt, double Cp, double tol, int32_t max_iter, 
   // particles take it as the next advance reads them (or before any other reader).
   launch_correction_field<T>(geo, c.topo, c.ne, c.prm.period_x, nullptr, nullptr, c.dP, dt, c.corr, s);
   launch_shift_means(c.ne, c.corr, c.emom, s);
-  launch_node_average(c.emom, c.ne_off, c.ne_list, c.nn, c.nmom, s);
+  launch_node_average(c.emom, c.ne_off, c.ne_list, c.nn, c.nmom, nullptr, 0, s);
   c.corr_pending = true;
   c.launches += 4;
   launch_add(c.nn, c.dP, c.P, s);

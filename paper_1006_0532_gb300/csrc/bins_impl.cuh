@@ -1945,6 +1945,20 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 ? 1280 : 1024) / 256) ran
   }
 }
 
+// Every element of a small grid in one launch, a block per element on the bucket-rank tile of
+// kTileBig (larger ones: stats_big_kernel): the classes' launches and their branches cost
+// more than they save there.
+template <typename T>
+__global__ void __launch_bounds__(256, (sizeof(T) == 4 ? 1280 : 1024) / 256) small_grid_kernel(const StatsArgs<T> a) {
+  extern __shared__ __align__(16) unsigned char rank_smem[];
+  RankTile<T, kTileBig, 256>& t = *reinterpret_cast<RankTile<T, kTileBig, 256>*>(rank_smem);
+  const int e = blockIdx.x;
+  if (e == 0 && threadIdx.x == 0 && a.step_inc) atomicAdd(a.step_inc, 1u);
+  const int moves = a.scal[16 * (a.einst ? a.einst[e] : 0)] > 0;
+  const int N = moves ? a.fin[e] : a.cnt[e];
+  if (N <= kTileBig) element_rank_tile<T, kTileBig, 256>(a, t, e, N, moves);
+}
+
 template <typename T> bool rank_configured[kMaxDevices];
 
 // One block per entry of one size class of the plan's tile lists (tile_element); the grid
@@ -1964,6 +1978,36 @@ __global__ void __launch_bounds__(THREADS, (sizeof(T) == 4 ? 1536 : 1024) / THRE
 }  // namespace
 
 template <typename T>
+void configure_tiles() {
+  if (!first_use_on_device(rank_configured<T>)) return;
+  constexpr size_t big = sizeof(RankTile<T, kTileBig, 256>);
+  static_assert(big <= 227 * 1024, "rank tile exceeds shared memory");
+  auto allow = [](const void* f, size_t bytes) {
+    cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
+  };
+  allow(reinterpret_cast<const void*>(small_grid_kernel<T>), big);
+  allow(reinterpret_cast<const void*>(rank_big_kernel<T>), big);
+  allow(reinterpret_cast<const void*>(rank_tile_kernel<T, 768, 192, 1>), sizeof(RankTile<T, 768, 192>));
+  allow(reinterpret_cast<const void*>(rank_list_kernel<T, 768, 192, 1>), sizeof(RankTile<T, 768, 192>));
+  allow(reinterpret_cast<const void*>(rank_tile_kernel<T, 512, 128, 2>), sizeof(RankTile<T, 512, 128>));
+  allow(reinterpret_cast<const void*>(rank_list_kernel<T, 512, 128, 2>), sizeof(RankTile<T, 512, 128>));
+  allow(reinterpret_cast<const void*>(warp_tile_kernel<T, 256, 4, 0>), warp_tile_smem<T, 256, 4>());
+  allow(reinterpret_cast<const void*>(warp_tile_kernel<T, 512, 2, 2>), warp_tile_smem<T, 512, 2>());
+}
+
+// A grid of up to four elements per multiprocessor (us per step, classes / one launch: 64
+// elements of 100 particles FP32 61.0 / 55.6, FP64 85.3 / 79.9; 400: 63.5 / 59.6, 113.7 /
+// 112.4; 900: 66.2 / 70.4, 170.0 / 166.7; 1,600: 73.5 / 83.9, 211 / 238).
+constexpr int kSmallGrid = 4;
+template <typename T>
+bool launch_stats_small_impl(const StatsArgs<T>& a, int num_sms, cudaStream_t s) {
+  if (a.ne <= 0 || a.ne > kSmallGrid * num_sms) return false;
+  configure_tiles<T>();
+  small_grid_kernel<T><<<static_cast<unsigned>(a.ne), 256, sizeof(RankTile<T, kTileBig, 256>), s>>>(a);
+  return true;
+}
+
+template <typename T>
 void launch_stats_tiles_impl(const StatsArgs<T>& a, int num_sms, cudaStream_t s_small, cudaStream_t s_mid,
                              cudaStream_t s_large) {
   if (a.ne <= 0) return;
@@ -1979,27 +2023,15 @@ void launch_stats_tiles_impl(const StatsArgs<T>& a, int num_sms, cudaStream_t s_
     stats_tile_kernel<T, 256, 128, 0, true><<<grid, 128, 0, s_small>>>(a);
     stats_tile_kernel<T, 512, 128, 2, true><<<grid, 128, 0, s_mid>>>(a);
   } else {
-    constexpr size_t big = sizeof(RankTile<T, kTileBig, 256>);
-    static_assert(big <= 227 * 1024, "rank tile exceeds shared memory");
-    if (first_use_on_device(rank_configured<T>)) {
-      auto allow = [](const void* f, size_t bytes) {
-        cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
-      };
-      allow(reinterpret_cast<const void*>(rank_big_kernel<T>), big);
-      allow(reinterpret_cast<const void*>(rank_tile_kernel<T, 768, 192, 1>), sizeof(RankTile<T, 768, 192>));
-      allow(reinterpret_cast<const void*>(rank_list_kernel<T, 768, 192, 1>), sizeof(RankTile<T, 768, 192>));
-      allow(reinterpret_cast<const void*>(rank_tile_kernel<T, 512, 128, 2>), sizeof(RankTile<T, 512, 128>));
-      allow(reinterpret_cast<const void*>(rank_list_kernel<T, 512, 128, 2>), sizeof(RankTile<T, 512, 128>));
-      allow(reinterpret_cast<const void*>(warp_tile_kernel<T, 256, 4, 0>), warp_tile_smem<T, 256, 4>());
-      allow(reinterpret_cast<const void*>(warp_tile_kernel<T, 512, 2, 2>), warp_tile_smem<T, 512, 2>());
-    }
+    configure_tiles<T>();
     // the classes above the mean count by a factor of two and more hold few elements: over
     // their lists where blocks that return would take 10 us and more (0.5 ns each)
     const int64_t mean = a.np / a.ne;
     const int few = a.ne >= 20000 ? 8 * (num_sms > 0 ? num_sms : 1) : 0;
     launch_rank_tile<T, 768, 192, 1>(a, mean <= 256 ? few : 0, s_large);
     // 769..1024 from the large-element list: 4 blocks per SM
-    rank_big_kernel<T><<<static_cast<unsigned>(4 * (num_sms > 0 ? num_sms : 1)), 256, big, s_large>>>(a);
+    rank_big_kernel<T><<<static_cast<unsigned>(4 * (num_sms > 0 ? num_sms : 1)), 256,
+                         sizeof(RankTile<T, kTileBig, 256>), s_large>>>(a);
     launch_warp_tile<T, 256, 4, 0>(a, s_small);
     // 257..512: a block per element with bucket levels in the FP32 form; where the moment sums
     // are FP64 a warp per element, whose register sort leaves the FP64 pipe the shorter wait

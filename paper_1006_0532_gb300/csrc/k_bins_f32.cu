@@ -9,4 +9,9 @@ void launch_stats_tiles<float>(const StatsArgs<float>& a, int num_sms, cudaStrea
   launch_stats_tiles_impl<float>(a, num_sms, s_small, s_mid, s_large);
 }
 
+template <>
+bool launch_stats_small<float>(const StatsArgs<float>& a, int num_sms, cudaStream_t s) {
+  return launch_stats_small_impl<float>(a, num_sms, s);
+}
+
 }  // namespace pdfx

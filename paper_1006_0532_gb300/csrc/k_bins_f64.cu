@@ -9,4 +9,9 @@ void launch_stats_tiles<double>(const StatsArgs<double>& a, int num_sms, cudaStr
   launch_stats_tiles_impl<double>(a, num_sms, s_small, s_mid, s_large);
 }
 
+template <>
+bool launch_stats_small<double>(const StatsArgs<double>& a, int num_sms, cudaStream_t s) {
+  return launch_stats_small_impl<double>(a, num_sms, s);
+}
+
 }  // namespace pdfx

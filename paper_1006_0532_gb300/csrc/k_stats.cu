@@ -222,6 +222,7 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(Plan pl, int32_t ne_
   // pass 1: offsets of the element lists, min / max, big elements (no moves)
   int32_t carry = p0, lmin = 0x7fffffff, lmax = -1, tA = 0, tB = 0, tM = 0;
   if (tid == 0 && !pass1_done) scal[3] = 0;
+  if (tid == 0 && inst == 0 && pl.brute_count) *pl.brute_count = 0;   // this step's search is done
   __syncthreads();
   // each pass's counts are loaded one pass ahead, so that the load overlaps the scan
   int32_t c_next = tid < ne && !pass1_done ? pl.cnt[eb + tid] : 0;
@@ -887,8 +888,12 @@ struct NodeRecip {
 __device__ const NodeRecip g_node_recip{};
 
 __global__ void node_average_kernel(const double* __restrict__ emom, const int32_t* __restrict__ ne_off,
-                                    const int32_t* __restrict__ ne_list, int32_t nn, double* nmom) {
+                                    const int32_t* __restrict__ ne_list, int32_t nn, double* nmom, int32_t* cnt,
+                                    int32_t ne) {
   const int64_t k = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  // the last kernel of a statistics pass also leaves the counts at zero for the next advance
+  if (cnt)
+    for (int64_t e = k; e < ne; e += static_cast<int64_t>(gridDim.x) * blockDim.x) cnt[e] = 0;
   if (k >= static_cast<int64_t>(nn) * kNS) return;
   const int32_t n = static_cast<int32_t>(k / kNS);
   const int s = static_cast<int>(k - static_cast<int64_t>(n) * kNS);
@@ -913,8 +918,10 @@ int launch_plan(Plan& pl, int32_t ne, int K, int minnpel, int allow_moves, cudaS
   // one instance with its histogram scratch: pass 1 over many blocks (the chunk totals live
   // in the histogram, which only the later passes of the particle-number control use), then
   // the one-block kernel for those passes, which returns at once when no particle moves
+  // (few elements: the one-block kernel takes pass 1 too, about 2 us per 1,024 elements
+  // against two more launches)
   const int nchunks = ne > 0 ? (ne + kPlanThreads - 1) / kPlanThreads : 1;
-  if (K <= 1 && pl.hist && nchunks <= kHistCap) {
+  if (K <= 1 && pl.hist && nchunks > 4 && nchunks <= kHistCap) {
     plan_chunk_totals<<<static_cast<unsigned>(nchunks), kPlanThreads, 0, s>>>(pl, ne, pl.hist);
     plan_chunk_offsets<<<static_cast<unsigned>(nchunks), kPlanThreads, 0, s>>>(pl, ne, nchunks, pl.hist);
     plan_kernel<<<1, kPlanThreads, 0, s>>>(pl, ne, minnpel, allow_moves, 1);
@@ -946,13 +953,19 @@ void launch_redistribute(Particles<T> p, Plan& pl, int K, const InstDev<T>* inst
   commit_moves_kernel<T><<<grid, 256, 0, s>>>(p, pl, K, np, ne, diag, err);
 }
 
+// Returns the kernels launched.
 template <typename T>
-void launch_stats(const StatsArgs<T>& a, int num_sms, cudaStream_t s, const SideStreams* side) {
+int launch_stats(const StatsArgs<T>& a, int num_sms, cudaStream_t s, const SideStreams* side) {
   const size_t big = stats_smem_bytes<T>(kBigCap);
   static_assert(5 * 8 * kBigCap + 11 * kBigCap <= 227 * 1024, "large-element tile exceeds shared memory");
   if (first_use_on_device(stats_configured<T>)) {
     cudaFuncSetAttribute(stats_big_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          static_cast<int>(big));
+  }
+  // a small grid: one launch for every element up to kTileBig, no branches
+  if (a.cond_mode != 1 && launch_stats_small<T>(a, num_sms, s)) {
+    stats_big_kernel<T><<<static_cast<unsigned>(num_sms > 0 ? num_sms : 1), kStatsThreads, big, s>>>(a);
+    return 2;
   }
   // The tile classes and the large-element kernel take disjoint elements and write disjoint
   // outputs: with the context's side streams they run as parallel branches (the 513..768
@@ -977,13 +990,16 @@ void launch_stats(const StatsArgs<T>& a, int num_sms, cudaStream_t s, const Side
     cudaStreamWaitEvent(s, side->ev[1], 0);
     cudaStreamWaitEvent(s, side->ev[2], 0);
   }
+  // three tile classes, the large-element kernel and (hierarchical bins) the bucket-rank tile
+  // over the large-element list
+  return a.cond_mode == 1 ? 4 : 5;
 }
 
 void launch_node_average(const double* emom, const int32_t* ne_off, const int32_t* ne_list,
-                         int32_t nn, double* nmom, cudaStream_t s) {
+                         int32_t nn, double* nmom, int32_t* cnt, int32_t ne, cudaStream_t s) {
   if (nn <= 0) return;
   const int64_t work = static_cast<int64_t>(nn) * kNS;
-  node_average_kernel<<<static_cast<unsigned>((work + 255) / 256), 256, 0, s>>>(emom, ne_off, ne_list, nn, nmom);
+  node_average_kernel<<<static_cast<unsigned>((work + 255) / 256), 256, 0, s>>>(emom, ne_off, ne_list, nn, nmom, cnt, ne);
 }
 
 namespace {
@@ -1188,7 +1204,7 @@ template void launch_derive_fields<double>(const ElemGeo<double>*, const ElemTop
                                        int64_t, const ElemGeo<T>*, const ElemTopo*,            \
                                        const uint32_t*,                                        \
                                        int, unsigned long long*, int*, cudaStream_t);          \
-  template void launch_stats<T>(const StatsArgs<T>&, int, cudaStream_t, const SideStreams*);
+  template int launch_stats<T>(const StatsArgs<T>&, int, cudaStream_t, const SideStreams*);
 PDFX_INSTANTIATE(double)
 PDFX_INSTANTIATE(float)
 #undef PDFX_INSTANTIATE

@@ -174,6 +174,7 @@ struct Plan {
   int32_t* movers = nullptr;   // [np] particle slots that move (by move index)
   int32_t* mrecip = nullptr;   // [np] recipient element per move
   double* mvals = nullptr;     // [np][7] new values per move
+  int* brute_count = nullptr;  // the brute-force list's length, zeroed by the plan for the next advance
   int tile_split = 256;        // elements of up to this many particles take the tile of
                                // kTileSplit (a warp each; chunk sorts for Fox's
                                // projection); larger ones up to kTileMid the tile of kTileMid
@@ -265,6 +266,7 @@ struct Ctx {
   int32_t* ne_list = nullptr;   // [3 ne]
   std::vector<int32_t> h_ne_off, h_ne_list;
   bool have_grid = false;
+  bool counts_clear = false;    // plan.cnt is zero on the stream: the last statistics pass cleared it
   // fields
   void* fields = nullptr;       // T[nn][32]
   double* fields64 = nullptr;   // staging for the FP32 conversion
@@ -379,14 +381,18 @@ void launch_redistribute(Particles<T> p, Plan& pl, int K, const InstDev<T>* inst
                          int64_t np, const ElemGeo<T>* geo, const ElemTopo* topo, const uint32_t* stepc,
                          int num_sms, unsigned long long* diag, int* err, cudaStream_t s);
 template <typename T>
-void launch_stats(const StatsArgs<T>& a, int num_sms, cudaStream_t s, const SideStreams* side);
+int launch_stats(const StatsArgs<T>& a, int num_sms, cudaStream_t s, const SideStreams* side);   // kernels launched
 // The tile classes of up to 256, 257..512 and 513..768 particles on s_small, s_mid and
 // s_large (k_bins_f32.cu / k_bins_f64.cu).
+// The hierarchical bins of a small grid in one launch (elements of up to kTileBig particles).
+template <typename T>
+bool launch_stats_small(const StatsArgs<T>& a, int num_sms, cudaStream_t s);   // false: not a small grid
 template <typename T>
 void launch_stats_tiles(const StatsArgs<T>& a, int num_sms, cudaStream_t s_small, cudaStream_t s_mid,
                         cudaStream_t s_large);
+// cnt: counts [ne] to clear for the next step (nullptr: none).
 void launch_node_average(const double* emom, const int32_t* ne_off, const int32_t* ne_list,
-                         int32_t nn, double* nmom, cudaStream_t s);
+                         int32_t nn, double* nmom, int32_t* cnt, int32_t ne, cudaStream_t s);
 // Eq. 26: max over nodes of ||(<U>, <V>, <W>, <omega>, <psi>)||_2 into out[0] (one block).
 void launch_cfl_norm(const double* nmom, int32_t nn, double* out, cudaStream_t s);
 // Eq. 31 (rho = 1): U -= dt grad(dP) with the element-constant gradient of the nodal dP[nn];

@@ -1,4 +1,4 @@
-"""The binning's warp tiles at the sizes, bin shapes and values where their sort could go wrong:
+"""The binning's warp tiles, and the one launch of a small grid, at the sizes, bin shapes and values where their sort could go wrong:
 empty elements, one word more or less than a register column, mapped values that collide, runs
 of equal velocities ordered by particle id, signed zeros and a wide range of magnitudes."""
 import numpy as np
@@ -44,15 +44,17 @@ def _state(g, values, seed):
     return {k: np.ascontiguousarray(v[perm]) for k, v in st.items()} | {"elem": np.ascontiguousarray(elem[perm])}
 
 
+@pytest.mark.parametrize("rows", [5, 18])    # 64 elements (one launch) and 680 (size classes)
 @pytest.mark.parametrize("precision", [0, 1])
 @pytest.mark.parametrize("values", ["spread", "few", "equal", "wide"])
 @pytest.mark.parametrize("bins,mpb", [((4, 4, 4), 2), ((1, 1, 1), 1), ((16, 1, 1), 1), ((1, 4, 1), 3), ((2, 3, 5), 1),
                                       ((16, 16, 1), 1), ((1, 1, 7), 2)])
-def test_order_bins_and_pointers_are_the_oracles(precision, values, bins, mpb):
+def test_order_bins_and_pointers_are_the_oracles(rows, precision, values, bins, mpb):
     """Pointers and effective bins exactly, conditional means and moments within the form's
     tolerance, for both size-class splits (which agree bit for bit)."""
-    g = synth.workload("channel_tiny")["grid"]
     w = synth.workload("channel_tiny")
+    g = w["grid"] if rows == 5 else synth.channel_grid(20, rows, seed=9)
+    w["fields"] = synth.channel_fields(g, 392.0)
     params = dict(w["params"], bins=bins, min_per_bin=mpb, minnpel=0)
     st = _state(g, values, 5)
     outs = []
