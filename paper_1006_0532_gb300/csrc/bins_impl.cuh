@@ -1950,6 +1950,8 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 ? 1280 : 1024) / 256) ran
 // more than they save there.
 template <typename T>
 __global__ void __launch_bounds__(256, (sizeof(T) == 4 ? 1280 : 1024) / 256) small_grid_kernel(const StatsArgs<T> a) {
+  chain_wait();
+  chain_go();
   extern __shared__ __align__(16) unsigned char rank_smem[];
   RankTile<T, kTileBig, 256>& t = *reinterpret_cast<RankTile<T, kTileBig, 256>*>(rank_smem);
   const int e = blockIdx.x;
@@ -2003,7 +2005,7 @@ template <typename T>
 bool launch_stats_small_impl(const StatsArgs<T>& a, int num_sms, cudaStream_t s) {
   if (a.ne <= 0 || a.ne > kSmallGrid * num_sms) return false;
   configure_tiles<T>();
-  small_grid_kernel<T><<<static_cast<unsigned>(a.ne), 256, sizeof(RankTile<T, kTileBig, 256>), s>>>(a);
+  launch_chained(small_grid_kernel<T>, a.ne, 256, sizeof(RankTile<T, kTileBig, 256>), s, a);
   return true;
 }
 

@@ -405,6 +405,8 @@ __device__ __forceinline__ void update_f64(const Model<double>& M, const Step64&
 // counters are flushed once, after its last tile.
 template <typename T, bool BATCH, bool PLAIN = false>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) advance_kernel(const AdvanceArgs<T> a) {
+  chain_wait();
+  chain_go();
   __shared__ unsigned bc[kDiagCount];
   block_counts_clear(bc);
   const int64_t ntiles = (a.np + blockDim.x - 1) / blockDim.x;
@@ -610,6 +612,8 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) advance_kernel(co
 // no-slip walls; free-slip reflection, wrap, source and walk as in the full model.
 template <typename T, bool BATCH>
 __global__ void __launch_bounds__(256) simple_advance_kernel(const AdvanceArgs<T> a) {
+  chain_wait();
+  chain_go();
   __shared__ unsigned bc[kDiagCount];
   block_counts_clear(bc);
   const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -663,6 +667,8 @@ __global__ void __launch_bounds__(256) simple_advance_kernel(const AdvanceArgs<T
 // particle in no element is flagged.
 template <typename T, bool BATCH>
 __global__ void __launch_bounds__(256) brute_search_kernel(AdvanceArgs<T> a) {
+  chain_wait();
+  chain_go();
   __shared__ int best_s[8];
   const int n = min(*a.brute_count, a.brute_cap);
   for (int j = blockIdx.x; j < n; j += gridDim.x) {
@@ -915,14 +921,14 @@ void launch_advance(const AdvanceArgs<T>& a, int num_sms, int block, cudaStream_
   const unsigned resident = bgrid * static_cast<unsigned>(1024 / block);
   const unsigned agrid = sizeof(T) == 4 && grid > 16u * resident ? 16u * resident : grid;
   if (a.einst) {
-    if (a.m.model == 1) simple_advance_kernel<T, true><<<grid, block, 0, s>>>(a);
-    else advance_kernel<T, true><<<agrid, block, 0, s>>>(a);
-    brute_search_kernel<T, true><<<bgrid, 256, 0, s>>>(a);
+    if (a.m.model == 1) launch_chained(simple_advance_kernel<T, true>, grid, block, 0, s, a);
+    else launch_chained(advance_kernel<T, true>, agrid, block, 0, s, a);
+    launch_chained(brute_search_kernel<T, true>, bgrid, 256, 0, s, a);
   } else {
-    if (a.m.model == 1) simple_advance_kernel<T, false><<<grid, block, 0, s>>>(a);
-    else if (sizeof(T) == 8 && a.coupled) advance_kernel<T, false, sizeof(T) == 8><<<agrid, block, 0, s>>>(a);
-    else advance_kernel<T, false><<<agrid, block, 0, s>>>(a);
-    brute_search_kernel<T, false><<<bgrid, 256, 0, s>>>(a);
+    if (a.m.model == 1) launch_chained(simple_advance_kernel<T, false>, grid, block, 0, s, a);
+    else if (sizeof(T) == 8 && a.coupled) launch_chained(advance_kernel<T, false, sizeof(T) == 8>, agrid, block, 0, s, a);
+    else launch_chained(advance_kernel<T, false>, agrid, block, 0, s, a);
+    launch_chained(brute_search_kernel<T, false>, bgrid, 256, 0, s, a);
   }
 }
 

@@ -358,6 +358,33 @@ inline bool first_use_on_device(bool (&flags)[kMaxDevices]) {
   return true;
 }
 
+// A step is a chain of kernels, most of them a few microseconds long on small grids, each
+// waiting for the one before.  Launched with launch_chained, a kernel may be set up while its
+// predecessor in the stream still runs (programmatic stream serialisation); it calls
+// chain_wait() before its first access to memory, which returns once the predecessor has
+// completed and its writes are visible, and chain_go() to let its own successor be set up.
+// Kernels launched in the ordinary way wait for everything before them as always.  Measured, a
+// step of 64 elements of 40 particles, FP64, 10 launches: 88.5 us with ordinary launches, 68 so;
+// 1,536 elements of 200 with redistribution: 189 us and 170.  A kernel that is most of a step
+// gains nothing and loses nothing.
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... P, typename... A>
+void launch_chained(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, A... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // Kernel launchers (defined in the .cu files).
 template <typename T>
 void launch_advance(const AdvanceArgs<T>& a, int num_sms, int block, cudaStream_t s);   // block <= 256
