@@ -532,33 +532,49 @@ int do_get_particles(Ctx& c, pdfx_soa* soa, int on_device, cudaStream_t s) {
 
 // Element geometry in the working precision: node coordinates (canonical x; FP32 form: as
 // FP32 pairs), the edges' vectors and 1 / (2 A_e).
-void geo_nodes(const HostGeo& g, int32_t e, ElemGeo<double>& o) {
+void place_edge(ElemGeo<double>& o, int k, int pivot, bool flip, double ex, double ey) {
+  o.ex[k] = ex;
+  o.ey[k] = ey;
+  o.code |= (static_cast<uint32_t>(pivot) | (flip ? 4u : 0u)) << (3 * k);
+}
+void place_nodes(const HostGeo& g, int32_t e, const int32_t*, const ElemTopo&, ElemGeo<double>& o) {
   for (int k = 0; k < 3; ++k) {
     o.x[k] = g.nx[3 * e + k];
     o.y[k] = g.vy[3 * e + k];
   }
-  o.pad = 0;
+  o.code = o.pad = 0u;
 }
-void geo_nodes(const HostGeo& g, int32_t e, ElemGeo<float>& o) {
-  for (int k = 0; k < 3; ++k) {
-    pair_of(g.nx[3 * e + k], o.xh[k], o.xl[k]);
-    pair_of(g.vy[3 * e + k], o.yh[k], o.yl[k]);
-  }
-  o.pad[0] = o.pad[1] = 0.0f;
+void place_edge(ElemGeo<float>& o, int k, int, bool flip, double ex, double ey) {
+  const int r = static_cast<int>((o.code >> (2 * k)) & 3u);
+  o.ex[r] = static_cast<float>(flip ? -ex : ex);
+  o.ey[r] = static_cast<float>(flip ? -ey : ey);
 }
-template <typename T>
-void geo_of(const HostGeo& g, int32_t e, const int32_t* tri, double L, ElemGeo<T>& o) {
-  geo_nodes(g, e, o);
-  // edge opposite vertex k: counter-clockwise from a = k + 1 to b = k + 2; pivot at the
-  // lower node id, vector from the pivot to the other node (minimum image in x)
+void place_nodes(const HostGeo& g, int32_t e, const int32_t* id, const ElemTopo& t, ElemGeo<float>& o) {
   o.code = 0u;
   for (int k = 0; k < 3; ++k) {
+    int r = 0;
+    for (int m = 0; m < 3; ++m) r += id[m] < id[k] ? 1 : 0;
+    GeoNode& n = r == 0 ? o.lo : (r == 1 ? o.mid : o.hi);
+    pair_of(g.nx[3 * e + k], n.xh, n.xl);
+    pair_of(g.vy[3 * e + k], n.yh, n.yl);
+    o.code |= static_cast<uint32_t>(r) << (2 * k);
+  }
+  o.nb[0] = t.nb0;
+  o.nb[1] = t.nb1;
+  o.nb[2] = t.nb2;
+  o.pad = 0;
+}
+template <typename T>
+void geo_of(const HostGeo& g, int32_t e, const int32_t* tri, const ElemTopo& t, double L, ElemGeo<T>& o) {
+  const int32_t* id = tri + 3 * static_cast<size_t>(e);
+  place_nodes(g, e, id, t, o);
+  // edge opposite vertex k: counter-clockwise from a = k + 1 to b = k + 2; pivot at the
+  // lower node id, vector from the pivot to the other node (minimum image in x)
+  for (int k = 0; k < 3; ++k) {
     const int a = (k + 1) % 3, b = (k + 2) % 3;
-    const bool flip = tri[3 * e + b] < tri[3 * e + a];
+    const bool flip = id[b] < id[a];
     const int p = flip ? b : a, q = flip ? a : b;
-    o.ex[k] = static_cast<T>(min_image(g.nx[3 * e + q] - g.nx[3 * e + p], L));
-    o.ey[k] = static_cast<T>(g.vy[3 * e + q] - g.vy[3 * e + p]);
-    o.code |= (static_cast<uint32_t>(p) | (flip ? 4u : 0u)) << (3 * k);
+    place_edge(o, k, p, flip, min_image(g.nx[3 * e + q] - g.nx[3 * e + p], L), g.vy[3 * e + q] - g.vy[3 * e + p]);
   }
   o.inv2a = static_cast<T>(1.0 / g.area2[e]);
 }
@@ -579,7 +595,7 @@ int upload_grid(Ctx& c, const HostGeo& g, const std::vector<ElemTopo>& topo,
                 const std::vector<double>& fse, const int32_t* tri, const std::vector<double>& period) {
   const int32_t ne = c.ne;
   std::vector<ElemGeo<T>> hg(static_cast<size_t>(ne));
-  for (int32_t e = 0; e < ne; ++e) geo_of(g, e, tri, period[e], hg[e]);
+  for (int32_t e = 0; e < ne; ++e) geo_of(g, e, tri, topo[e], period[e], hg[e]);
   dev_free(c, c.geo);
   c.geo = dev_alloc(c, sizeof(ElemGeo<T>) * ne);
   if (!c.geo) return PDFX_ERR_ALLOC;

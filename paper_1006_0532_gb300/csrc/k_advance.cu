@@ -35,10 +35,23 @@ __device__ __forceinline__ int lowest(double a, double b, double c) {
 }
 
 template <typename T>
-__device__ __forceinline__ bool inside(const ElemGeo<T>& g, const ElemTopo& t, const Pos<T>& P, T L) {
-  T na, nb, nc;
-  area_cross(g, t.n0, t.n1, t.n2, P, L, na, nb, nc);
-  return nonneg(na) && nonneg(nb) && nonneg(nc);
+__device__ __forceinline__ bool inside(const ElemGeo<T>& g, const Pos<T>& P, T L) {
+  T n[3];
+  area_cross(g, P, L, n);
+  return nonneg(n[0]) && nonneg(n[1]) && nonneg(n[2]);
+}
+
+// The neighbour across the edge opposite local vertex k (the FP32 form's geometry has them,
+// the FP64 form reads the topology with the geometry).
+struct Neighbours {
+  int nb0, nb1, nb2;
+};
+__device__ __forceinline__ Neighbours neighbours(const ElemGeo<float>& g, const ElemTopo*, int) {
+  return {g.nb[0], g.nb[1], g.nb[2]};
+}
+__device__ __forceinline__ Neighbours neighbours(const ElemGeo<double>&, const ElemTopo* topo, int e) {
+  const ElemTopo t = topo[e];
+  return {t.nb0, t.nb1, t.nb2};
 }
 
 // Sect. 3.6: walk to the neighbour opposite the lowest area coordinate (ties: lowest local
@@ -55,12 +68,13 @@ __device__ int walk(const AdvanceArgs<T>& a, int e0, Pos<T>& P, T (&U)[3], T L, 
   hops = 0;
   for (;;) {
     const ElemGeo<T> g = a.geo[e];
-    const ElemTopo t = a.topo[e];
-    T la, lb, lc;   // 2 N^k: signs and order of the area coordinates
-    area_cross(g, t.n0, t.n1, t.n2, P, L, la, lb, lc);
-    if (nonneg(la) && nonneg(lb) && nonneg(lc)) return e;
+    const Neighbours t = neighbours(g, a.topo, e);
+    T n[3];   // 2 N^k: signs and order of the area coordinates
+    area_cross(g, P, L, n);
+    if (nonneg(n[0]) && nonneg(n[1]) && nonneg(n[2])) return e;
     if (hops >= kHopLimit) break;
-    const int k = lowest(la, lb, lc);
+    local_order(g, n);
+    const int k = lowest(n[0], n[1], n[2]);
     const int nb = k == 0 ? t.nb0 : (k == 1 ? t.nb1 : t.nb2);
     if (nb < 0) {
       if (nb == -1) break;
@@ -87,7 +101,7 @@ __device__ int walk(const AdvanceArgs<T>& a, int e0, Pos<T>& P, T (&U)[3], T L, 
     for (int i = a.ne_off[nd]; i < a.ne_off[nd + 1]; ++i) {
       const int f = a.ne_list[i];
       if (best >= 0 && f >= best) continue;
-      if (inside(a.geo[f], a.topo[f], P, L)) best = f;
+      if (inside(a.geo[f], P, L)) best = f;
     }
   }
   if (best >= 0) return best;
@@ -183,11 +197,6 @@ __device__ __forceinline__ void warp_count(unsigned long long* diag, int slot, i
   const unsigned s = __reduce_add_sync(kFull, static_cast<unsigned>(v));
   if ((threadIdx.x & 31) == 0 && s) atomicAdd(diag + slot, static_cast<unsigned long long>(s));
 }
-// The same per warp into the block's counters in shared memory.
-__device__ __forceinline__ void warp_count(unsigned* bc, int slot, int v) {
-  const unsigned s = __reduce_add_sync(kFull, static_cast<unsigned>(v));
-  if ((threadIdx.x & 31) == 0 && s) atomicAdd(bc + slot, s);
-}
 // Block counters: cleared at the start of a kernel, added to the diagnostics at its end (one
 // global atomic per block and counter instead of one per warp on the same address).
 __device__ __forceinline__ void block_counts_clear(unsigned* bc) {
@@ -200,11 +209,11 @@ __device__ __forceinline__ void block_counts_flush(unsigned* bc, unsigned long l
     if (bc[k]) atomicAdd(diag + k, static_cast<unsigned long long>(bc[k]));
 }
 
-// Per-particle event flags of one update, summed per warp into the diagnostics.
+// The events of one particle update: bit k for the diagnostic k (below 32), and the hops.
 struct StepFlags {
-  int hops = 0, fb = 0, brute = 0, lost = 0, wall = 0, fs = 0, oref = 0, c0 = 0, gex = 0,
-      src = 0, nf = 0;
-  int hop_bin = -1;
+  unsigned ev = 0;
+  int hops = 0;
+  __device__ __forceinline__ void set(int k) { ev |= 1u << k; }
 };
 
 // The end of one particle update, common to both models: free-slip reflection with reversal
@@ -221,7 +230,7 @@ __device__ __forceinline__ int finish_update(const AdvanceArgs<T>& a, const Mode
     const Line<T> ln = a.fslines[tp.fslip];
     const T d1 = line_dist(ln, Pn, L);
     if (d1 < T(0)) {
-      f.fs = 1;
+      f.set(kDiagFreeSlip);
       pos_reflect(Pn, d1, ln.nx, ln.ny);
       const T un = Un[0] * ln.nx + Un[1] * ln.ny;
       Un[0] -= T(2) * un * ln.nx;
@@ -229,28 +238,27 @@ __device__ __forceinline__ int finish_update(const AdvanceArgs<T>& a, const Mode
     }
   }
   pos_wrap(Pn, L);
-  if (!state_finite(Pn, Un, wn, psin)) f.nf = 1;
+  if (!state_finite(Pn, Un, wn, psin)) f.set(kDiagNonFinite);
 
   int hops = 0, fb = 0, brute = 0, refl = 0;
   int e_new = walk(a, e, Pn, Un, L, hops, fb, brute, refl);
   f.hops = hops;
-  f.fb = fb;
-  f.brute = brute;
-  f.hop_bin = hops < 7 ? hops : 7;
+  if (fb) f.set(kDiagFallback);
+  if (brute) f.set(kDiagBrute);
   if (refl) {
-    f.fs = 1;
+    f.set(kDiagFreeSlip);
     pos_wrap(Pn, L);
   }
   if (M.source_on && in_source(M, Pn, L)) {
     psin = T(1);
-    f.src = 1;
+    f.set(kDiagSource);
   }
   if (e_new < 0) {
     // counted in the old element for now; the brute-force kernel moves it (or flags it)
     e_new = e;
     const int at = atomicAdd(a.brute_count, 1);
     if (at < a.brute_cap) a.brute_list[at] = static_cast<int32_t>(i);
-    else f.lost = 1;
+    else f.set(kDiagLost);
   }
 
   store_pos(a.p, i, Pn);
@@ -282,25 +290,22 @@ __device__ __forceinline__ void count_update(const AdvanceArgs<T>& a, bool valid
     }
   }
   // hops: the few lanes that hopped add to the block's counters themselves
-  if (f.hops > 0) atomicAdd(bc + kDiagHops, static_cast<unsigned>(f.hops));
-  if (__any_sync(kFull, f.fb | f.brute | f.lost | f.nf | f.gex | f.c0)) {
-    warp_count(bc, kDiagFallback, f.fb);
-    warp_count(bc, kDiagBrute, f.brute);
-    warp_count(bc, kDiagLost, f.lost);
-    warp_count(bc, kDiagNonFinite, f.nf);
-    warp_count(bc, kDiagGammaExhausted, f.gex);
-    warp_count(bc, kDiagC0Clamp, f.c0);
+  if (f.hops > 0) {
+    atomicAdd(bc + kDiagHops, static_cast<unsigned>(f.hops));
+    atomicAdd(bc + kDiagHopHist0 + min(f.hops, 7), 1u);
   }
-  if (__any_sync(kFull, f.lost) && (threadIdx.x & 31) == 0) atomicCAS(a.err, 0, PDFX_ERR_LOST_PARTICLE);
-  if (__any_sync(kFull, f.nf) && (threadIdx.x & 31) == 0) atomicCAS(a.err, 0, PDFX_ERR_NONFINITE);
-  if (__any_sync(kFull, f.wall | f.fs | f.oref | f.src)) {
-    warp_count(bc, kDiagWall, f.wall);
-    warp_count(bc, kDiagFreeSlip, f.fs);
-    warp_count(bc, kDiagOmegaReflect, f.oref);
-    warp_count(bc, kDiagSource, f.src);
+  // events: each kind that some lane met, one after the other
+  for (unsigned m = __reduce_or_sync(kFull, f.ev); m; m &= m - 1) {
+    const int k = __ffs(m) - 1;
+    const unsigned lanes = __ballot_sync(kFull, (f.ev >> k) & 1u);
+    if ((threadIdx.x & 31) == 0) {
+      atomicAdd(bc + k, static_cast<unsigned>(__popc(lanes)));
+      if (k == kDiagLost) atomicCAS(a.err, 0, PDFX_ERR_LOST_PARTICLE);
+      if (k == kDiagNonFinite) atomicCAS(a.err, 0, PDFX_ERR_NONFINITE);
+    }
   }
-  if (f.hop_bin > 0) atomicAdd(bc + kDiagHopHist0 + f.hop_bin, 1u);
 }
+static_assert(kDiagHopHist0 < 32, "an event's bit is its diagnostic's slot");
 
 // The FP64 form's new velocity, position, frequency and scalar before the walls (Eqs. 7, 27,
 // 19, 24 with the closure of Eqs. 11, 18, 20, 25), from the fields q at the particle.  The
@@ -348,7 +353,7 @@ __device__ __forceinline__ void update_f64(const Model<double>& M, const Step64&
     s = fma(q[20], q[27], s); s = fma(q[21], q[28], s); s = fma(q[22], q[25], s);
     c0e = -2.0 / 3.0 * s * ik;
   }
-  if (!m64::nonneg(c0e) && c0e < 0.0) { c0e = 0.0; f.c0 = 1; }
+  if (!m64::nonneg(c0e) && c0e < 0.0) { c0e = 0.0; f.set(kDiagC0Clamp); }
   const double prod = -(q[23] * q[5] + q[26] * q[6] + q[26] * q[7] + q[24] * q[8] + q[27] * q[9] + q[28] * q[10]);
   const double Somega = M.Cw2 - M.Cw1 * prod * ieps;
   double itm;
@@ -393,7 +398,7 @@ __device__ __forceinline__ void update_f64(const Model<double>& M, const Step64&
   wn = fma(-(M.C3 * Omdt), w0 - Om, w0);
   wn = fma(-(Somega * Omdt), w0, wn);
   wn = fma(fabs(Om) * (D.s2c34sdt * m64::root(wpos)), xi[5], wn);
-  if (!m64::nonneg(wn) && wn < 0.0) { wn = -wn; f.oref = 1; }
+  if (!m64::nonneg(wn) && wn < 0.0) { wn = -wn; f.set(kDiagOmegaReflect); }
   psin = fma(-(psi0 - phic), D.dt * itm, psi0);
 }
 
@@ -442,7 +447,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) advance_kernel(co
       if (M.interp_mode == 1) {
         la = lb = lc = T(1) / T(3);
       } else {
-        area_coords(g, tp.n0, tp.n1, tp.n2, P0, L, la, lb, lc);
+        area_coords(g, P0, L, la, lb, lc);
       }
       T q[kNF];
       interp_fields(a.fields, tp.n0, tp.n1, tp.n2, la, lb, lc, q);
@@ -538,7 +543,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) advance_kernel(co
         // Eq. 27 (C0 eps < 0 is clamped under the root and counted);
         // G_ij (U_j - <U_j>) = (wp_ij (U_j - <U_j>) - eps/2 (U_i - <U_i>)) / k  (Eq. 11)
         T c0e = C0 * eps;
-        if (c0e < T(0)) { c0e = T(0); f.c0 = 1; }
+        if (c0e < T(0)) { c0e = T(0); f.set(kDiagC0Clamp); }
         const T sc0e = tsqrt(c0e) * sdt;
         const T dU[3] = {U0[0] - Um[0], U0[1] - Um[1], U0[2] - Um[2]};
 #pragma unroll
@@ -556,7 +561,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) advance_kernel(co
         const T wpos = w0 > T(0) ? w0 : T(0);
         wn = w0 - M.C3 * Om * (w0 - Om) * dt - Somega * Om * w0 * dt +
                tsqrt(T(2) * M.C3 * M.C4 * Om * Om * wpos) * (sdt * xi[5]);
-        if (wn < T(0)) { wn = -wn; f.oref = 1; }
+        if (wn < T(0)) { wn = -wn; f.set(kDiagOmegaReflect); }
         // Eq. 24 with the conditional mean of the particle's bin
         const T phic = static_cast<T>(a.vcce[(size_t)e * a.G + cpi]);
         psin = psi0 - (psi0 - phic) * dt * itm;
@@ -587,14 +592,14 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) advance_kernel(co
           }
         }
         if (any_hit) {
-          f.wall = 1;
+          f.set(kDiagWall);
           Un[0] = Un[1] = Un[2] = T(0);                  // Eq. 56
           int ex = 0;                                    // Eq. 58
           if constexpr (sizeof(T) == 8)
             q[30] = la * a.fields[(size_t)kNF * tp.n0 + 30] + lb * a.fields[(size_t)kNF * tp.n1 + 30] +
                     lc * a.fields[(size_t)kNF * tp.n2 + 30];
           wn = gamma_draw<T>(k0, k1, pid, step, kPurWallGamma, T(1) / M.C4, M.C4 * q[30], &ex);
-          f.gex = ex;
+          if (ex) f.set(kDiagGammaExhausted);
         }
       }
       e_new = finish_update(a, M, i, e, tp, Pn, Un, wn, psin, f);
@@ -636,7 +641,7 @@ __global__ void __launch_bounds__(256) simple_advance_kernel(const AdvanceArgs<T
     if (M.interp_mode == 1) {
       la = lb = lc = T(1) / T(3);
     } else {
-      area_coords(a.geo[e], tp.n0, tp.n1, tp.n2, P0, M.period_x, la, lb, lc);
+      area_coords(a.geo[e], P0, M.period_x, la, lb, lc);
     }
     const double* m0 = a.nmom + static_cast<size_t>(kNS) * tp.n0;
     const double* m1 = a.nmom + static_cast<size_t>(kNS) * tp.n1;
@@ -679,7 +684,7 @@ __global__ void __launch_bounds__(256) brute_search_kernel(AdvanceArgs<T> a) {
     const T L = BATCH ? a.inst[ki].m.period_x : a.m.period_x;
     int best = 0x7fffffff;
     for (int f = f0 + threadIdx.x; f < f1; f += blockDim.x)
-      if (f < best && inside(a.geo[f], a.topo[f], P, L)) best = f;
+      if (f < best && inside(a.geo[f], P, L)) best = f;
     for (int o = 16; o > 0; o >>= 1) best = min(best, __shfl_xor_sync(kFull, best, o));
     if ((threadIdx.x & 31) == 0) best_s[threadIdx.x >> 5] = best;
     __syncthreads();
@@ -730,7 +735,7 @@ __device__ __forceinline__ int init_one(Particles<T> p, int64_t i, int e, uint32
     if (m.interp_mode == 1) {
       la = lb = lc = T(1) / T(3);
     } else {
-      area_coords(g, tp.n0, tp.n1, tp.n2, P, m.period_x, la, lb, lc);
+      area_coords(g, P, m.period_x, la, lb, lc);
     }
     T q[kNF];
     interp_fields(fields, tp.n0, tp.n1, tp.n2, la, lb, lc, q);

@@ -34,14 +34,15 @@ constexpr int kBruteCap = 4096;    // particles per step that may need the brute
 // particle's offset from a node, and with it the area coordinates, keep FP32 precision
 // relative to the cell rather than to the domain (a first cell 4.6e-5 high at y = 1 is 770
 // FP32 spacings of y).
-template <typename T>
-struct ElemGeo;
 //
 // Both keep each edge's vector, from the edge's lower-numbered node (its pivot) to the other,
 // computed once in FP64 from the nodes' coordinates (and in the FP32 form rounded): the same
-// numbers for both elements of the edge.  code holds, for the edge opposite local vertex k,
-// the pivot's local index (bits 3k, 3k + 1) and whether the pivot is the edge's second
-// node in counter-clockwise order (bit 3k + 2, the cross product's sign flips).
+// numbers for both elements of the edge.
+template <typename T>
+struct ElemGeo;
+// FP64 form: code holds, for the edge opposite local vertex k, the pivot's local index (bits
+// 3k, 3k + 1) and whether the pivot is the edge's second node in counter-clockwise order (bit
+// 3k + 2, the cross product's sign flips).
 template <>
 struct __align__(16) ElemGeo<double> {
   double x[3], y[3];
@@ -49,13 +50,26 @@ struct __align__(16) ElemGeo<double> {
   double inv2a;
   uint32_t code, pad;
 };
+// FP32 form, whose advance is bound by the instructions it issues: the nodes in ascending order
+// of their ids, so that an edge's pivot needs no selection (node lo for the edges opposite mid
+// and hi, node mid for the one opposite lo) and the third node's offset is not formed; the
+// edges in the order of the nodes opposite them, their vectors negated where the cross
+// product's sign flips; and the neighbours (ElemTopo's, in local order), which the walk then
+// reads with the rest.  code: bits 2k, 2k + 1 the place of local vertex k in that order.
+// 12,100-triangle channel, 3.6M particles: 1,262 warp instructions per 32 particles and 166 us
+// with the nodes in local order (a selection per edge) and an event's own counter in every
+// thread, 1,073 and 155 us so; at 25M particles 1,050 us and 930.
+struct GeoNode {
+  float xh, yh, xl, yl;
+};
 template <>
 struct __align__(16) ElemGeo<float> {
-  float xh[3], yh[3], xl[3], yl[3];
+  GeoNode lo, mid;
   float ex[3], ey[3];
   float inv2a;
   uint32_t code;
-  float pad[2];
+  int32_t nb[3], pad;
+  GeoNode hi;
 };
 
 // Per-element topology: node ids, neighbour across the edge opposite each vertex (-1 = a
@@ -205,8 +219,18 @@ __host__ __device__ __forceinline__ double pair_value(float h, float l) {
 // Node k's coordinates as FP64 (the FP32 form's pairs summed).
 __device__ __forceinline__ double node_x(const ElemGeo<double>& g, int k) { return g.x[k]; }
 __device__ __forceinline__ double node_y(const ElemGeo<double>& g, int k) { return g.y[k]; }
-__device__ __forceinline__ double node_x(const ElemGeo<float>& g, int k) { return pair_value(g.xh[k], g.xl[k]); }
-__device__ __forceinline__ double node_y(const ElemGeo<float>& g, int k) { return pair_value(g.yh[k], g.yl[k]); }
+__device__ __forceinline__ GeoNode local_node(const ElemGeo<float>& g, int k) {
+  const uint32_t r = (g.code >> (2 * k)) & 3u;
+  return r == 0u ? g.lo : (r == 1u ? g.mid : g.hi);
+}
+__device__ __forceinline__ double node_x(const ElemGeo<float>& g, int k) {
+  const GeoNode n = local_node(g, k);
+  return pair_value(n.xh, n.xl);
+}
+__device__ __forceinline__ double node_y(const ElemGeo<float>& g, int k) {
+  const GeoNode n = local_node(g, k);
+  return pair_value(n.yh, n.yl);
+}
 
 // min_image and wrap_period of the FP64 form, their tests on the bits (a comparison takes the
 // FP64 pipe like any other operation): d stays while its high word is below L / 2's, which a
@@ -221,11 +245,16 @@ __device__ __forceinline__ double near_period(double x, double L) {
   return bl > 0 && (bx < 0 || bx >= bl) ? wrap_period(x, L) : x;
 }
 
-// Node m minus node k (minimum image in x), in the working precision.
-__device__ __forceinline__ void node_vec(const ElemGeo<float>& g, int k, int m, float L, float& ex,
-                                         float& ey) {
-  ex = __fadd_rn(min_image(__fsub_rn(g.xh[m], g.xh[k]), L), __fsub_rn(g.xl[m], g.xl[k]));
-  ey = __fadd_rn(__fsub_rn(g.yh[m], g.yh[k]), __fsub_rn(g.yl[m], g.yl[k]));
+// The FP32 form's: one comparison decides (the same differences as min_image's).
+__device__ __forceinline__ float near_image(float d, float L) {
+  if (L > 0.0f && fabsf(d) > 0.5f * L) return min_image(d, L);
+  return d;
+}
+
+// Node b minus node a (minimum image in x), in the working precision.
+__device__ __forceinline__ void node_vec(const GeoNode& a, const GeoNode& b, float L, float& ex, float& ey) {
+  ex = __fadd_rn(min_image(__fsub_rn(b.xh, a.xh), L), __fsub_rn(b.xl, a.xl));
+  ey = __fadd_rn(__fsub_rn(b.yh, a.yh), __fsub_rn(b.yl, a.yl));
 }
 // Particle minus node k (minimum image in x), in the working precision.
 __device__ __forceinline__ void node_rel(const ElemGeo<double>& g, int k, const Pos<double>& P, double L,
@@ -233,10 +262,9 @@ __device__ __forceinline__ void node_rel(const ElemGeo<double>& g, int k, const 
   dx = near_image(P.x - g.x[k], L);
   dy = P.y - g.y[k];
 }
-__device__ __forceinline__ void node_rel(const ElemGeo<float>& g, int k, const Pos<float>& P, float L,
-                                         float& dx, float& dy) {
-  dx = __fadd_rn(min_image(__fsub_rn(P.xh, g.xh[k]), L), __fsub_rn(P.xl, g.xl[k]));
-  dy = __fadd_rn(__fsub_rn(P.yh, g.yh[k]), __fsub_rn(P.yl, g.yl[k]));
+__device__ __forceinline__ void node_rel(const GeoNode& n, const Pos<float>& P, float L, float& dx, float& dy) {
+  dx = __fadd_rn(near_image(__fsub_rn(P.xh, n.xh), L), __fsub_rn(P.xl, n.xl));
+  dy = __fadd_rn(__fsub_rn(P.yh, n.yh), __fsub_rn(P.yl, n.yl));
 }
 
 // Particle minus a point given in FP64 (FP32 form: as the pair (ph, pl)), minimum image in x.
@@ -245,7 +273,7 @@ __device__ __forceinline__ double rel_x(const Pos<double>& P, double px, double,
 }
 __device__ __forceinline__ double rel_y(const Pos<double>& P, double py, double) { return P.y - py; }
 __device__ __forceinline__ float rel_x(const Pos<float>& P, float ph, float pl, float L) {
-  return __fadd_rn(min_image(__fsub_rn(P.xh, ph), L), __fsub_rn(P.xl, pl));
+  return __fadd_rn(near_image(__fsub_rn(P.xh, ph), L), __fsub_rn(P.xl, pl));
 }
 __device__ __forceinline__ float rel_y(const Pos<float>& P, float ph, float pl) {
   return __fadd_rn(__fsub_rn(P.yh, ph), __fsub_rn(P.yl, pl));
@@ -322,35 +350,48 @@ __device__ __forceinline__ float xmul(float a, float b) { return __fmul_rn(a, b)
 // evaluate it with identical rounding and opposite signs (watertight point location).
 // The particle's offsets from the three nodes, formed from the nodes' own coordinates and the
 // particle's alone, then each edge's stored vector crossed with the offset from its pivot.
-template <typename T>
-__device__ __forceinline__ void area_cross(const ElemGeo<T>& g, int, int, int, const Pos<T>& P, T L, T& n0, T& n1,
-                                           T& n2) {
-  T dx[3], dy[3];
+__device__ __forceinline__ void area_cross(const ElemGeo<double>& g, const Pos<double>& P, double L, double (&n)[3]) {
+  double dx[3], dy[3];
 #pragma unroll
   for (int m = 0; m < 3; ++m) node_rel(g, m, P, L, dx[m], dy[m]);
-  T n[3];
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     const uint32_t c = g.code >> (3 * k);
     const int pv = static_cast<int>(c & 3u);
-    const T px = pv == 0 ? dx[0] : (pv == 1 ? dx[1] : dx[2]);
-    const T py = pv == 0 ? dy[0] : (pv == 1 ? dy[1] : dy[2]);
-    const T cr = xmul(g.ex[k], py) - xmul(g.ey[k], px);
+    const double px = pv == 0 ? dx[0] : (pv == 1 ? dx[1] : dx[2]);
+    const double py = pv == 0 ? dy[0] : (pv == 1 ? dy[1] : dy[2]);
+    const double cr = xmul(g.ex[k], py) - xmul(g.ey[k], px);
     n[k] = (c & 4u) ? -cr : cr;
   }
-  n0 = n[0];
-  n1 = n[1];
-  n2 = n[2];
+}
+// FP32 form: in the order of the nodes' ids (local_order puts them back).
+__device__ __forceinline__ void area_cross(const ElemGeo<float>& g, const Pos<float>& P, float L, float (&n)[3]) {
+  float ax, ay, bx, by;
+  node_rel(g.lo, P, L, ax, ay);
+  node_rel(g.mid, P, L, bx, by);
+  n[0] = xmul(g.ex[0], by) - xmul(g.ey[0], bx);
+  n[1] = xmul(g.ex[1], ay) - xmul(g.ey[1], ax);
+  n[2] = xmul(g.ex[2], ay) - xmul(g.ey[2], ax);
+}
+__device__ __forceinline__ void local_order(const ElemGeo<double>&, double (&)[3]) {}
+__device__ __forceinline__ void local_order(const ElemGeo<float>& g, float (&n)[3]) {
+  const float v[3] = {n[0], n[1], n[2]};
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const uint32_t r = (g.code >> (2 * k)) & 3u;
+    n[k] = r == 0u ? v[0] : (r == 1u ? v[1] : v[2]);
+  }
 }
 
 // Area coordinates lambda_k = N^k / A_e (Eqs. 37-38 shapefunction values at the particle).
 template <typename T>
-__device__ __forceinline__ void area_coords(const ElemGeo<T>& g, int na, int nb, int nc, const Pos<T>& P,
-                                            T L, T& la, T& lb, T& lc) {
-  area_cross(g, na, nb, nc, P, L, la, lb, lc);
-  la *= g.inv2a;
-  lb *= g.inv2a;
-  lc *= g.inv2a;
+__device__ __forceinline__ void area_coords(const ElemGeo<T>& g, const Pos<T>& P, T L, T& la, T& lb, T& lc) {
+  T n[3];
+  area_cross(g, P, L, n);
+  local_order(g, n);
+  la = n[0] * g.inv2a;
+  lb = n[1] * g.inv2a;
+  lc = n[2] * g.inv2a;
 }
 
 // Point in the triangle with weights (1 - s) A + s (1 - t) B + s t C (Osada et al.).
@@ -362,9 +403,10 @@ __device__ __forceinline__ Pos<double> triangle_point(const ElemGeo<double>& g, 
 }
 __device__ __forceinline__ Pos<float> triangle_point(const ElemGeo<float>& g, float s, float t, float L) {
   float bx, by, cx, cy;
-  node_vec(g, 0, 1, L, bx, by);
-  node_vec(g, 0, 2, L, cx, cy);
-  Pos<float> P{g.xh[0], g.xl[0], g.yh[0], g.yl[0]};
+  const GeoNode n0 = local_node(g, 0);
+  node_vec(n0, local_node(g, 1), L, bx, by);
+  node_vec(n0, local_node(g, 2), L, cx, cy);
+  Pos<float> P{n0.xh, n0.xl, n0.yh, n0.yl};
   pos_add(P, s * (1.0f - t) * bx + s * t * cx, s * (1.0f - t) * by + s * t * cy);
   return P;
 }
