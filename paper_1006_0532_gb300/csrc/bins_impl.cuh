@@ -1857,8 +1857,17 @@ __device__ void element_warp_tile(const StatsArgs<T>& a, WarpTile<T, CAP>& t, in
   }
 }
 
+// extra: the block that only waits (sibling_enter), for a later sibling.
+template <typename T>
+void launch_sibling(void (*kernel)(const StatsArgs<T>, Place), unsigned grid, unsigned extra, unsigned block,
+                    size_t smem, cudaStream_t s, const StatsArgs<T>& a, Place at) {
+  if (at == Place::kBranch) kernel<<<grid, block, smem, s>>>(a, at);
+  else launch_chained(kernel, at == Place::kLater ? grid + extra : grid, block, smem, s, a, at);
+}
+
 template <typename T, int CAP, int WARPS, int CLS>
-__global__ void __launch_bounds__(32 * WARPS) warp_tile_kernel(const StatsArgs<T> a) {
+__global__ void __launch_bounds__(32 * WARPS) warp_tile_kernel(const StatsArgs<T> a, Place at) {
+  if (!sibling_enter(at)) return;
   extern __shared__ __align__(16) unsigned char warp_smem[];
   const int warp = threadIdx.x >> 5;
   const int b = static_cast<int>(blockIdx.x) * WARPS + warp;
@@ -1872,9 +1881,9 @@ __global__ void __launch_bounds__(32 * WARPS) warp_tile_kernel(const StatsArgs<T
 template <typename T, int CAP, int WARPS>
 constexpr int warp_tile_smem() { return static_cast<int>(sizeof(WarpTile<T, CAP>)) * WARPS; }
 template <typename T, int CAP, int WARPS, int CLS>
-void launch_warp_tile(const StatsArgs<T>& a, cudaStream_t s) {
-  warp_tile_kernel<T, CAP, WARPS, CLS>
-      <<<static_cast<unsigned>((a.ne + WARPS - 1) / WARPS), 32 * WARPS, warp_tile_smem<T, CAP, WARPS>(), s>>>(a);
+void launch_warp_tile(const StatsArgs<T>& a, Place at, cudaStream_t s) {
+  launch_sibling(warp_tile_kernel<T, CAP, WARPS, CLS>, static_cast<unsigned>((a.ne + WARPS - 1) / WARPS), 1,
+                 32 * WARPS, warp_tile_smem<T, CAP, WARPS>(), s, a, at);
 }
 
 // Residency: the FP32 bucket-rank tiles fit 10 blocks of 128 threads up to 512 particles
@@ -1882,7 +1891,8 @@ void launch_warp_tile(const StatsArgs<T>& a, cudaStream_t s) {
 // matches.
 template <typename T, int CAP, int THREADS, int CLS>
 __global__ void __launch_bounds__(THREADS, (sizeof(T) == 4 ? (THREADS == 192 ? 1344 : 1280) : 1024) / THREADS)
-    rank_tile_kernel(const StatsArgs<T> a) {
+    rank_tile_kernel(const StatsArgs<T> a, Place at) {
+  if (!sibling_enter(at)) return;
   extern __shared__ __align__(16) unsigned char rank_smem[];
   RankTile<T, CAP, THREADS>& t = *reinterpret_cast<RankTile<T, CAP, THREADS>*>(rank_smem);
   int moves = 0;
@@ -1897,7 +1907,8 @@ __global__ void __launch_bounds__(THREADS, (sizeof(T) == 4 ? (THREADS == 192 ? 1
 // 24% measured on a full class).
 template <typename T, int CAP, int THREADS, int CLS>
 __global__ void __launch_bounds__(THREADS, (sizeof(T) == 4 ? 1024 : 768) / THREADS)
-    rank_list_kernel(const StatsArgs<T> a) {
+    rank_list_kernel(const StatsArgs<T> a, Place at) {
+  sibling_start(at);
   static_assert(CLS != 0, "the class of the step counter takes a block per entry");
   extern __shared__ __align__(16) unsigned char rank_smem[];
   RankTile<T, CAP, THREADS>& t = *reinterpret_cast<RankTile<T, CAP, THREADS>*>(rank_smem);
@@ -1912,20 +1923,23 @@ __global__ void __launch_bounds__(THREADS, (sizeof(T) == 4 ? 1024 : 768) / THREA
       __syncthreads();   // done with the shared memory
     }
   }
+  sibling_leave(at);
 }
 // few: 0, or the blocks of the list kernel.
 template <typename T, int CAP, int THREADS, int CLS>
-void launch_rank_tile(const StatsArgs<T>& a, int few, cudaStream_t s) {
+void launch_rank_tile(const StatsArgs<T>& a, int few, Place at, cudaStream_t s) {
   constexpr int smem = static_cast<int>(sizeof(RankTile<T, CAP, THREADS>));
-  if (few > 0 && few < a.ne) rank_list_kernel<T, CAP, THREADS, CLS><<<static_cast<unsigned>(few), THREADS, smem, s>>>(a);
-  else rank_tile_kernel<T, CAP, THREADS, CLS><<<static_cast<unsigned>(a.ne), THREADS, smem, s>>>(a);
+  const bool list = few > 0 && few < a.ne;
+  launch_sibling(list ? rank_list_kernel<T, CAP, THREADS, CLS> : rank_tile_kernel<T, CAP, THREADS, CLS>,
+                 static_cast<unsigned>(list ? few : a.ne), list ? 0 : 1, THREADS, smem, s, a, at);
 }
 
 // The plan's large-element lists (every instance's), entries of up to kTileBig particles, on
 // the bucket-rank tile of kTileBig: a few blocks per SM, each over entries gridDim.x apart;
 // stats_big_kernel takes the larger ones.
 template <typename T>
-__global__ void __launch_bounds__(256, (sizeof(T) == 4 ? 1280 : 1024) / 256) rank_big_kernel(const StatsArgs<T> a) {
+__global__ void __launch_bounds__(256, (sizeof(T) == 4 ? 1280 : 1024) / 256) rank_big_kernel(const StatsArgs<T> a, Place at) {
+  sibling_start(at);
   extern __shared__ __align__(16) unsigned char rank_smem[];
   RankTile<T, kTileBig, 256>& t = *reinterpret_cast<RankTile<T, kTileBig, 256>*>(rank_smem);
   bool used = false;
@@ -1943,6 +1957,7 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 ? 1280 : 1024) / 256) ran
       element_rank_tile<T, kTileBig, 256>(a, t, e, N, moves);
     }
   }
+  sibling_leave(at);
 }
 
 // Every element of a small grid in one launch, a block per element on the bucket-rank tile of
@@ -1968,7 +1983,8 @@ template <typename T> bool rank_configured[kMaxDevices];
 // threads resident per SM in the FP32 form, 1024 in the FP64 form.
 template <typename T, int CAP, int THREADS, int CLS, bool FOX>
 __global__ void __launch_bounds__(THREADS, (sizeof(T) == 4 ? 1536 : 1024) / THREADS)
-    stats_tile_kernel(const StatsArgs<T> a) {
+    stats_tile_kernel(const StatsArgs<T> a, Place at) {
+  if (!sibling_enter(at)) return;
   __shared__ Tile<T, CAP, FOX> t;
   int moves = 0;
   const int e = tile_element<CLS>(a, blockIdx.x, moves);
@@ -2020,28 +2036,30 @@ void launch_stats_tiles_impl(const StatsArgs<T>& a, int num_sms, cudaStream_t s_
   // class (groups of at most 32 positions are sorted by one warp in registers; the largest
   // class in a tile of 1,024).
   const unsigned grid = static_cast<unsigned>(a.ne);
+  const bool one = s_small == s_mid && s_large == s_mid;
+  const Place first = one ? Place::kFirst : Place::kBranch, later = one ? Place::kLater : Place::kBranch;
   if (a.cond_mode == 1) {
-    stats_tile_kernel<T, 1024, 256, 1, true><<<grid, 256, 0, s_large>>>(a);
-    stats_tile_kernel<T, 256, 128, 0, true><<<grid, 128, 0, s_small>>>(a);
-    stats_tile_kernel<T, 512, 128, 2, true><<<grid, 128, 0, s_mid>>>(a);
+    launch_sibling(stats_tile_kernel<T, 1024, 256, 1, true>, grid, 1, 256, 0, s_large, a, first);
+    launch_sibling(stats_tile_kernel<T, 512, 128, 2, true>, grid, 1, 128, 0, s_mid, a, later);
+    launch_sibling(stats_tile_kernel<T, 256, 128, 0, true>, grid, 1, 128, 0, s_small, a, later);
   } else {
     configure_tiles<T>();
     // the classes above the mean count by a factor of two and more hold few elements: over
     // their lists where blocks that return would take 10 us and more (0.5 ns each)
     const int64_t mean = a.np / a.ne;
     const int few = a.ne >= 20000 ? 8 * (num_sms > 0 ? num_sms : 1) : 0;
-    launch_rank_tile<T, 768, 192, 1>(a, mean <= 256 ? few : 0, s_large);
+    launch_rank_tile<T, 768, 192, 1>(a, mean <= 256 ? few : 0, first, s_large);
     // 769..1024 from the large-element list: 4 blocks per SM
-    rank_big_kernel<T><<<static_cast<unsigned>(4 * (num_sms > 0 ? num_sms : 1)), 256,
-                         sizeof(RankTile<T, kTileBig, 256>), s_large>>>(a);
-    launch_warp_tile<T, 256, 4, 0>(a, s_small);
+    launch_sibling(rank_big_kernel<T>, 4 * (num_sms > 0 ? num_sms : 1), 0, 256, sizeof(RankTile<T, kTileBig, 256>),
+                   s_large, a, later);
+    launch_warp_tile<T, 256, 4, 0>(a, later, s_small);
     // 257..512: a block per element with bucket levels in the FP32 form; where the moment sums
     // are FP64 a warp per element, whose register sort leaves the FP64 pipe the shorter wait
     // (8,100 elements of 300 and 500 particles: FP64 form 350 and 530 us -> 292 and 408, FP64
     // accumulation 326 and 464 -> 244 and 363; FP32 form 216 -> 359 us for 12,100 of 350, its
     // 15 resident warps too few)
-    if (mean > 128 && (sizeof(T) == 8 || a.acc64)) launch_warp_tile<T, 512, 2, 2>(a, s_mid);
-    else launch_rank_tile<T, 512, 128, 2>(a, mean <= 128 ? few : 0, s_mid);
+    if (mean > 128 && (sizeof(T) == 8 || a.acc64)) launch_warp_tile<T, 512, 2, 2>(a, later, s_mid);
+    else launch_rank_tile<T, 512, 128, 2>(a, mean <= 128 ? few : 0, later, s_mid);
   }
 }
 

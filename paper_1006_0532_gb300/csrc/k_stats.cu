@@ -858,9 +858,8 @@ __device__ void process_element(const StatsArgs<T>& a, int e, int N, int cap, un
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kStatsThreads) stats_big_kernel(const StatsArgs<T> a) {
-  chain_wait();
-  chain_go();
+__global__ void __launch_bounds__(kStatsThreads) stats_big_kernel(const StatsArgs<T> a, Place at) {
+  sibling_start(at);
   extern __shared__ __align__(16) unsigned char raw[];
   for (int inst = 0; inst < a.K; ++inst) {
   const int32_t* sc = a.scal + 16 * inst;
@@ -881,6 +880,7 @@ __global__ void __launch_bounds__(kStatsThreads) stats_big_kernel(const StatsArg
     process_element(a, e, N, kBigCap, raw, moves);
   }
   }
+  sibling_leave(at);
 }
 
 template <typename T>
@@ -972,6 +972,13 @@ void launch_redistribute(Particles<T> p, Plan& pl, int K, const InstDev<T>* inst
   launch_chained(commit_moves_kernel<T>, grid, 256, 0, s, p, pl, K, np, ne, diag, err);
 }
 
+// Below this many elements the statistics' classes are siblings on one stream, above it branches
+// (four times as many with Fox's projection, whose classes take longer).  us per step, branches /
+// siblings, FP32: 900 elements of 40 particles 42 / 37, of 100 48 / 40; 2,500: 50 / 46, 59 / 56;
+// 4,900: 64 / 64, 83 / 83; 8,100: 80 / 83, 108 / 111; 12,100: 94 / 106, 138 / 150.  Fox, 12,100:
+// 154 / 153, 216 / 208; 20,000: 240 / 242, 362 / 347.  A redistributing step of 1,536 elements of
+// 200: 171 / 147.
+constexpr int kForkElements = 6144;
 // Returns the kernels launched.
 template <typename T>
 int launch_stats(const StatsArgs<T>& a, int num_sms, cudaStream_t s, const SideStreams* side) {
@@ -983,27 +990,26 @@ int launch_stats(const StatsArgs<T>& a, int num_sms, cudaStream_t s, const SideS
   }
   // a small grid: one launch for every element up to kTileBig, no branches
   if (a.cond_mode != 1 && launch_stats_small<T>(a, num_sms, s)) {
-    launch_chained(stats_big_kernel<T>, num_sms > 0 ? num_sms : 1, kStatsThreads, big, s, a);
+    launch_chained(stats_big_kernel<T>, num_sms > 0 ? num_sms : 1, kStatsThreads, big, s, a, Place::kLater);
     return 2;
   }
-  // The tile classes and the large-element kernel take disjoint elements and write disjoint
-  // outputs: with the context's side streams they run as parallel branches (the 513..768
-  // class and the large-element list's 769..1024 on side[0]; the class of up to 256 and the
-  // large-element kernel on side[1]; the
-  // 257..512 class on s), so that each one's last wave, and its blocks of other classes,
-  // which return at once, overlap the others' work; s then waits for both branches.
-  const bool fork = side && side->ok;
-  cudaStream_t s_large = s, s_small = s;
-  if (fork) {
+  // The tile classes and the large-element kernels take disjoint elements and write disjoint
+  // outputs, so that each one's last wave, and its blocks of other classes, which return at
+  // once, can overlap the others' work.  On a large grid they run as parallel branches on the
+  // context's side streams (the 513..768 class and the large-element list's 769..1024 on
+  // side[0]; the class of up to 256 and the large-element kernel on side[1]; the 257..512
+  // class on s) and s then waits for both; below kForkElements they are siblings on s.
+  if (!side || !side->ok || a.ne < (a.cond_mode == 1 ? 4 : 1) * kForkElements) {
+    launch_stats_tiles<T>(a, num_sms, s, s, s);
+    launch_chained(stats_big_kernel<T>, num_sms > 0 ? num_sms : 1, kStatsThreads, big, s, a,
+                   a.ne > 0 ? Place::kLater : Place::kFirst);
+  } else {
     cudaEventRecord(side->ev[0], s);
     cudaStreamWaitEvent(side->side[0], side->ev[0], 0);
     cudaStreamWaitEvent(side->side[1], side->ev[0], 0);
-    s_large = side->side[0];
-    s_small = side->side[1];
-  }
-  launch_stats_tiles<T>(a, num_sms, s_small, s, s_large);
-  stats_big_kernel<T><<<static_cast<unsigned>(num_sms > 0 ? num_sms : 1), kStatsThreads, big, s_small>>>(a);
-  if (fork) {
+    launch_stats_tiles<T>(a, num_sms, side->side[1], s, side->side[0]);
+    stats_big_kernel<T><<<static_cast<unsigned>(num_sms > 0 ? num_sms : 1), kStatsThreads, big, side->side[1]>>>(
+        a, Place::kBranch);
     cudaEventRecord(side->ev[1], side->side[0]);
     cudaEventRecord(side->ev[2], side->side[1]);
     cudaStreamWaitEvent(s, side->ev[1], 0);

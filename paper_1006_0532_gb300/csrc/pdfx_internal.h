@@ -233,9 +233,9 @@ constexpr int kRedBlocks = 256;                  // blocks of the solvers' reduc
 constexpr int kPcgActive = eops::S_ACTIVE;
 constexpr int kPcgIters = eops::S_ITERS;
 
-// Two streams and three events for the statistics tiles' size classes, which are independent
-// (disjoint elements and outputs) and run as parallel branches of the step: fork after the
-// lists, join before the large-element kernel.  Captured into a graph they become parallel
+// Two streams and three events for the statistics tiles' size classes on a large grid, which are
+// independent (disjoint elements and outputs) and run as parallel branches of the step: fork
+// after the lists, join before the nodal averages.  Captured into a graph they become parallel
 // nodes.  Created with the context, outside any capture; ok is false when creation failed
 // (the classes then run one after another on the caller's stream).
 struct SideStreams {
@@ -369,6 +369,29 @@ inline bool first_use_on_device(bool (&flags)[kMaxDevices]) {
 // gains nothing and loses nothing.
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// Siblings: kernels launched one after another that need what ran before the first of them and
+// nothing of one another's.  The first waits as above and only then lets the next start; a
+// later one starts when every block of its predecessor has, so after the first one's wait, and
+// need not wait for its input.  One of its blocks waits before it ends, so that a kernel's end
+// still implies that of everything launched before it: a block more that does only that
+// (sibling_enter, which then tells it to return), or, in a kernel whose blocks share a list,
+// the last one after its part (sibling_leave).  kBranch: none of this (an ordinary launch in a
+// branch of its own).
+enum class Place : int { kBranch, kFirst, kLater };
+__device__ __forceinline__ void sibling_start(Place at) {
+  if (at == Place::kBranch) return;
+  if (at == Place::kFirst) chain_wait();
+  chain_go();
+}
+__device__ __forceinline__ bool sibling_enter(Place at) {
+  sibling_start(at);
+  if (at != Place::kLater || blockIdx.x != gridDim.x - 1) return true;
+  chain_wait();
+  return false;
+}
+__device__ __forceinline__ void sibling_leave(Place at) {
+  if (at == Place::kLater && blockIdx.x == gridDim.x - 1) chain_wait();
+}
 
 template <typename... P, typename... A>
 void launch_chained(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, A... args) {
@@ -409,11 +432,12 @@ void launch_redistribute(Particles<T> p, Plan& pl, int K, const InstDev<T>* inst
                          int num_sms, unsigned long long* diag, int* err, cudaStream_t s);
 template <typename T>
 int launch_stats(const StatsArgs<T>& a, int num_sms, cudaStream_t s, const SideStreams* side);   // kernels launched
-// The tile classes of up to 256, 257..512 and 513..768 particles on s_small, s_mid and
-// s_large (k_bins_f32.cu / k_bins_f64.cu).
 // The hierarchical bins of a small grid in one launch (elements of up to kTileBig particles).
 template <typename T>
 bool launch_stats_small(const StatsArgs<T>& a, int num_sms, cudaStream_t s);   // false: not a small grid
+// The tile classes of up to 256, 257..512 and 513..1024 particles: on s_small, s_mid and s_large,
+// or, these being one stream, the first chained to the kernel before it and the others its
+// siblings (k_bins_f32.cu / k_bins_f64.cu).
 template <typename T>
 void launch_stats_tiles(const StatsArgs<T>& a, int num_sms, cudaStream_t s_small, cudaStream_t s_mid,
                         cudaStream_t s_large);
