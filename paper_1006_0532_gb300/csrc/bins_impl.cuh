@@ -270,21 +270,9 @@ struct ProjSrc {
   const T* c[3];
 };
 
-// Members only Fox's projection uses: an empty base of the hierarchical kernels' tile.
-template <typename T, bool FOX>
-struct TileFox {};
-template <typename T>
-struct TileFox<T, true> {
-  double mhx[3], mlx[3];            // sums of d_a d_phi (value/error pairs), Eq. 66
-  double em[kNS];                   // the element's statistics
-  double fox[6];                    // projection factors f_a and means <U_a> (Eqs. 64-66)
-  ProjSrc<T> proj;                  // the projected velocity's source
-};
-
-// Shared tile of one element.  Chunk tables are needed only when groups exceed 32
-// positions: then there are fewer than CAP/32 groups and fewer than 2 CAP/32 chunks.
-template <typename T, int CAP, bool FOX>
-struct Tile : TileFox<T, FOX> {
+// Shared tile of one element (Fox's projection).
+template <typename T, int CAP>
+struct Tile {
   static constexpr int kChunks = 2 * CAP / 32;
   int32_t ord[CAP];                 // particle slots in the current order
   int32_t nord[CAP];                // the next level's order
@@ -293,10 +281,12 @@ struct Tile : TileFox<T, FOX> {
     KeyArr<typename KeyPolicy<T, true>::K, kChunks * 32> exact;
   } sk;
   int32_t spay[kChunks * 32];       // their slots
-  int tie[3];                       // a tie was found at level l (fast pass)
-  int32_t gfc[CAP / 32 + 1];        // first chunk of each group
-  uint8_t cg[kChunks];              // group of each chunk
+  int tie[2];                       // a tie was found at level l (fast pass)
   double mh[12], ml[12], msh[5];    // moment sums (value/error pairs) and shift values
+  double mhx[3], mlx[3];            // sums of d_a d_phi (value/error pairs), Eq. 66
+  double em[kNS];                   // the element's statistics
+  double fox[6];                    // projection factors f_a and means <U_a> (Eqs. 64-66)
+  ProjSrc<T> proj;                  // the projected velocity's source
   int n_gathered;
 };
 
@@ -316,128 +306,76 @@ __device__ __forceinline__ int run_count_below(const Arr& s, int base, int len, 
   return pos;
 }
 
-// One sorting level: the groups of the current order (Gprev groups over n positions, the
-// largest of M) are each ordered by the level's key into nxt.  With M <= 32 a group is one
-// warp sort; otherwise chunks of 32 (tables t.gfc, t.cg) are sorted first.  A key's rank
-// is its chunk rank plus its count in every other chunk of its group; with MERGE, in groups
-// above 256 positions sorted runs (32, 64, 128, ... positions of a group) are merged
-// pairwise instead (measured faster only where two whole-element levels are ranked), a key's
-// place in the merged run being its place in its own run plus its count in the partner
-// run, with the keys at their group positions in one half of sk and spay and written to
-// the other half (n <= CAP positions each), the last round into nxt.  The fast pass (EXACT
-// false) sets *tie when two real keys of a group are equal; until the first round in which
-// two equal keys meet the runs are exact, so that round's search finds the tie.  Its places
-// never leave the group or run pair, so every index stays within bounds either way.
-template <typename T, int CAP, int THREADS, bool EXACT, bool MERGE, bool FOX, typename Arr,
-          typename ValFn>
-__device__ void sort_level(const StatsArgs<T>& a, Tile<T, CAP, FOX>& t, Arr& sk, const int32_t* cur,
-                           int32_t* nxt, const ValFn& val, int n, int Gprev, int M, float invG,
-                           int* tie) {
+// One sorting level: the n positions of the current order are ordered by the level's key into
+// nxt.  Chunks of 32 are sorted first, a warp each in registers.  A key's rank is its chunk rank
+// plus its count in every other chunk; above 256 positions sorted runs (32, 64, 128, ...
+// positions) are merged pairwise instead, a key's place in the merged run being its place in
+// its own run plus its count in the partner run, with the keys at their positions in one half
+// of sk and spay and written to the other half (n <= CAP positions each), the last round into
+// nxt.  The fast pass (EXACT false) sets *tie when two real keys are equal; until the first
+// round in which two equal keys meet the runs are exact, so that round's search finds the
+// tie.  Its places never leave the run pair, so every index stays within bounds either way.
+template <typename T, int CAP, int THREADS, bool EXACT, typename Arr, typename ValFn>
+__device__ void sort_level(const StatsArgs<T>& a, Tile<T, CAP>& t, Arr& sk, const int32_t* cur, int32_t* nxt,
+                           const ValFn& val, int n, int* tie) {
   using P = KeyPolicy<T, EXACT>;
   using K = typename P::K;
   constexpr int W = THREADS / 32;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int nchunks = (n + 31) >> 5;
   bool found = false;
-  if (M <= 32) {
-    for (int c = warp; c < Gprev; c += W) {
-      const int gs = group_start(c, n, Gprev, invG), len = group_start(c + 1, n, Gprev, invG) - gs;
-      K k;
-      int32_t q = -1;
-      if (lane < len) {
-        q = cur[gs + lane];
-        k = P::make(val(q), a.p.pid, q);
-      } else {
-        pad_key(k);
-      }
-      warp_sort32(k, q, lane);
-      if (!EXACT) {
-        const K nk = kdown(k);   // every lane takes part in the shuffle
-        found |= (lane + 1 < len) && keq(k, nk);
-      }
-      if (lane < len) nxt[gs + lane] = q;
+  for (int c = warp; c < nchunks; c += W) {
+    const int len = n - 32 * c;   // lanes from len on hold padding
+    const int at = 32 * c + lane;
+    K k;
+    int32_t q = -1;
+    if (lane < len) {
+      q = cur[at];
+      k = P::make(val(q), a.p.pid, q);
+    } else {
+      pad_key(k);
     }
-  } else if (MERGE && M > 256) {
-    const int nchunks = t.gfc[Gprev];
-    for (int c = warp; c < nchunks; c += W) {
-      const int gi = t.cg[c];
-      const int gs = group_start(gi, n, Gprev, invG), ge = group_start(gi + 1, n, Gprev, invG);
-      const int cs = gs + 32 * (c - t.gfc[gi]), len = min(32, ge - cs);
-      K k;
-      int32_t q = -1;
-      if (lane < len) {
-        q = cur[cs + lane];
-        k = P::make(val(q), a.p.pid, q);
-      } else {
-        pad_key(k);
-      }
-      warp_sort32(k, q, lane);
-      if (!EXACT) {
-        const K nk = kdown(k);   // every lane takes part in the shuffle
-        found |= (lane + 1 < len) && keq(k, nk);
-      }
-      if (lane < len) {
-        sk.set(cs + lane, k);
-        t.spay[cs + lane] = q;
-      }
+    warp_sort32(k, q, lane);
+    if (!EXACT) {
+      const K nk = kdown(k);   // every lane takes part in the shuffle
+      found |= lane < 31 && (lane + 1 < len) && keq(k, nk);
     }
-    __syncthreads();
+    if (n <= 32) {
+      if (lane < len) nxt[at] = q;
+    } else {
+      sk.set(at, k);
+      t.spay[at] = q;
+    }
+  }
+  if (n > 32) __syncthreads();
+  if (n > 256) {
     int src = 0;
-    for (int lgR = 5; (1 << lgR) < M; ++lgR) {
+    for (int lgR = 5; (1 << lgR) < n; ++lgR) {
       const int R = 1 << lgR;
-      const bool last = 2 * R >= M;
+      const bool last = 2 * R >= n;
       const int dst = CAP - src;
-      for (int c = warp; c < nchunks; c += W) {
-        const int gi = t.cg[c];
-        const int gs = group_start(gi, n, Gprev, invG), ge = group_start(gi + 1, n, Gprev, invG);
-        const int li = 32 * (c - t.gfc[gi]) + lane;    // position in the group
-        if (li < ge - gs) {
-          const int m = li >> lgR, ps = (m ^ 1) << lgR;   // own run, partner run start
-          const int plen = min(R, ge - gs - ps);        // <= 0: no partner
-          const K k = sk.get(src + gs + li);
-          bool eq = false;
-          const int cnt = plen > 0 ? run_count_below<CAP / 2>(sk, src + gs + ps, plen, R, k, eq) : 0;
-          if (!EXACT) found |= eq;
-          const int np = ((m & ~1) << lgR) + (li - (m << lgR)) + cnt;
-          const int32_t q = t.spay[src + gs + li];
-          if (last) {
-            nxt[gs + np] = q;
-          } else {
-            sk.set(dst + gs + np, k);
-            t.spay[dst + gs + np] = q;
-          }
+      for (int li = threadIdx.x; li < n; li += THREADS) {
+        const int m = li >> lgR, ps = (m ^ 1) << lgR;   // own run, partner run start
+        const int plen = min(R, n - ps);                // <= 0: no partner
+        const K k = sk.get(src + li);
+        bool eq = false;
+        const int cnt = plen > 0 ? run_count_below<CAP / 2>(sk, src + ps, plen, R, k, eq) : 0;
+        if (!EXACT) found |= eq;
+        const int np = ((m & ~1) << lgR) + (li - (m << lgR)) + cnt;
+        const int32_t q = t.spay[src + li];
+        if (last) {
+          nxt[np] = q;
+        } else {
+          sk.set(dst + np, k);
+          t.spay[dst + np] = q;
         }
       }
       __syncthreads();
       src = dst;
     }
-  } else {
-    const int nchunks = t.gfc[Gprev];
+  } else if (n > 32) {
     for (int c = warp; c < nchunks; c += W) {
-      const int gi = t.cg[c];
-      const int gs = group_start(gi, n, Gprev, invG), ge = group_start(gi + 1, n, Gprev, invG);
-      const int cs = gs + 32 * (c - t.gfc[gi]), len = min(32, ge - cs);
-      K k;
-      int32_t q = -1;
-      if (lane < len) {
-        q = cur[cs + lane];
-        k = P::make(val(q), a.p.pid, q);
-      } else {
-        pad_key(k);
-      }
-      warp_sort32(k, q, lane);
-      if (!EXACT) {
-        const K nk = kdown(k);   // every lane takes part in the shuffle
-        found |= (lane + 1 < len) && keq(k, nk);
-      }
-      sk.set(c * 32 + lane, k);
-      t.spay[c * 32 + lane] = q;
-    }
-    __syncthreads();
-    for (int c = warp; c < nchunks; c += W) {
-      const int gi = t.cg[c];
-      const int gs = group_start(gi, n, Gprev, invG), ge = group_start(gi + 1, n, Gprev, invG);
-      const int c0 = t.gfc[gi], c1 = t.gfc[gi + 1];
-      const int cs = gs + 32 * (c - c0), len = min(32, ge - cs);
+      const int len = n - 32 * c;
       const K k = sk.get(c * 32 + lane);
       int r = lane;
       bool eq_any = false;
@@ -445,14 +383,14 @@ __device__ void sort_level(const StatsArgs<T>& a, Tile<T, CAP, FOX>& t, Arr& sk,
       // compiler's default unrolling grows the kernel past what its instruction cache holds
       // (2-5% slower per step).
 #pragma unroll 1
-      for (int c2 = c0; c2 < c1; ++c2) {
+      for (int c2 = 0; c2 < nchunks; ++c2) {
         if (c2 == c) continue;
         bool eq;
         r += count_below(sk, c2 * 32, k, eq);
         eq_any |= eq;
       }
       if (!EXACT) found |= eq_any && lane < len;
-      if (lane < len) nxt[gs + r] = t.spay[c * 32 + lane];
+      if (lane < len) nxt[r] = t.spay[c * 32 + lane];
     }
   }
   if (!EXACT) {
@@ -464,11 +402,6 @@ __device__ void sort_level(const StatsArgs<T>& a, Tile<T, CAP, FOX>& t, Arr& sk,
 // Key value of a particle at one level: a velocity component, or Fox's projected velocity
 // sum_a f_a (U_a - <U_a>) (Eq. 64, formed in FP64 and rounded to the state precision) from
 // the factors, means and component arrays in shared memory.
-template <typename T>
-struct ArrVal {
-  const T* v;
-  __device__ __forceinline__ T operator()(int32_t q) const { return v[q]; }
-};
 // Eq. 64's projected velocity from the factors f_a and the means m_a, summed left to right
 // with every operation rounded on its own (no fused multiply-add): in FP64 the oracle's bits.
 template <typename T>
@@ -502,56 +435,64 @@ struct ProjVal {
   }
 };
 
-// Sect. 3.3, Eqs. 35-36, by warp 0 in the order cur: sums of d = x - x_0 and of products of
-// d in precision A (each product rounded on its own, never fused into the sum, so that every
-// tile kernel forms the same sums bit for bit), x_0 the first particle of the order; mean = x_0 + S1/N, central =
-// S2/N - (S1/N)^2; lanes combine as value/error pairs (FP32) or in FP64, then the 13
-// outputs are formed in FP64, one per lane.  Inlined: as an out-of-line call it measured
-// slower (its spills and the call outweigh the spills it saves in the sorting loops).
-// FOX: also the sums of d_a d_phi, then <u_a phi'> and the factors of Eqs. 65-66.
-template <typename A, bool FOX, typename T, typename TileT, typename I>
-__device__ __forceinline__ void element_moments(const T* __restrict__ pu, const T* __restrict__ pv,
-                                                const T* __restrict__ pw, const T* __restrict__ pom,
-                                                const T* __restrict__ ppsi, double* emom_e,
-                                                int32_t* gbin_e, TileT& t,
-                                                const I* cur, int n, int g0, int g1, int g2) {
-  const int lane = threadIdx.x & 31;
-  A sh[5] = {A(0), A(0), A(0), A(0), A(0)};
+// Sect. 3.3, Eqs. 35-36 and 66 in the order cur: sums of d = x - x_0 and of products of d in
+// precision A (each product rounded on its own, never fused into the sum), x_0 the first
+// particle of the order; four warps take four (the last three) of the fifteen sums each over
+// all particles, lane l the positions l, l + 32, ...; lanes combine as value/error pairs
+// (FP32) or in FP64.  One warp with all fifteen kept the others at the barrier and took 900
+// bytes of spills (a step of 12,100 elements of 300 particles, FP32: 516 us, 432 so; 441 at 1,280
+// resident threads per SM, 463 at 1,024; 454 with six warps per element, 477 with eight).
+template <typename A, typename T, int CAP>
+__device__ __forceinline__ void fox_sums(const StatsArgs<T>& a, Tile<T, CAP>& t, const int32_t* cur, int n) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (warp >= 4) return;
+  // warp 0: d_u, d_u d_u, d_u d_v, d_u d_psi; 1: d_v, d_v d_v, d_v d_w, d_v d_psi; 2: d_w, d_w d_w,
+  // d_u d_w, d_w d_psi; 3: d_omega, d_psi, d_psi d_psi
+  const T* xa = warp == 0 ? a.p.u : warp == 1 ? a.p.v : warp == 2 ? a.p.w : a.p.om;
+  const T* xb = warp == 0 ? a.p.v : warp == 1 ? a.p.w : warp == 2 ? a.p.u : a.p.psi;
+  A sa = A(0), sb = A(0), sp = A(0);
   if (n > 0) {
     const int q0 = cur[0];
-    sh[0] = A(pu[q0]); sh[1] = A(pv[q0]); sh[2] = A(pw[q0]);
-    sh[3] = A(pom[q0]); sh[4] = A(ppsi[q0]);
+    sa = A(xa[q0]);
+    sb = A(xb[q0]);
+    sp = A(a.p.psi[q0]);
   }
-  Acc<A> m[12];
-  Acc<A> mx[3];   // FOX only
+  Acc<A> m0, m1, m2, m3;
 #pragma unroll 2
   for (int p = lane; p < n; p += 32) {
     const int q = cur[p];
-    const A du = A(pu[q]) - sh[0], dv = A(pv[q]) - sh[1], dw = A(pw[q]) - sh[2];
-    const A dom = A(pom[q]) - sh[3], dp = A(ppsi[q]) - sh[4];
-    m[0].add(du); m[1].add(dv); m[2].add(dw); m[3].add(dom); m[4].add(dp);
-    m[5].add(xmul(du, du)); m[6].add(xmul(dv, dv)); m[7].add(xmul(dw, dw));
-    m[8].add(xmul(du, dv)); m[9].add(xmul(du, dw)); m[10].add(xmul(dv, dw));
-    m[11].add(xmul(dp, dp));
-    if constexpr (FOX) { mx[0].add(xmul(du, dp)); mx[1].add(xmul(dv, dp)); mx[2].add(xmul(dw, dp)); }
-  }
-#pragma unroll
-  for (int c = 0; c < 12; ++c) {
-    A h, l;
-    m[c].warp_pair(h, l);
-    if (lane == c) { t.mh[c] = h; t.ml[c] = l; }
-  }
-  if constexpr (FOX) {
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      A h, l;
-      mx[c].warp_pair(h, l);
-      if (lane == c) { t.mhx[c] = h; t.mlx[c] = l; }
+    const A da = A(xa[q]) - sa, db = A(xb[q]) - sb;
+    m0.add(da);
+    if (warp < 3) {
+      m1.add(xmul(da, da));
+      m2.add(xmul(da, db));
+      m3.add(xmul(da, A(a.p.psi[q]) - sp));
+    } else {
+      m1.add(db);
+      m2.add(xmul(db, db));
     }
   }
-  if (lane < 5)
-    t.msh[lane] = lane == 0 ? sh[0] : lane == 1 ? sh[1] : lane == 2 ? sh[2] : lane == 3 ? sh[3] : sh[4];
-  __syncwarp();
+  const int c0 = warp, c1 = warp < 3 ? 5 + warp : 4;
+  const int c2 = warp == 0 ? 8 : warp == 1 ? 10 : warp == 2 ? 9 : 11;
+  A h[4], l[4];
+  m0.warp_pair(h[0], l[0]);
+  m1.warp_pair(h[1], l[1]);
+  m2.warp_pair(h[2], l[2]);
+  m3.warp_pair(h[3], l[3]);
+  if (lane == 0) {
+    t.mh[c0] = h[0]; t.ml[c0] = l[0];
+    t.mh[c1] = h[1]; t.ml[c1] = l[1];
+    t.mh[c2] = h[2]; t.ml[c2] = l[2];
+    t.msh[warp] = sa;
+    if (warp < 3) { t.mhx[warp] = h[3]; t.mlx[warp] = l[3]; }
+    else t.msh[4] = sb;
+  }
+}
+// The 13 outputs in FP64, one per lane of warp 0 (mean = x_0 + S1/N, central = S2/N -
+// (S1/N)^2), and the projection's factors.
+template <typename T, int CAP>
+__device__ __forceinline__ void fox_moments(const StatsArgs<T>& a, Tile<T, CAP>& t, int n, int e, const int (&g)[3]) {
+  const int lane = threadIdx.x & 31;
   if (lane < kNS) {
     const double inv = recip_n(n);
     const int ix = mom_nib(kMomX, lane), iy = mom_nib(kMomY, lane);
@@ -565,70 +506,34 @@ __device__ __forceinline__ void element_moments(const T* __restrict__ pu, const 
     }
     if (lane == 0) v = static_cast<double>(n);
     else if (n == 0) v = 0.0;
-    emom_e[lane] = v;
-    if constexpr (FOX) t.em[lane] = v;
+    a.emom[static_cast<size_t>(kNS) * e + lane] = v;
+    t.em[lane] = v;
   }
-  if (lane < 3) gbin_e[lane] = lane == 0 ? g0 : lane == 1 ? g1 : g2;
-  if constexpr (FOX) {
-    __syncwarp();
-    if (lane == 0) {
-      // <u_a phi'> = S(d_a d_phi)/N - (S d_a/N)(S d_phi/N); then Eqs. 65-66
-      const double inv = recip_n(n);
-      const double sp = (t.mh[4] + t.ml[4]) * inv;
-      double uphi[3], f[3];
-      for (int k = 0; k < 3; ++k)
-        uphi[k] = (t.mhx[k] + t.mlx[k]) * inv - (t.mh[k] + t.ml[k]) * inv * sp;
-      fox_factors(t.em, uphi, f);
-      for (int k = 0; k < 3; ++k) { t.fox[k] = f[k]; t.fox[3 + k] = t.em[1 + k]; }
-    }
+  if (lane < 3) a.gbin[3 * e + lane] = lane == 0 ? g[0] : lane == 1 ? g[1] : g[2];
+  __syncwarp();
+  if (lane == 0) {
+    // <u_a phi'> = S(d_a d_phi)/N - (S d_a/N)(S d_phi/N); then Eqs. 65-66
+    const double inv = recip_n(n);
+    const double sp = (t.mh[4] + t.ml[4]) * inv;
+    double uphi[3], f[3];
+    for (int k = 0; k < 3; ++k)
+      uphi[k] = (t.mhx[k] + t.mlx[k]) * inv - (t.mh[k] + t.ml[k]) * inv * sp;
+    fox_factors(t.em, uphi, f);
+    for (int k = 0; k < 3; ++k) { t.fox[k] = f[k]; t.fox[3 + k] = t.em[1 + k]; }
   }
+  __syncwarp();
 }
 
-// Moments in the state precision (FP32 form: compensated) or, with acc64 in the FP32
-// form, in FP64.
-template <typename T, int CAP, bool FOX>
-__device__ __forceinline__ void element_moments_of(const StatsArgs<T>& a, Tile<T, CAP, FOX>& t,
-                                                   const int32_t* cur, int n, int e,
-                                                   const int (&g)[3]) {
-  double* const emom_e = a.emom + static_cast<size_t>(kNS) * e;
-  int32_t* const gbin_e = a.gbin + 3 * e;
-  if (sizeof(T) == 4 && a.acc64)
-    element_moments<double, FOX>(a.p.u, a.p.v, a.p.w, a.p.om, a.p.psi, emom_e, gbin_e, t, cur, n,
-                                 g[0], g[1], g[2]);
-  else
-    element_moments<T, FOX>(a.p.u, a.p.v, a.p.w, a.p.om, a.p.psi, emom_e, gbin_e, t, cur, n,
-                            g[0], g[1], g[2]);
-}
-
-// Chunk tables of one level (warp 0): the first chunk of each of the Gprev groups over n
-// positions (Gprev < n / 32 <= CAP / 32 <= 32 groups, one lane each) and the group of each
-// chunk.
-template <typename T, int CAP, bool FOX>
-__device__ __forceinline__ void chunk_tables(Tile<T, CAP, FOX>& t, int n, int Gprev, float invG, int lane) {
-  int nch = 0;
-  if (lane < Gprev) nch = (group_start(lane + 1, n, Gprev, invG) - group_start(lane, n, Gprev, invG) + 31) >> 5;
-  int incl = nch;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int y = __shfl_up_sync(kFull, incl, o);
-    if (lane >= o) incl += y;
-  }
-  if (lane < Gprev) {
-    t.gfc[lane] = incl - nch;
-    for (int j = 0; j < nch; ++j) t.cg[incl - nch + j] = static_cast<uint8_t>(lane);
-  }
-  if (lane == Gprev - 1) t.gfc[Gprev] = incl;
-}
-
-// One element of N <= CAP particles (list size after redistribution) by a block of THREADS.
-template <typename T, int CAP, int THREADS, bool FOX>
-__device__ void element_tile(const StatsArgs<T>& a, Tile<T, CAP, FOX>& t, int e, int N, int moves) {
+// One element of N <= CAP particles (list size after redistribution) by a block of THREADS,
+// Fox's projection.
+template <typename T, int CAP, int THREADS>
+__device__ void element_tile(const StatsArgs<T>& a, Tile<T, CAP>& t, int e, int N, int moves) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned below = (1u << lane) - 1u;
 
   // gather: the element's list minus particles moved out, plus those moved in
   if (threadIdx.x == 0) t.n_gathered = 0;
-  if (threadIdx.x < 3) t.tie[threadIdx.x] = 0;
+  if (threadIdx.x < 2) t.tie[threadIdx.x] = 0;
   __syncthreads();
   {
     const int32_t o = a.off[e], c = a.cnt[e];
@@ -675,91 +580,45 @@ __device__ void element_tile(const StatsArgs<T>& a, Tile<T, CAP, FOX>& t, int e,
   if (n != N && threadIdx.x == 0) atomicCAS(a.err, 0, PDFX_ERR_CAPACITY);
   n = min(min(n, N), CAP);
 
-  // effective bins (reading of Sect. 3.5): g_l = max(1, min(b_l, n / (g_1..g_{l-1} min_per_bin)));
   // Fox's projection: max(1, min(fox_bins, n / min_per_bin)) intervals
-  int g[3];
-  if constexpr (FOX) {
-    int nc = n / a.min_per_bin;
-    if (a.fox_bins < nc) nc = a.fox_bins;
-    g[0] = nc < 1 ? 1 : nc;
-    g[1] = g[2] = 1;
-  } else {
-    int Gp = 1;
-#pragma unroll
-    for (int l = 0; l < 3; ++l) {
-      const int capl = n / (Gp * a.min_per_bin);
-      int gl = a.bins[l] < capl ? a.bins[l] : capl;
-      if (gl < 1) gl = 1;
-      g[l] = gl;
-      Gp *= gl;
-    }
-  }
+  int nc = n / a.min_per_bin;
+  if (a.fox_bins < nc) nc = a.fox_bins;
+  const int g[3] = {nc < 1 ? 1 : nc, 1, 1};
 
   int32_t* cur = t.ord;
   int32_t* nxt = t.nord;
-  if constexpr (!FOX) {
-    // levels by (u, id), (v, id), (w, id) within the groups of the previous level
-    int Gprev = 1;
-    if (n > 0) {
-#pragma unroll 1
-      for (int l = 0; l < 3; ++l) {
-        if (l > 0 && g[l] <= 1) continue;
-        const ArrVal<T> val{l == 0 ? a.p.u : (l == 1 ? a.p.v : a.p.w)};
-        const int M = (n + Gprev - 1) / Gprev;   // largest group
-        const float invG = 1.0f / static_cast<float>(Gprev);
-        if (M > 32 && warp == 0) chunk_tables(t, n, Gprev, invG, lane);
-        __syncthreads();
-        sort_level<T, CAP, THREADS, false, false>(a, t, t.sk.fast, cur, nxt, val, n, Gprev, M, invG,
-                                                  &t.tie[l]);
-        __syncthreads();
-        if (t.tie[l]) {
-          sort_level<T, CAP, THREADS, true, false>(a, t, t.sk.exact, cur, nxt, val, n, Gprev, M,
-                                                   invG, nullptr);
-          __syncthreads();
-        }
-        int32_t* tmp = cur;
-        cur = nxt;
-        nxt = tmp;
-        Gprev *= g[l];
-      }
+  // Fox's projection (Eqs. 64-66): the particle-id order fixes the order of the moment
+  // sums; the moments give the factors; then one level over the whole element by U_rho
+  auto whole_level = [&](const auto& val, int ti) {
+    sort_level<T, CAP, THREADS, false>(a, t, t.sk.fast, cur, nxt, val, n, &t.tie[ti]);
+    __syncthreads();
+    if (t.tie[ti]) {
+      sort_level<T, CAP, THREADS, true>(a, t, t.sk.exact, cur, nxt, val, n, nullptr);
+      __syncthreads();
     }
-    // moments (warp 0) in the final order
-    if (warp == 0) element_moments_of(a, t, cur, n, e, g);
-  } else {
-    // Fox's projection (Eqs. 64-66): the particle-id order fixes the order of the moment
-    // sums; the moments give the factors; then one level over the whole element by U_rho
-    auto whole_level = [&](const auto& val, int ti) {
-      const float invG = 1.0f;
-      if (n > 32 && warp == 0) chunk_tables(t, n, 1, invG, lane);
-      __syncthreads();
-      sort_level<T, CAP, THREADS, false, true>(a, t, t.sk.fast, cur, nxt, val, n, 1, n, invG,
-                                               &t.tie[ti]);
-      __syncthreads();
-      if (t.tie[ti]) {
-        sort_level<T, CAP, THREADS, true, true>(a, t, t.sk.exact, cur, nxt, val, n, 1, n, invG,
-                                                nullptr);
-        __syncthreads();
-      }
-      int32_t* tmp = cur;
-      cur = nxt;
-      nxt = tmp;
-    };
-    if (n > 0) whole_level(PidVal<T>{a.p.pid}, 0);
-    if (warp == 0) element_moments_of(a, t, cur, n, e, g);   // an empty element writes zeros
-    if (n > 0) {
-      if (threadIdx.x < 3) {
-        const int k = threadIdx.x;
-        t.proj.f[k] = t.fox[k];
-        t.proj.m[k] = t.fox[3 + k];
-        t.proj.c[k] = k == 0 ? a.p.u : (k == 1 ? a.p.v : a.p.w);
-      }
-      __syncthreads();
-      // all factors zero (a constant scalar, or a degenerate correlation system): every
-      // U_rho is 0 and the order of (U_rho, id) is the id order the element already has
-      if (!(t.fox[0] == 0.0 && t.fox[1] == 0.0 && t.fox[2] == 0.0)) whole_level(ProjVal<T>{&t.proj}, 1);
+    int32_t* tmp = cur;
+    cur = nxt;
+    nxt = tmp;
+  };
+  if (n > 0) whole_level(PidVal<T>{a.p.pid}, 0);
+  // moments (an empty element writes zeros)
+  if (sizeof(T) == 4 && a.acc64) fox_sums<double>(a, t, cur, n);
+  else fox_sums<T>(a, t, cur, n);
+  __syncthreads();
+  if (warp == 0) fox_moments(a, t, n, e, g);
+  if (n > 0) {
+    if (threadIdx.x < 3) {
+      const int k = threadIdx.x;
+      t.proj.f[k] = t.fox[k];
+      t.proj.m[k] = t.fox[3 + k];
+      t.proj.c[k] = k == 0 ? a.p.u : (k == 1 ? a.p.v : a.p.w);
     }
+    __syncthreads();
+    // all factors zero (a constant scalar, or a degenerate correlation system): every
+    // U_rho is 0 and the order of (U_rho, id) is the id order the element already has
+    if (!(t.fox[0] == 0.0 && t.fox[1] == 0.0 && t.fox[2] == 0.0)) whole_level(ProjVal<T>{&t.proj}, 1);
   }
-  const int G = g[0] * g[1] * g[2];
+  const int G = g[0];
 
   // Appendix A bins: conditional scalar means over the final order's bins
   double* vc = a.vcce + static_cast<size_t>(a.G) * e;
@@ -1217,7 +1076,7 @@ __device__ void order_level(RankTile<T, CAP, THREADS>& t, const T* key, int n, i
 // 5..11: uu, vv, ww, uv, uw, vw, psi psi (products of d; x_0 the first particle of the
 // order).  Warp w < 4 takes three of the twelve sums over all particles, lane l the
 // positions l, l + 32, ... (compensated FP32 per lane, or FP64; products rounded on their
-// own as in element_moments, whose sums these equal bit for bit); the lanes then combine by
+// own as in fox_sums, whose sums these equal bit for bit); the lanes then combine by
 // a shuffle tree in a fixed order (value/error pairs in FP32).  Called by every thread.
 template <typename A, typename T, int CAP, int THREADS>
 __device__ __forceinline__ void rank_moments(RankTile<T, CAP, THREADS>& t, int n) {
@@ -1981,16 +1840,16 @@ template <typename T> bool rank_configured[kMaxDevices];
 // One block per entry of one size class of the plan's tile lists (tile_element); the grid
 // covers every element and blocks past the class count return.  The register cap keeps 1536
 // threads resident per SM in the FP32 form, 1024 in the FP64 form.
-template <typename T, int CAP, int THREADS, int CLS, bool FOX>
+template <typename T, int CAP, int THREADS, int CLS>
 __global__ void __launch_bounds__(THREADS, (sizeof(T) == 4 ? 1536 : 1024) / THREADS)
     stats_tile_kernel(const StatsArgs<T> a, Place at) {
   if (!sibling_enter(at)) return;
-  __shared__ Tile<T, CAP, FOX> t;
+  __shared__ Tile<T, CAP> t;
   int moves = 0;
   const int e = tile_element<CLS>(a, blockIdx.x, moves);
   if (e < 0) return;
   const int N = moves ? a.fin[e] : a.cnt[e];
-  element_tile<T, CAP, THREADS, FOX>(a, t, e, min(N, CAP), moves);
+  element_tile<T, CAP, THREADS>(a, t, e, min(N, CAP), moves);
 }
 
 }  // namespace
@@ -2039,9 +1898,9 @@ void launch_stats_tiles_impl(const StatsArgs<T>& a, int num_sms, cudaStream_t s_
   const bool one = s_small == s_mid && s_large == s_mid;
   const Place first = one ? Place::kFirst : Place::kBranch, later = one ? Place::kLater : Place::kBranch;
   if (a.cond_mode == 1) {
-    launch_sibling(stats_tile_kernel<T, 1024, 256, 1, true>, grid, 1, 256, 0, s_large, a, first);
-    launch_sibling(stats_tile_kernel<T, 512, 128, 2, true>, grid, 1, 128, 0, s_mid, a, later);
-    launch_sibling(stats_tile_kernel<T, 256, 128, 0, true>, grid, 1, 128, 0, s_small, a, later);
+    launch_sibling(stats_tile_kernel<T, 1024, 256, 1>, grid, 1, 256, 0, s_large, a, first);
+    launch_sibling(stats_tile_kernel<T, 512, 128, 2>, grid, 1, 128, 0, s_mid, a, later);
+    launch_sibling(stats_tile_kernel<T, 256, 128, 0>, grid, 1, 128, 0, s_small, a, later);
   } else {
     configure_tiles<T>();
     // the classes above the mean count by a factor of two and more hold few elements: over
