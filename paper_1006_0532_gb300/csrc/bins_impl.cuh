@@ -406,9 +406,9 @@ __device__ void sort_level(const StatsArgs<T>& a, Tile<T, CAP>& t, Arr& sk, cons
 // with every operation rounded on its own (no fused multiply-add): in FP64 the oracle's bits.
 template <typename T>
 __device__ __forceinline__ T fox_key(const double* f, const double* m, T u, T v, T w) {
-  const double a = __dmul_rn(f[0], __dsub_rn(static_cast<double>(u), m[0]));
-  const double b = __dmul_rn(f[1], __dsub_rn(static_cast<double>(v), m[1]));
-  const double c = __dmul_rn(f[2], __dsub_rn(static_cast<double>(w), m[2]));
+  const double a = __dmul_rn(f[0], __dsub_rn(m64::widened(u), m[0]));
+  const double b = __dmul_rn(f[1], __dsub_rn(m64::widened(v), m[1]));
+  const double c = __dmul_rn(f[2], __dsub_rn(m64::widened(w), m[2]));
   return static_cast<T>(__dadd_rn(__dadd_rn(a, b), c));
 }
 // The sort value of a particle id: a positive normal number whose bits are 2^23 (FP32) or
@@ -435,13 +435,50 @@ struct ProjVal {
   }
 };
 
+// One level of the moment sums' tree over the lanes, N sums in and N / 2 (rounded up) out: a
+// lane sends its partner (lane ^ o) the half it gives up and joins the other half's value of
+// both, the lower lane's first, as Acc::warp_pair does for one sum in every lane.
+template <int N, typename A, int S>
+__device__ __forceinline__ void pair_level(A (&h)[S], A (&l)[S], int o, int lane) {
+  constexpr int H = (N + 1) / 2;
+  const bool low = (lane & o) == 0;
+#pragma unroll
+  for (int s = 0; s < H; ++s) {
+    const int t = N > 1 ? (s + H < N ? s + H : N - 1) : 0;   // the upper half's sum at this place
+    const A mh = low ? h[s] : h[t], ml = low ? l[s] : l[t];
+    const A gh = low ? h[t] : h[s], gl = low ? l[t] : l[s];
+    const A oh = __shfl_xor_sync(kFull, gh, o);
+    const A ah = low ? mh : oh, bh = low ? oh : mh;
+    if (sizeof(A) == 4) {
+      const A ol = __shfl_xor_sync(kFull, gl, o);
+      const A al = low ? ml : ol, bl = low ? ol : ml;
+      const A sh = ah + bh;
+      const A bb = sh - ah;
+      const A se = (ah - (sh - bb)) + (bh - bb);
+      const A lw = se + (al + bl);
+      h[s] = sh + lw;
+      l[s] = lw - (h[s] - sh);
+    } else {
+      h[s] = ah + bh;
+    }
+  }
+}
+
 // Sect. 3.3, Eqs. 35-36 and 66 in the order cur: sums of d = x - x_0 and of products of d in
 // precision A (each product rounded on its own, never fused into the sum), x_0 the first
 // particle of the order; four warps take four (the last three) of the fifteen sums each over
 // all particles, lane l the positions l, l + 32, ...; lanes combine as value/error pairs
 // (FP32) or in FP64.  One warp with all fifteen kept the others at the barrier and took 900
 // bytes of spills (a step of 12,100 elements of 300 particles, FP32: 516 us, 432 so; 441 at 1,280
-// resident threads per SM, 463 at 1,024; 454 with six warps per element, 477 with eight).
+// resident threads per SM, 463 at 1,024; 454 with six warps per element, 477 with eight).  With
+// FP64 accumulation the FP64 pipe is the limit, and every operation on it counts: the lanes
+// combine by halves (24 additions an element instead of 80) and the values widen by their bits
+// (11 conversions a row saved): 760 us, as with one warp; 811 with neither kept.
+template <typename A, typename T>
+__device__ __forceinline__ A as_acc(T x) {   // exact
+  if constexpr (sizeof(A) == 8) return m64::widened(x);
+  else return x;
+}
 template <typename A, typename T, int CAP>
 __device__ __forceinline__ void fox_sums(const StatsArgs<T>& a, Tile<T, CAP>& t, const int32_t* cur, int n) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -461,31 +498,37 @@ __device__ __forceinline__ void fox_sums(const StatsArgs<T>& a, Tile<T, CAP>& t,
 #pragma unroll 2
   for (int p = lane; p < n; p += 32) {
     const int q = cur[p];
-    const A da = A(xa[q]) - sa, db = A(xb[q]) - sb;
+    const A da = as_acc<A>(xa[q]) - sa, db = as_acc<A>(xb[q]) - sb;
     m0.add(da);
     if (warp < 3) {
       m1.add(xmul(da, da));
       m2.add(xmul(da, db));
-      m3.add(xmul(da, A(a.p.psi[q]) - sp));
+      m3.add(xmul(da, as_acc<A>(a.p.psi[q]) - sp));
     } else {
       m1.add(db);
       m2.add(xmul(db, db));
     }
   }
-  const int c0 = warp, c1 = warp < 3 ? 5 + warp : 4;
-  const int c2 = warp == 0 ? 8 : warp == 1 ? 10 : warp == 2 ? 9 : 11;
-  A h[4], l[4];
-  m0.warp_pair(h[0], l[0]);
-  m1.warp_pair(h[1], l[1]);
-  m2.warp_pair(h[2], l[2]);
-  m3.warp_pair(h[3], l[3]);
+  A h[4] = {m0.s, m1.s, m2.s, m3.s};
+  A l[4] = {-Acc<A>::err(m0), -Acc<A>::err(m1), -Acc<A>::err(m2), -Acc<A>::err(m3)};
+  pair_level<4>(h, l, 16, lane);
+  pair_level<2>(h, l, 8, lane);
+  pair_level<1>(h, l, 4, lane);
+  pair_level<1>(h, l, 2, lane);
+  pair_level<1>(h, l, 1, lane);
+  // lanes 0, 8, 16 and 24 hold the four sums
+  if ((lane & 7) == 0) {
+    const int k = lane >> 3;
+    const int c = k == 0   ? warp
+                  : k == 1 ? (warp < 3 ? 5 + warp : 4)
+                           : (warp == 0 ? 8 : warp == 1 ? 10 : warp == 2 ? 9 : 11);
+    const A lo = sizeof(A) == 4 ? l[0] : A(0);
+    if (k < 3) { t.mh[c] = h[0]; t.ml[c] = lo; }
+    else if (warp < 3) { t.mhx[warp] = h[0]; t.mlx[warp] = lo; }
+  }
   if (lane == 0) {
-    t.mh[c0] = h[0]; t.ml[c0] = l[0];
-    t.mh[c1] = h[1]; t.ml[c1] = l[1];
-    t.mh[c2] = h[2]; t.ml[c2] = l[2];
     t.msh[warp] = sa;
-    if (warp < 3) { t.mhx[warp] = h[3]; t.mlx[warp] = l[3]; }
-    else t.msh[4] = sb;
+    if (warp == 3) t.msh[4] = sb;
   }
 }
 // The 13 outputs in FP64, one per lane of warp 0 (mean = x_0 + S1/N, central = S2/N -
@@ -1537,35 +1580,6 @@ __device__ __forceinline__ void warp_levels(WarpTile<T, CAP>& t, int n, const in
     }
     __syncwarp();
     Gprev *= g[l];
-  }
-}
-
-// One level of the moment sums' tree over the lanes, N sums in and N / 2 (rounded up) out: a
-// lane sends its partner (lane ^ o) the half it gives up and joins the other half's value of
-// both, the lower lane's first, as Acc::warp_pair does for one sum in every lane.
-template <int N, typename A>
-__device__ __forceinline__ void pair_level(A (&h)[12], A (&l)[12], int o, int lane) {
-  constexpr int H = (N + 1) / 2;
-  const bool low = (lane & o) == 0;
-#pragma unroll
-  for (int s = 0; s < H; ++s) {
-    const int t = N > 1 ? (s + H < N ? s + H : N - 1) : 0;   // the upper half's sum at this place
-    const A mh = low ? h[s] : h[t], ml = low ? l[s] : l[t];
-    const A gh = low ? h[t] : h[s], gl = low ? l[t] : l[s];
-    const A oh = __shfl_xor_sync(kFull, gh, o);
-    const A ah = low ? mh : oh, bh = low ? oh : mh;
-    if (sizeof(A) == 4) {
-      const A ol = __shfl_xor_sync(kFull, gl, o);
-      const A al = low ? ml : ol, bl = low ? ol : ml;
-      const A sh = ah + bh;
-      const A bb = sh - ah;
-      const A se = (ah - (sh - bb)) + (bh - bb);
-      const A lw = se + (al + bl);
-      h[s] = sh + lw;
-      l[s] = lw - (h[s] - sh);
-    } else {
-      h[s] = ah + bh;
-    }
   }
 }
 

@@ -197,6 +197,18 @@ PDFX_M64 double rcbrt(double x) {
   return fma(fma(e, 2.0 / 9.0, 1.0 / 3.0) * e, z, z);
 }
 
+// Any FP32 number as FP64 by its bits (the conversion takes the FP64 pipe like any other FP64
+// operation): the exponent is re-biased; zero keeps its sign; subnormal, infinite and NaN go
+// through the conversion.
+PDFX_M64 double widened(float x) {
+  const uint32_t b = fbits(x), m = b & 0x7fffffffu;
+  const bool normal = m - 0x00800000u < 0x7f000000u;
+  if (!normal && m != 0u) return static_cast<double>(x);
+  const uint32_t hi = (b & 0x80000000u) | (normal ? (m >> 3) + 0x38000000u : 0u);
+  return from_bits(static_cast<int64_t>(static_cast<uint64_t>(hi) << 32 | static_cast<uint64_t>(b << 29)));
+}
+PDFX_M64 double widened(double x) { return x; }
+
 // x >= 0 (a zero of either sign; false for NaN) and x < c for a positive c, on the bits.
 PDFX_M64 bool nonneg(double x) {
   const uint64_t b = static_cast<uint64_t>(bits(x));

@@ -23,3 +23,14 @@ def test_errors_in_units_in_the_last_place(tmp_path):
     assert set(out) == {"log", "cos", "sin", "rcp", "root", "rcbrt"}
     for k, v in out.items():
         assert float(v) < 2.0, (k, v)
+
+
+def test_widened_is_the_conversion(tmp_path):
+    exe = str(tmp_path / "widened")
+    try:
+        subprocess.run(["g++", "-O2", "-std=c++17", "-I", CSRC, os.path.join(ROOT, "tests", "math64_widened_harness.cpp"),
+                        "-o", exe], check=True)
+    except FileNotFoundError:
+        pytest.skip("no g++")
+    bad, n = subprocess.run([exe], check=True, capture_output=True, text=True).stdout.split()
+    assert bad == "0" and int(n) > 1000000
