@@ -1837,9 +1837,8 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 ? 1280 : 1024) / 256) ran
 // kTileBig (larger ones: stats_big_kernel): the classes' launches and their branches cost
 // more than they save there.
 template <typename T>
-__global__ void __launch_bounds__(256, (sizeof(T) == 4 ? 1280 : 1024) / 256) small_grid_kernel(const StatsArgs<T> a) {
-  chain_wait();
-  chain_go();
+__global__ void __launch_bounds__(256, (sizeof(T) == 4 ? 1280 : 1024) / 256) small_grid_kernel(const StatsArgs<T> a, Place at) {
+  if (!sibling_enter(at)) return;
   extern __shared__ __align__(16) unsigned char rank_smem[];
   RankTile<T, kTileBig, 256>& t = *reinterpret_cast<RankTile<T, kTileBig, 256>*>(rank_smem);
   const int e = blockIdx.x;
@@ -1886,16 +1885,10 @@ void configure_tiles() {
   allow(reinterpret_cast<const void*>(warp_tile_kernel<T, 512, 2, 2>), warp_tile_smem<T, 512, 2>());
 }
 
-// A grid of up to four elements per multiprocessor (us per step, classes / one launch: 64
-// elements of 100 particles FP32 61.0 / 55.6, FP64 85.3 / 79.9; 400: 63.5 / 59.6, 113.7 /
-// 112.4; 900: 66.2 / 70.4, 170.0 / 166.7; 1,600: 73.5 / 83.9, 211 / 238).
-constexpr int kSmallGrid = 4;
 template <typename T>
-bool launch_stats_small_impl(const StatsArgs<T>& a, int num_sms, cudaStream_t s) {
-  if (a.ne <= 0 || a.ne > kSmallGrid * num_sms) return false;
+void launch_stats_small_impl(const StatsArgs<T>& a, cudaStream_t s) {
   configure_tiles<T>();
-  launch_chained(small_grid_kernel<T>, a.ne, 256, sizeof(RankTile<T, kTileBig, 256>), s, a);
-  return true;
+  launch_sibling(small_grid_kernel<T>, a.ne, 1, 256, sizeof(RankTile<T, kTileBig, 256>), s, a, Place::kLater);
 }
 
 template <typename T>
@@ -1910,29 +1903,29 @@ void launch_stats_tiles_impl(const StatsArgs<T>& a, int num_sms, cudaStream_t s_
   // class in a tile of 1,024).
   const unsigned grid = static_cast<unsigned>(a.ne);
   const bool one = s_small == s_mid && s_large == s_mid;
-  const Place first = one ? Place::kFirst : Place::kBranch, later = one ? Place::kLater : Place::kBranch;
+  const Place at = one ? Place::kLater : Place::kBranch;   // after the large-element kernel
   if (a.cond_mode == 1) {
-    launch_sibling(stats_tile_kernel<T, 1024, 256, 1>, grid, 1, 256, 0, s_large, a, first);
-    launch_sibling(stats_tile_kernel<T, 512, 128, 2>, grid, 1, 128, 0, s_mid, a, later);
-    launch_sibling(stats_tile_kernel<T, 256, 128, 0>, grid, 1, 128, 0, s_small, a, later);
+    launch_sibling(stats_tile_kernel<T, 1024, 256, 1>, grid, 1, 256, 0, s_large, a, at);
+    launch_sibling(stats_tile_kernel<T, 512, 128, 2>, grid, 1, 128, 0, s_mid, a, at);
+    launch_sibling(stats_tile_kernel<T, 256, 128, 0>, grid, 1, 128, 0, s_small, a, at);
   } else {
     configure_tiles<T>();
     // the classes above the mean count by a factor of two and more hold few elements: over
     // their lists where blocks that return would take 10 us and more (0.5 ns each)
     const int64_t mean = a.np / a.ne;
     const int few = a.ne >= 20000 ? 8 * (num_sms > 0 ? num_sms : 1) : 0;
-    launch_rank_tile<T, 768, 192, 1>(a, mean <= 256 ? few : 0, first, s_large);
+    launch_rank_tile<T, 768, 192, 1>(a, mean <= 256 ? few : 0, at, s_large);
     // 769..1024 from the large-element list: 4 blocks per SM
     launch_sibling(rank_big_kernel<T>, 4 * (num_sms > 0 ? num_sms : 1), 0, 256, sizeof(RankTile<T, kTileBig, 256>),
-                   s_large, a, later);
-    launch_warp_tile<T, 256, 4, 0>(a, later, s_small);
+                   s_large, a, at);
+    launch_warp_tile<T, 256, 4, 0>(a, at, s_small);
     // 257..512: a block per element with bucket levels in the FP32 form; where the moment sums
     // are FP64 a warp per element, whose register sort leaves the FP64 pipe the shorter wait
     // (8,100 elements of 300 and 500 particles: FP64 form 350 and 530 us -> 292 and 408, FP64
     // accumulation 326 and 464 -> 244 and 363; FP32 form 216 -> 359 us for 12,100 of 350, its
     // 15 resident warps too few)
-    if (mean > 128 && (sizeof(T) == 8 || a.acc64)) launch_warp_tile<T, 512, 2, 2>(a, later, s_mid);
-    else launch_rank_tile<T, 512, 128, 2>(a, mean <= 128 ? few : 0, later, s_mid);
+    if (mean > 128 && (sizeof(T) == 8 || a.acc64)) launch_warp_tile<T, 512, 2, 2>(a, at, s_mid);
+    else launch_rank_tile<T, 512, 128, 2>(a, mean <= 128 ? few : 0, at, s_mid);
   }
 }
 

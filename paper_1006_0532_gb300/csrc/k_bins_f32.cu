@@ -10,8 +10,8 @@ void launch_stats_tiles<float>(const StatsArgs<float>& a, int num_sms, cudaStrea
 }
 
 template <>
-bool launch_stats_small<float>(const StatsArgs<float>& a, int num_sms, cudaStream_t s) {
-  return launch_stats_small_impl<float>(a, num_sms, s);
+void launch_stats_small<float>(const StatsArgs<float>& a, cudaStream_t s) {
+  launch_stats_small_impl<float>(a, s);
 }
 
 }  // namespace pdfx

@@ -10,8 +10,8 @@ void launch_stats_tiles<double>(const StatsArgs<double>& a, int num_sms, cudaStr
 }
 
 template <>
-bool launch_stats_small<double>(const StatsArgs<double>& a, int num_sms, cudaStream_t s) {
-  return launch_stats_small_impl<double>(a, num_sms, s);
+void launch_stats_small<double>(const StatsArgs<double>& a, cudaStream_t s) {
+  launch_stats_small_impl<double>(a, s);
 }
 
 }  // namespace pdfx
