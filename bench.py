@@ -832,7 +832,7 @@ def main():
                                         "x particles)" if traffic is not None else
                                         "null: no ncu capture of these kernel sources (sha256 %s)"
                                         % src_hash[:16]),
-                     "kernel": ("binning: stats_tile_kernel<float> and rank_tile_kernel<float> "
+                     "kernel": ("binning: warp_tile_kernel<float> and rank_tile_kernel<float> "
                                  "(three size-class launches per step)"
                                 if dom == "statistics_binning" else "advance_kernel<float>"),
                      "algorithmic_bytes_per_particle": per_p, "peak_source": peak_kind,
