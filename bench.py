@@ -46,18 +46,19 @@ SINGLE_POSITION_STEP_BYTES = 98
 # measured, so after any change of the code the bench reports traffic as null until the
 # next capture.
 NCU_RECORDS = {
-    # channel_50k, 25.0M particles (FP32) and 5.0M (FP64 form), one GB300
-    "884109f4ef9f937ec8e6c0f340dcb09331d34ffda8b87605775c6a478bbb70d9": {
-        "traffic": {"advance": (1162.113e6 + 949.069312e6) / 25.0e6,
-                    "statistics_binning": (0.066048e6 + 688.4096e6 + 49.580032e6 + 237.703168e6
-                                           + 10.723072e6) / 25.0e6},
-        "limiter": {"advance": "instruction issue: 76% issue-active at 49% warps active (64 "
-                               "registers cap 4 blocks of 256), long-scoreboard stalls first; "
-                               "DRAM 25% of peak",
-                    "statistics_binning": "instruction issue and shared-memory latency: 71% "
+    # the benchmark's grid family at 23,908 elements, 11.95M particles (DRAM) and 12,152
+    # elements, 6.08M particles (limiters; FP64 form 1.22M), one GB300
+    "1242a8212d14486341fa32bbc8634b7ff516c4f375ce2fe044324b92e35c3940": {
+        "traffic": {"advance": (554.974464e6 + 418.765056e6) / 11.954e6,
+                    "statistics_binning": (86.025472e6 + 0.096256e6 + 0.06784e6 + 0.06656e6 + 330.97344e6
+                                           + 19.071488e6 + 0.067328e6) / 11.954e6},
+        "limiter": {"advance": "instruction issue and latency: 67% issue-active at 48% warps active "
+                               "(64 registers cap 4 blocks of 256), long-scoreboard stalls first; "
+                               "DRAM 23% of peak",
+                    "statistics_binning": "instruction issue and shared-memory latency: 69% "
                                           "issue-active (<= 512 class), short-scoreboard stalls "
-                                          "first; DRAM 13% of peak"},
-        "f64_advance_fp64_inst_per_particle": (1407568787 + 454038118 + 836638858) / 5.0e6,
+                                          "first; DRAM 10% of peak"},
+        "f64_advance_fp64_inst_per_particle": (222434799 + 75662106 + 138463756) / 1.2152e6,
     },
 }
 STAGES = ["advance", "plan", "lists", "redistribute", "statistics_binning", "node_average"]
