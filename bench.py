@@ -48,14 +48,14 @@ SINGLE_POSITION_STEP_BYTES = 98
 NCU_RECORDS = {
     # the benchmark's grid family at 23,908 elements, 11.95M particles (DRAM) and 12,152
     # elements, 6.08M particles (limiters; FP64 form 1.22M), one GB300
-    "1242a8212d14486341fa32bbc8634b7ff516c4f375ce2fe044324b92e35c3940": {
-        "traffic": {"advance": (554.974464e6 + 418.765056e6) / 11.954e6,
-                    "statistics_binning": (86.025472e6 + 0.096256e6 + 0.06784e6 + 0.06656e6 + 330.97344e6
-                                           + 19.071488e6 + 0.067328e6) / 11.954e6},
+    "0826dbb91f2d07780009902878957367a0de916e9e0d4930764a3aea45b27082": {
+        "traffic": {"advance": (555.000832e6 + 418.712576e6) / 11.954e6,
+                    "statistics_binning": (86.046464e6 + 0.105216e6 + 0.067328e6 + 0.06656e6 + 330.742016e6
+                                           + 19.325184e6 + 0.067072e6) / 11.954e6},
         "limiter": {"advance": "instruction issue and latency: 67% issue-active at 48% warps active "
                                "(64 registers cap 4 blocks of 256), long-scoreboard stalls first; "
                                "DRAM 23% of peak",
-                    "statistics_binning": "instruction issue and shared-memory latency: 69% "
+                    "statistics_binning": "instruction issue and shared-memory latency: 67% "
                                           "issue-active (<= 512 class), short-scoreboard stalls "
                                           "first; DRAM 10% of peak"},
         "f64_advance_fp64_inst_per_particle": (222434799 + 75662106 + 138463756) / 1.2152e6,
