@@ -261,6 +261,17 @@ PDFX_HD void pcg_direction(bool fr, const double* s, double z, double* d) {
   *d = fr ? z + s[S_BETA] * *d : 0.0;
 }
 
+// Where a solve that runs in one launch leaves the sum of one of a component's `per` items, to be
+// read by every block: pass 0's sums (d q) in set 0, pass 1's (r z and z z) in sets 1 and 2.  A
+// block publishes a pass's sums, arrives at the barrier and only then reads the others', so a
+// block that is through the barrier may publish the next pass's while another still reads this
+// one's: passes that follow one another need sets of their own.  A set is written again two
+// passes later, after a barrier at which every reader has arrived.
+constexpr int kPcgSumSets = 3;
+PDFX_HD size_t pcg_sum_slot(int pass, int which, int C, int per, int c, int item) {
+  return (static_cast<size_t>(pass + which) * C + c) * static_cast<size_t>(per) + item;
+}
+
 // A component with a zero reduced load has the zero solution on its free nodes.
 PDFX_HD void pcg_trivial(bool fr, const double* s, double* x) {
   if (s[S_BNORM] == 0.0 && fr) *x = 0.0;

@@ -158,8 +158,9 @@ __global__ void pcg_scalar_kernel(int step, int nblk, const double* __restrict__
 // * CLUSTER, where a component fits one cluster of 16 blocks: a cluster per component, no
 //   traffic beyond it.  Neighbours' z and d are read from, and item sums pushed to, the
 //   other blocks' shared memory, with a hardware cluster barrier per pass.
-// * Otherwise a cooperative launch: z and d in global memory, item sums in slots, one
-//   arrival counter for all blocks.  (A counter costs 2,900 cycles at any block count;
+// * Otherwise a cooperative launch: z and d in global memory, item sums in slots (three sets,
+//   since blocks read a pass's sums after they have arrived: eops::pcg_sum_slot), one arrival
+//   counter for all blocks.  (A counter costs 2,900 cycles at any block count;
 //   polling every block's slot instead 2,600 at 5 blocks but 7,600 at 99, since writers and
 //   pollers share the slots' lines.)  The wait is bounded: a block that gives up leaves its
 //   mark in the scalars and returns, and so do the others, whose own waits then run out.
@@ -181,7 +182,7 @@ struct SolveArgs {
   double *x, *r, *z, *q, *d0, *d1;
   double tol;
   double* sc;
-  double* slots;         // [2][C][nvb P] item sums of a pass
+  double* slots;         // [kPcgSumSets][C][nvb P] item sums (eops::pcg_sum_slot)
   unsigned* arrived;     // blocks that have published, over all passes (zero at the start)
 };
 
@@ -261,7 +262,7 @@ __device__ __forceinline__ bool grid_exchange(const SolveArgs& a, unsigned targe
 
 // Totals of a pass's item sums and the scalars from them (eops::pcg_scalars steps 2 and 3,
 // its two sums apart), one component and sum per warp; every block forms them all.  sums: the
-// pass's sums, [which][item] in the cluster, [which][component][item] in the slots.
+// cluster's sums of the pass, [which][item], or the slots.
 template <int P, int W, bool CLUSTER>
 __device__ __forceinline__ void solve_totals(const SolveArgs& a, int pass, int c0, int c1, const double* sums,
                                              double* ssc, const int* on, int* on_next) {
@@ -273,8 +274,8 @@ __device__ __forceinline__ void solve_totals(const SolveArgs& a, int pass, int c
   double v[V][P];
   auto fetch = [&](int t) {
     const int c = c0 + (pass ? t >> 1 : t), which = pass ? t & 1 : 0;
-    const double* src = CLUSTER ? sums + which * kRedBlocks
-                                : sums + (static_cast<size_t>(which) * a.C + c) * static_cast<size_t>(per);
+    const double* src = sums + (CLUSTER ? static_cast<size_t>(which) * kRedBlocks
+                                        : eops::pcg_sum_slot(pass, which, a.C, per, c, 0));
 #pragma unroll
     for (int m = 0; m < V; ++m) {
       const int vb = lane + 32 * m;
@@ -525,7 +526,7 @@ __global__ void __launch_bounds__(kEB / P) pcg_solve_kernel(SolveArgs a) {
           if (lane < kClusterBlocks)
             cluster_store(cluster_addr(&csum[pass + which][part_of(k)], static_cast<uint32_t>(lane)), sum);
         } else if (lane == 0) {
-          __stcg(a.slots + static_cast<size_t>(which) * a.C * per + static_cast<size_t>(c) * per + part_of(k), sum);
+          __stcg(a.slots + eops::pcg_sum_slot(pass, which, a.C, per, c, part_of(k)), sum);
         }
       }
       if (CLUSTER) {
@@ -633,13 +634,13 @@ __global__ void __launch_bounds__(kEB) pcg_stream_kernel(SolveArgs a) {
         __syncthreads();
         for (int t = warp; t < nr * (pass + 1); t += W) {
           const int q = pass ? t >> 1 : t, which = pass ? t & 1 : 0;
-          const int i = i0 + q * static_cast<int>(gridDim.x);
-          if (!act[cur][i / a.nvb]) continue;
+          const int i = i0 + q * static_cast<int>(gridDim.x), c = i / a.nvb;
+          if (!act[cur][c]) continue;
           double v[8];
 #pragma unroll
           for (int m = 0; m < 8; ++m) v[m] = sums[q][which][lane + 32 * m];
           const double sum = tree256(v, W);
-          if (lane == 0) __stcg(a.slots + static_cast<size_t>(which) * items + i, sum);
+          if (lane == 0) __stcg(a.slots + eops::pcg_sum_slot(pass, which, a.C, a.nvb, c, i - c * a.nvb), sum);
         }
         __syncthreads();
       }
@@ -812,7 +813,7 @@ int pcg_blocks(int nn) {
 // Partial sums and scalars of the setup passes, the solve kernel's slots and counter.
 size_t pcg_scratch_doubles(int nn, int C) {
   const size_t nb = static_cast<size_t>(C) * static_cast<size_t>(pcg_blocks(nn));
-  return 2 * nb + static_cast<size_t>(C) * kSc + 4 * nb + 1;
+  return 2 * nb + static_cast<size_t>(C) * kSc + eops::kPcgSumSets * nb + 1;
 }
 
 template <typename T>
@@ -931,7 +932,7 @@ cudaError_t launch_pcg_solve(const FemDev& m, const PcgArgs& a, int limit, int n
   k.tol = a.tol;
   k.sc = a.scratch + 2 * static_cast<size_t>(a.C) * k.nvb;
   k.slots = k.sc + static_cast<size_t>(a.C) * kSc;
-  k.arrived = reinterpret_cast<unsigned*>(k.slots + 4 * static_cast<size_t>(a.C) * k.nvb);
+  k.arrived = reinterpret_cast<unsigned*>(k.slots + eops::kPcgSumSets * static_cast<size_t>(a.C) * k.nvb);
   cudaError_t e = cudaMemsetAsync(k.arrived, 0, sizeof(double), s);
   if (e != cudaSuccess) return e;
   e = cudaMemsetAsync(k.sc + S_FAILED, 0, sizeof(double), s);
