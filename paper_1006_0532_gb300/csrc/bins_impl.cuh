@@ -1825,7 +1825,7 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 ? 1280 : 1024) / 256) sma
   if (N <= kTileBig) element_rank_tile<T, kTileBig, 256>(a, t, e, N, moves);
 }
 
-template <typename T> bool rank_configured[kMaxDevices];
+template <typename T> OncePerDevice rank_configured;
 
 // One block per entry of one size class of the plan's tile lists (tile_element); the grid
 // covers every element and blocks past the class count return.  The register cap keeps 1536
@@ -1846,20 +1846,23 @@ __global__ void __launch_bounds__(THREADS, (sizeof(T) == 4 ? 1536 : 1024) / THRE
 
 template <typename T>
 void configure_tiles() {
-  if (!first_use_on_device(rank_configured<T>)) return;
   constexpr size_t big = sizeof(RankTile<T, kTileBig, 256>);
   static_assert(big <= 227 * 1024, "rank tile exceeds shared memory");
-  auto allow = [](const void* f, size_t bytes) {
-    cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
-  };
-  allow(reinterpret_cast<const void*>(small_grid_kernel<T>), big);
-  allow(reinterpret_cast<const void*>(rank_big_kernel<T>), big);
-  allow(reinterpret_cast<const void*>(rank_tile_kernel<T, 768, 192, 1>), sizeof(RankTile<T, 768, 192>));
-  allow(reinterpret_cast<const void*>(rank_list_kernel<T, 768, 192, 1>), sizeof(RankTile<T, 768, 192>));
-  allow(reinterpret_cast<const void*>(rank_tile_kernel<T, 512, 128, 2>), sizeof(RankTile<T, 512, 128>));
-  allow(reinterpret_cast<const void*>(rank_list_kernel<T, 512, 128, 2>), sizeof(RankTile<T, 512, 128>));
-  allow(reinterpret_cast<const void*>(warp_tile_kernel<T, 256, 4, 0>), warp_tile_smem<T, 256, 4>());
-  allow(reinterpret_cast<const void*>(warp_tile_kernel<T, 512, 2, 2>), warp_tile_smem<T, 512, 2>());
+  once_on_device(rank_configured<T>, [] {
+    cudaError_t rc = cudaSuccess;
+    auto allow = [&](const void* f, size_t bytes) {
+      if (rc == cudaSuccess) rc = allow_shared(f, bytes);
+    };
+    allow(reinterpret_cast<const void*>(small_grid_kernel<T>), big);
+    allow(reinterpret_cast<const void*>(rank_big_kernel<T>), big);
+    allow(reinterpret_cast<const void*>(rank_tile_kernel<T, 768, 192, 1>), sizeof(RankTile<T, 768, 192>));
+    allow(reinterpret_cast<const void*>(rank_list_kernel<T, 768, 192, 1>), sizeof(RankTile<T, 768, 192>));
+    allow(reinterpret_cast<const void*>(rank_tile_kernel<T, 512, 128, 2>), sizeof(RankTile<T, 512, 128>));
+    allow(reinterpret_cast<const void*>(rank_list_kernel<T, 512, 128, 2>), sizeof(RankTile<T, 512, 128>));
+    allow(reinterpret_cast<const void*>(warp_tile_kernel<T, 256, 4, 0>), warp_tile_smem<T, 256, 4>());
+    allow(reinterpret_cast<const void*>(warp_tile_kernel<T, 512, 2, 2>), warp_tile_smem<T, 512, 2>());
+    return rc;
+  });
 }
 
 template <typename T>

@@ -868,6 +868,21 @@ namespace {
 
 constexpr size_t kMaxSolveSmem = 220 * 1024;   // dynamic, beside the kernel's own arrays
 
+OncePerDevice solve_configured;
+cudaError_t configure_solves() {
+  return once_on_device(solve_configured, [] {
+    const void* const kernels[] = {reinterpret_cast<const void*>(pcg_solve_kernel<2, true>),
+                                   reinterpret_cast<const void*>(pcg_solve_kernel<1, true>),
+                                   reinterpret_cast<const void*>(pcg_solve_kernel<1, false>)};
+    for (int k = 0; k < 3; ++k) {
+      cudaError_t e = allow_shared(kernels[k], kMaxSolveSmem);
+      if (e == cudaSuccess && k < 2) e = cudaFuncSetAttribute(kernels[k], cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+      if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+  });
+}
+
 template <int P, bool CLUSTER>
 size_t solve_smem(const SolveArgs& k) {
   constexpr int NT = kEB / P;
@@ -877,9 +892,6 @@ size_t solve_smem(const SolveArgs& k) {
 
 cudaError_t start_solve(void (*f)(SolveArgs), SolveArgs k, int blocks, int threads, size_t smem, bool cluster,
                         cudaStream_t s) {
-  cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-  if (e == cudaSuccess && cluster) e = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  if (e != cudaSuccess) return e;
   cudaLaunchAttribute at{};
   if (cluster) {
     at.id = cudaLaunchAttributeClusterDimension;
@@ -933,7 +945,9 @@ cudaError_t launch_pcg_solve(const FemDev& m, const PcgArgs& a, int limit, int n
   k.sc = a.scratch + 2 * static_cast<size_t>(a.C) * k.nvb;
   k.slots = k.sc + static_cast<size_t>(a.C) * kSc;
   k.arrived = reinterpret_cast<unsigned*>(k.slots + eops::kPcgSumSets * static_cast<size_t>(a.C) * k.nvb);
-  cudaError_t e = cudaMemsetAsync(k.arrived, 0, sizeof(double), s);
+  cudaError_t e = configure_solves();
+  if (e != cudaSuccess) return e;
+  e = cudaMemsetAsync(k.arrived, 0, sizeof(double), s);
   if (e != cudaSuccess) return e;
   e = cudaMemsetAsync(k.sc + S_FAILED, 0, sizeof(double), s);
   if (e != cudaSuccess) return e;

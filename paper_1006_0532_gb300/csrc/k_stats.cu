@@ -933,8 +933,8 @@ __global__ void node_average_kernel(const double* __restrict__ emom, const int32
   nmom[k] = acc * r;
 }
 
-template <typename T> bool redist_configured[kMaxDevices];
-template <typename T> bool stats_configured[kMaxDevices];
+template <typename T> OncePerDevice redist_configured;
+template <typename T> OncePerDevice stats_configured;
 
 }  // namespace
 
@@ -968,10 +968,8 @@ void launch_redistribute(Particles<T> p, Plan& pl, int K, const InstDev<T>* inst
                          int num_sms, unsigned long long* diag, int* err, cudaStream_t s) {
   const unsigned grid = static_cast<unsigned>(num_sms > 0 ? num_sms : 1);
   const size_t apply_smem = 12 * static_cast<size_t>(kRedistCap);
-  if (first_use_on_device(redist_configured<T>)) {
-    cudaFuncSetAttribute(apply_moves_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         static_cast<int>(apply_smem));
-  }
+  once_on_device(redist_configured<T>,
+                 [&] { return allow_shared(reinterpret_cast<const void*>(apply_moves_kernel<T>), apply_smem); });
   launch_chained(select_donors_kernel<T>, grid, kRedistThreads, 0, s, p, pl, K);
   launch_chained(apply_moves_kernel<T>, grid, kRedistThreads, apply_smem, s, p, pl, K, inst, np, geo, topo, stepc);
   launch_chained(commit_moves_kernel<T>, grid, 256, 0, s, p, pl, K, np, ne, diag, err);
@@ -989,10 +987,8 @@ template <typename T>
 int launch_stats(const StatsArgs<T>& a, int num_sms, cudaStream_t s, const SideStreams* side) {
   const size_t big = stats_smem_bytes<T>(kBigCap);
   static_assert(5 * 8 * kBigCap + 11 * kBigCap <= 227 * 1024, "large-element tile exceeds shared memory");
-  if (first_use_on_device(stats_configured<T>)) {
-    cudaFuncSetAttribute(stats_big_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         static_cast<int>(big));
-  }
+  once_on_device(stats_configured<T>,
+                 [&] { return allow_shared(reinterpret_cast<const void*>(stats_big_kernel<T>), big); });
   // a small grid: one launch for every element up to kTileBig, no branches
   // Large elements, one per block and multiprocessor: with all its threads where the mean count
   // lets many exist; else mostly none does, and half the threads start sooner (64 elements of 40

@@ -8,6 +8,7 @@
 
 #include "../../include/pdfx.h"
 #include "eulerian_ops.h"
+#include "once.h"
 #include "pdfx_device.cuh"
 
 namespace pdfx {
@@ -346,16 +347,15 @@ struct Ctx {
 template <typename T>
 Particles<T> particles_of(Ctx& c, int which);
 
-// Kernel attributes are per device: a flag per device records that a kernel's attributes
-// were set on it (setting them twice from racing host threads is harmless).  True on the
-// first call for the current device (and whenever the device cannot be told).
-constexpr int kMaxDevices = 64;
-inline bool first_use_on_device(bool (&flags)[kMaxDevices]) {
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return true;
-  if (flags[dev]) return false;
-  flags[dev] = true;
-  return true;
+// set() once for the current device (every time where the device cannot be told).
+template <typename F>
+inline cudaError_t once_on_device(OncePerDevice& once, F set) {
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess) dev = -1;
+  return static_cast<cudaError_t>(once.run(dev, set));
+}
+inline cudaError_t allow_shared(const void* kernel, size_t bytes) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
 }
 
 // A step is a chain of kernels, most of them a few microseconds long on small grids, each
