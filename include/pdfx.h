@@ -305,6 +305,14 @@ int  pdfx_get_launch_shapes(const void *ctx, int32_t *adv_block, int32_t *sort_e
  * 256 particles).  None of them changes a result.  PDFX_ERR_ARG for any other value. */
 int  pdfx_set_launch_shapes(void *ctx, int32_t adv_block, int32_t sort_every, int32_t tile_split);
 
+/* The form of the conjugate-gradient solves' launch to start from: 0 (default) thread-block
+ * clusters of 16 where the grid is small enough for them, 1 one cooperative launch with the
+ * systems in shared memory, 2 one cooperative launch that streams them, 3 plain kernels.  A
+ * solve takes the first form from there on that the context is granted (a context with a
+ * share of the device's multiprocessors may get neither of the first).  Every form gives the
+ * same bits and iteration counts.  PDFX_ERR_ARG for any other value. */
+int  pdfx_set_solve_form(void *ctx, int32_t form);
+
 /* Nodal statistics [nn][13] and element statistics [ne][13] with counts [ne] of the last
  * step (or initialisation), into host or device memory.  Synchronous for host output. */
 int  pdfx_get_nodal_stats(void *ctx, double *out, int on_device, void *stream);

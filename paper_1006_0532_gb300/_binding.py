@@ -121,6 +121,7 @@ def lib():
                 "pdfx_measure_fp64_rate": (C.c_int, [C.POINTER(C.c_double), vp]),
                 "pdfx_get_launch_shapes": (C.c_int, [vp, vp, vp, vp]),
                 "pdfx_set_launch_shapes": (C.c_int, [vp, i32, i32, i32]),
+                "pdfx_set_solve_form": (C.c_int, [vp, i32]),
                 "pdfx_wp_rhs": (C.c_int, [vp, vp, vp, vp]),
                 "pdfx_wp_solve": (C.c_int, [vp, vp, vp, vp, dp, i32, C.POINTER(i32), vp]),
                 "pdfx_update_wp": (C.c_int, [vp, dp, i32, C.POINTER(i32), vp]),
@@ -420,6 +421,10 @@ class Context:
         """Sets the launch shapes that change no result (-1 keeps the current one)."""
         self._check(lib().pdfx_set_launch_shapes(self.h, int(adv_block), int(sort_every),
                                                  int(tile_split)), "pdfx_set_launch_shapes")
+
+    def set_solve_form(self, form: int):
+        """The first form of the conjugate-gradient solves' launch to try (0 to 3; changes no result)."""
+        self._check(lib().pdfx_set_solve_form(self.h, int(form)), "pdfx_set_solve_form")
 
     def step_many(self, dt: float, nsteps: int, use_graph: bool = True, stream=None):
         self._check(lib().pdfx_step_many(self.h, float(dt), int(nsteps), int(bool(use_graph)),

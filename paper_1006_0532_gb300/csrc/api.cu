@@ -1168,11 +1168,12 @@ WpConst wp_const(const Ctx& c) {
 }
 
 // Iterates until every component meets its stopping rule (a component that has converged
-// stops changing), in launches of kPcgChunk iterations that end early once none is left;
+// stops changing), in launches of at most kPcgChunk iterations that end early once none is left;
 // the host reads the scalars after each.  As many iterations as fit max_iter rounded up to
 // a multiple of 16 may run; more than max_iter of a component is an error.
 constexpr int kPcgChunk = 512;
-int run_pcg(Ctx& c, const PcgArgs& a, int32_t max_iter, int32_t* iters, cudaStream_t s) {
+int run_pcg(Ctx& c, PcgArgs a, int32_t max_iter, int32_t* iters, cudaStream_t s) {
+  a.form = c.solve_form;
   launch_pcg_setup(c.fem, a, s);
   c.launches += 8;
   const double* sc = pcg_scalars(a, c.nn);
@@ -1182,9 +1183,10 @@ int run_pcg(Ctx& c, const PcgArgs& a, int32_t max_iter, int32_t* iters, cudaStre
   for (;;) {
     const int chunk = static_cast<int>(std::min<int64_t>(kPcgChunk, most_iter - done));
     if (chunk > 0) {
-      PDFX_CUDA(launch_pcg_solve(c.fem, a, chunk, c.num_sms, s));
-      c.launches++;
-      done += chunk;
+      int ran = 0, launches = 0;
+      PDFX_CUDA(launch_pcg_solve(c.fem, a, chunk, c.num_sms, &ran, &launches, s));
+      c.launches += launches;
+      done += ran;
     }
     PDFX_CUDA(cudaMemcpyAsync(h.data(), sc, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, s));
     PDFX_CUDA(cudaStreamSynchronize(s));
@@ -1630,6 +1632,13 @@ int pdfx_set_launch_shapes(void* ctx, int32_t adv_block, int32_t sort_every, int
   if (sort_every >= 0) c->prm.sort_every = sort_every;
   if (tile_split >= 0) c->tile_split = tile_split;
   drop_graph(*c);
+  return PDFX_OK;
+}
+
+int pdfx_set_solve_form(void* ctx, int32_t form) {
+  Ctx* c = as_ctx(ctx);
+  if (!c || form < kSolveCluster || form > kSolvePlain) return PDFX_ERR_ARG;
+  c->solve_form = form;
   return PDFX_OK;
 }
 

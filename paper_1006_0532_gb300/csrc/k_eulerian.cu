@@ -137,6 +137,15 @@ __global__ void pcg_scalar_kernel(int step, int nblk, const double* __restrict__
   if (threadIdx.x == 0) eops::pcg_scalars(step, t0, t1, tol, sc + c * kSc);
 }
 
+// d = free ? z + beta d : 0 for the components still iterating.
+__global__ void pcg_direction_kernel(int nn, int C, const uint8_t* __restrict__ fixed, const double* __restrict__ z,
+                                     double* __restrict__ d, const double* __restrict__ sc) {
+  const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (i >= static_cast<int64_t>(nn) * C) return;
+  const int c = static_cast<int>(i / nn);
+  eops::pcg_direction(!fixed || !fixed[i], sc + c * kSc, z[i], d + i);
+}
+
 // ---------------------------------------------------------------------------------------
 // The conjugate-gradient iterations of a solve in one launch.  The grids here hold 1e3 to
 // 1e5 nodes, so an iteration is a chain of latencies (two sums over all nodes, each needed by
@@ -908,13 +917,51 @@ cudaError_t start_solve(void (*f)(SolveArgs), SolveArgs k, int blocks, int threa
   cfg.stream = s;
   cfg.attrs = &at;
   cfg.numAttrs = 1;
+  if (cluster) {   // none fits where the context has a share of the device without 16 multiprocessors together
+    int fit = 0;
+    const cudaError_t e = cudaOccupancyMaxActiveClusters(&fit, f, &cfg);
+    if (e != cudaSuccess || fit < 1) return e != cudaSuccess ? e : cudaErrorInvalidClusterSize;
+  }
   return cudaLaunchKernelEx(&cfg, f, k);
 }
+
+// A launch that the context's share of the device does not grant, and nothing worse: nothing has
+// run and a smaller one may.
+bool refused(cudaError_t e) {
+  if (e != cudaErrorCooperativeLaunchTooLarge && e != cudaErrorInvalidClusterSize &&
+      e != cudaErrorLaunchOutOfResources && e != cudaErrorInvalidConfiguration && e != cudaErrorNotSupported)
+    return false;
+  cudaGetLastError();   // it was the launch's alone
+  return true;
+}
+
+// Iterations of every component still iterating as six plain kernels each, for a context that is
+// granted no launch whose blocks may wait for one another: the same bits.
+void launch_pcg_iterations(const FemDev& m, const PcgArgs& a, int n, cudaStream_t s) {
+  const int nn = m.nn, C = a.C, nblk = pcg_blocks(nn);
+  const int64_t all = static_cast<int64_t>(nn) * C;
+  double* part = a.scratch;
+  double* sc = a.scratch + 2 * static_cast<size_t>(C) * nblk;
+  const dim3 grid(static_cast<unsigned>(nblk), static_cast<unsigned>(C));
+  for (int it = 0; it < n; ++it) {
+    pcg_direction_kernel<<<blocks_for(all), kEB, 0, s>>>(nn, C, a.fixed, a.z, a.d, sc);
+    spmv_kernel<<<blocks_for(all), kEB, 0, s>>>(nn, C, m.row, m.col, a.val, a.d, a.q);
+    for (int step = 2; step <= 3; ++step) {
+      pcg_pass_kernel<<<grid, kEB, 0, s>>>(step, nn, a.fixed, a.diag, a.b, a.x, a.r, a.z, a.d, a.q, sc, part);
+      pcg_scalar_kernel<<<C, kEB, 0, s>>>(step, nblk, part, a.tol, sc);
+    }
+  }
+}
+constexpr int kPlainChunk = 16;   // iterations between two looks at the scalars
 
 }  // namespace
 
 // Up to `limit` (even) iterations of every component still iterating, in one launch.  After
-// a launch that ran them all the direction is back in a.d.
+// a launch that ran them all the direction is back in a.d.  Where the context is not granted
+// that launch (a share of the device's multiprocessors), the next form down is taken, from a.form
+// on: cluster, cooperative with the rows in shared memory, streamed with as many blocks as are
+// granted, plain kernels.  Every form forms the same sums in the same order, so the bits and the
+// iterations do not depend on it.  *ran: the iterations that may have run, *launches: kernels.
 //
 // A component takes a cluster where that leaves a block at most two slices: beyond, the FP64
 // work of 16 multiprocessors (and the eight clusters of 16 that the GPU holds apart) outweighs
@@ -923,8 +970,11 @@ cudaError_t start_solve(void (*f)(SolveArgs), SolveArgs k, int blocks, int threa
 // 10.0 / 10.9 at 12,600, - / 10.0 / 11.0 at 25,200; 9 components 6.8 / 14.4 / 15.4, 11.5 /
 // 18.1 / 20.5, 26.2 / 21.1 / 24.9, - / 29 / 38 (two kernels per iteration: 20 and 23 at 1,104
 // and 25,200 nodes with 1 component).
-cudaError_t launch_pcg_solve(const FemDev& m, const PcgArgs& a, int limit, int num_sms, cudaStream_t s) {
+cudaError_t launch_pcg_solve(const FemDev& m, const PcgArgs& a, int limit, int num_sms, int* ran, int* launches,
+                             cudaStream_t s) {
   if (a.C > kMaxSystems) return cudaErrorInvalidValue;
+  *ran = limit;
+  *launches = 1;
   SolveArgs k{};
   k.nn = m.nn;
   k.C = a.C;
@@ -955,16 +1005,28 @@ cudaError_t launch_pcg_solve(const FemDev& m, const PcgArgs& a, int limit, int n
   const bool node_per_thread = m.nn <= kEB * kRedBlocks;
   const int P = 2 * k.nvb <= kClusterBlocks ? 2 : 1;
   k.K = (k.nvb * P + kClusterBlocks - 1) / kClusterBlocks;
-  if (node_per_thread && k.K <= 2) {
+  if (a.form <= kSolveCluster && node_per_thread && k.K <= 2) {
     const int blocks = k.C * kClusterBlocks;
-    return P == 2 ? start_solve(pcg_solve_kernel<2, true>, k, blocks, kEB / 2, solve_smem<2, true>(k), true, s)
-                  : start_solve(pcg_solve_kernel<1, true>, k, blocks, kEB, solve_smem<1, true>(k), true, s);
+    e = P == 2 ? start_solve(pcg_solve_kernel<2, true>, k, blocks, kEB / 2, solve_smem<2, true>(k), true, s)
+               : start_solve(pcg_solve_kernel<1, true>, k, blocks, kEB, solve_smem<1, true>(k), true, s);
+    if (!refused(e)) return e;
   }
   const int items = k.C * k.nvb;
   k.K = (items + sms - 1) / sms;
-  if (node_per_thread && solve_smem<1, false>(k) <= kMaxSolveSmem)
-    return start_solve(pcg_solve_kernel<1, false>, k, (items + k.K - 1) / k.K, kEB, solve_smem<1, false>(k), false, s);
-  return start_solve(pcg_stream_kernel, k, items < sms ? items : sms, kEB, 0, false, s);
+  if (a.form <= kSolveRows && node_per_thread && solve_smem<1, false>(k) <= kMaxSolveSmem) {
+    e = start_solve(pcg_solve_kernel<1, false>, k, (items + k.K - 1) / k.K, kEB, solve_smem<1, false>(k), false, s);
+    if (!refused(e)) return e;
+  }
+  if (a.form <= kSolveStream) {
+    for (int blocks = items < sms ? items : sms; blocks > 0; blocks /= 2) {
+      e = start_solve(pcg_stream_kernel, k, blocks, kEB, 0, false, s);
+      if (!refused(e)) return e;
+    }
+  }
+  *ran = limit < kPlainChunk ? limit : kPlainChunk;
+  *launches = 6 * *ran;
+  launch_pcg_iterations(m, a, *ran, s);
+  return cudaSuccess;
 }
 
 bool pcg_solve_failed(const double* h) { return h[S_FAILED] != 0.0; }

@@ -228,7 +228,9 @@ struct PcgArgs {
   double* d2 = nullptr;            // [C][nn] the second direction buffer
   double* scratch = nullptr;       // pcg_scratch_doubles(nn, C)
   double tol = 0.0;
+  int form = 0;                    // the first of the launch's forms to try
 };
+enum { kSolveCluster = 0, kSolveRows = 1, kSolveStream = 2, kSolvePlain = 3 };
 constexpr int kPcgScalars = eops::kPcgScalars;   // per component: rz, |b|, zz, alpha, beta, active, iterations
 constexpr int kRedBlocks = 256;                  // blocks of the solvers' reduction passes, at most
 constexpr int kPcgActive = eops::S_ACTIVE;
@@ -292,6 +294,7 @@ struct Ctx {
   // launch shapes (pdfx_autotune)
   int adv_block = 256;
   int tile_split = kTileSplit;  // the binning's size-class split (Plan::tile_split)
+  int solve_form = kSolveCluster;   // the first form of the solves' launch to try
   // instances of a batch (K = 1: the whole grid)
   int K = 1;
   std::vector<pdfx_params> iprm;        // [K] parameters (K > 1 only)
@@ -490,7 +493,8 @@ void launch_wp_bc(const T* fields, int nn, const WpConst& k, const int8_t* ncls,
 void launch_assemble_wp(const FemDev& m, const double* L, double* aval, double* adiag, cudaStream_t s);
 void launch_spmv(const FemDev& m, const double* val, int C, const double* x, double* y, cudaStream_t s);
 void launch_pcg_setup(const FemDev& m, const PcgArgs& a, cudaStream_t s);
-cudaError_t launch_pcg_solve(const FemDev& m, const PcgArgs& a, int limit, int num_sms, cudaStream_t s);
+cudaError_t launch_pcg_solve(const FemDev& m, const PcgArgs& a, int limit, int num_sms, int* ran, int* launches,
+                             cudaStream_t s);
 bool pcg_solve_failed(const double* scalars);   // host copy of the scalars: a wait in the solve ran out
 void launch_node_gradients(const FemDev& m, const int32_t* ne_off, const int32_t* ne_list, int nq,
                            const double* q, double* eg, double* gn, cudaStream_t s);
