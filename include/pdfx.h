@@ -22,11 +22,11 @@
  *    boundary.  pdfx_strerror() names a code.
  *  - Device work is enqueued on the caller's CUDA stream (a cudaStream_t passed as void*,
  *    NULL = the legacy default stream) and is asynchronous unless a call says otherwise.
- *    On large grids the statistics of a step fork onto two streams of the context's own and
- *    join back (events), so that the caller's stream sees every call's work in order, and a
- *    stream capture of a call records the branches as parallel nodes.  The step's kernels
- *    are launched with programmatic stream serialisation: each is set up while the one
- *    before it runs and waits for it before it touches memory.
+ *    The statistics of a step fork onto two streams of the context's own and join back
+ *    (events) on all but the smallest grids, so that the caller's stream sees every call's
+ *    work in order, and a stream capture of a call records the branches as parallel nodes.
+ *    The other kernels of a step are launched with programmatic stream serialisation: each is
+ *    set up while the one before it runs and waits for it before it touches memory.
  *    Problems found on the device (a particle found in no element, an element above the
  *    per-element capacity, a non-finite state) set a device error word; it is read by
  *    pdfx_get_diag() and pdfx_check(), which synchronise the stream.

@@ -863,8 +863,9 @@ __device__ void process_element(const StatsArgs<T>& a, int e, int N, int cap, un
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kStatsThreads) stats_big_kernel(const StatsArgs<T> a, Place at) {
-  sibling_start(at);
+__global__ void __launch_bounds__(kStatsThreads) stats_big_kernel(const StatsArgs<T> a) {
+  chain_wait();
+  chain_go();
   extern __shared__ __align__(16) unsigned char raw[];
   for (int inst = 0; inst < a.K; ++inst) {
   const int32_t* sc = a.scal + 16 * inst;
@@ -885,7 +886,6 @@ __global__ void __launch_bounds__(kStatsThreads) stats_big_kernel(const StatsArg
     process_element(a, e, N, kBigCap, raw, moves);
   }
   }
-  sibling_leave(at);
 }
 
 template <typename T>
@@ -975,13 +975,6 @@ void launch_redistribute(Particles<T> p, Plan& pl, int K, const InstDev<T>* inst
   launch_chained(commit_moves_kernel<T>, grid, 256, 0, s, p, pl, K, np, ne, diag, err);
 }
 
-// Below this many elements the statistics' classes are siblings on one stream, above it branches
-// (four times as many with Fox's projection, whose classes take longer).  us per step, branches /
-// siblings, FP32: 900 elements of 40 particles 42 / 37, of 100 48 / 40; 2,500: 50 / 46, 59 / 56;
-// 4,900: 64 / 64, 83 / 83; 8,100: 80 / 83, 108 / 111; 12,100: 94 / 106, 138 / 150.  Fox, 12,100:
-// 154 / 153, 216 / 208; 20,000: 240 / 242, 362 / 347.  A redistributing step of 1,536 elements of
-// 200: 171 / 147.
-constexpr int kForkElements = 6144;
 // Returns the kernels launched.
 template <typename T>
 int launch_stats(const StatsArgs<T>& a, int num_sms, cudaStream_t s, const SideStreams* side) {
@@ -989,34 +982,35 @@ int launch_stats(const StatsArgs<T>& a, int num_sms, cudaStream_t s, const SideS
   static_assert(5 * 8 * kBigCap + 11 * kBigCap <= 227 * 1024, "large-element tile exceeds shared memory");
   once_on_device(stats_configured<T>,
                  [&] { return allow_shared(reinterpret_cast<const void*>(stats_big_kernel<T>), big); });
-  // a small grid: one launch for every element up to kTileBig, no branches
   // Large elements, one per block and multiprocessor: with all its threads where the mean count
   // lets many exist; else mostly none does, and half the threads start sooner (64 elements of 40
   // particles, FP64: 72 us a step against 74).
   const unsigned nbig = num_sms > 0 ? num_sms : 1;
   const unsigned tbig = a.ne > 0 && a.np / a.ne >= 256 ? kStatsThreads : kStatsThreads / 2;
+  // a small grid: one launch for every element up to kTileBig, no branches
   if (a.cond_mode != 1 && small_grid(a.ne, num_sms)) {
-    launch_chained(stats_big_kernel<T>, nbig, tbig, big, s, a, Place::kFirst);
+    launch_chained(stats_big_kernel<T>, nbig, tbig, big, s, a);
     launch_stats_small<T>(a, s);
     return 2;
   }
   // The tile classes and the large-element kernels take disjoint elements and write disjoint
   // outputs, so that each one's last wave, and its blocks of other classes, which return at
-  // once, can overlap the others' work.  On a large grid they run as parallel branches on the
-  // context's side streams (the 513..768 class and the large-element list's 769..1024 on
-  // side[0]; the class of up to 256 and the large-element kernel on side[1]; the 257..512
-  // class on s) and s then waits for both; below kForkElements they are siblings on s, the
-  // large elements, which take longest, first (1,080 elements of 647 particles on the graded
-  // canyon, some above 1,024: 411 us a step with them last, 390 with them first).
-  if (!side || !side->ok || a.ne < (a.cond_mode == 1 ? 4 : 1) * kForkElements) {
-    launch_chained(stats_big_kernel<T>, nbig, tbig, big, s, a, Place::kFirst);
+  // once, can overlap the others' work: they run as parallel branches on the context's side
+  // streams (the 513..768 class and the large-element list's 769..1024 on side[0]; the class of
+  // up to 256 and the large-element kernel on side[1]; the 257..512 class on s) and s then waits
+  // for both.  us per step as one chain on s / as branches, FP32, eager steps: 924 elements of 100
+  // particles 39 / 45, of 300 64 / 56; 2,520: 60 / 58, 111 / 94; 9,660: 133 / 136, 323 / 291;
+  // 24,420: 263 / 268, 691 / 664; replayed from a graph, where a branch costs no launch, 37 / 36,
+  // 72 / 48; 57 / 49, 111 / 87; 128 / 120, 314 / 281; 258 / 259, 685 / 654.
+  if (!side || !side->ok) {
+    launch_chained(stats_big_kernel<T>, nbig, tbig, big, s, a);
     launch_stats_tiles<T>(a, num_sms, s, s, s);
   } else {
     cudaEventRecord(side->ev[0], s);
     cudaStreamWaitEvent(side->side[0], side->ev[0], 0);
     cudaStreamWaitEvent(side->side[1], side->ev[0], 0);
     launch_stats_tiles<T>(a, num_sms, side->side[1], s, side->side[0]);
-    stats_big_kernel<T><<<nbig, tbig, big, side->side[1]>>>(a, Place::kBranch);
+    stats_big_kernel<T><<<nbig, tbig, big, side->side[1]>>>(a);
     cudaEventRecord(side->ev[1], side->side[0]);
     cudaEventRecord(side->ev[2], side->side[1]);
     cudaStreamWaitEvent(s, side->ev[1], 0);

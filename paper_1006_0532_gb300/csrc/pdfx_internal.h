@@ -236,10 +236,10 @@ constexpr int kRedBlocks = 256;                  // blocks of the solvers' reduc
 constexpr int kPcgActive = eops::S_ACTIVE;
 constexpr int kPcgIters = eops::S_ITERS;
 
-// Two streams and three events for the statistics tiles' size classes on a large grid, which are
-// independent (disjoint elements and outputs) and run as parallel branches of the step: fork
-// after the lists, join before the nodal averages.  Captured into a graph they become parallel
-// nodes.  Created with the context, outside any capture; ok is false when creation failed
+// Two streams and three events for the statistics tiles' size classes, which are independent
+// (disjoint elements and outputs) and run as parallel branches of the step: fork after the
+// lists, join before the nodal averages.  Captured into a graph they become parallel nodes.
+// Created with the context, outside any capture; ok is false when creation failed
 // (the classes then run one after another on the caller's stream).
 struct SideStreams {
   cudaStream_t side[2] = {nullptr, nullptr};
@@ -372,32 +372,6 @@ inline cudaError_t allow_shared(const void* kernel, size_t bytes) {
 // gains nothing and loses nothing.
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-// Siblings: kernels launched one after another that need what ran before the first of them and
-// nothing of one another's.  The first waits as above and only then lets the next start; a
-// later one starts when every block of its predecessor has, so after the first one's wait, when
-// everything before them has completed, and need not wait for its input; a fence at its start
-// keeps it from what the multiprocessor's L1 may still hold of earlier values (0.4% to 1% of a
-// step, or less than nothing: 1,536 elements with redistribution 149 us without, 146.5 with).
-// One of its blocks waits before it ends, so that a kernel's end still implies that of
-// everything launched before it: a block more that does only that (sibling_enter, which then
-// tells it to return), or, in a kernel whose blocks share a list, the last one after its part
-// (sibling_leave).  kBranch: none of this (an ordinary launch in a branch of its own).
-enum class Place : int { kBranch, kFirst, kLater };
-__device__ __forceinline__ void sibling_start(Place at) {
-  if (at == Place::kBranch) return;
-  if (at == Place::kFirst) chain_wait();
-  else asm volatile("fence.acq_rel.gpu;" ::: "memory");
-  chain_go();
-}
-__device__ __forceinline__ bool sibling_enter(Place at) {
-  sibling_start(at);
-  if (at != Place::kLater || blockIdx.x != gridDim.x - 1) return true;
-  chain_wait();
-  return false;
-}
-__device__ __forceinline__ void sibling_leave(Place at) {
-  if (at == Place::kLater && blockIdx.x == gridDim.x - 1) chain_wait();
-}
 
 template <typename... P, typename... A>
 void launch_chained(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, A... args) {
@@ -445,9 +419,8 @@ void launch_stats_small(const StatsArgs<T>& a, cudaStream_t s);   // after the l
 // elements of 100 particles FP32 61.0 / 55.6, FP64 85.3 / 79.9; 400: 63.5 / 59.6, 113.7 /
 // 112.4; 900: 66.2 / 70.4, 170.0 / 166.7; 1,600: 73.5 / 83.9, 211 / 238).
 inline bool small_grid(int32_t ne, int num_sms) { return ne > 0 && ne <= 4 * num_sms; }
-// The tile classes of up to 256, 257..512 and 513..1024 particles: on s_small, s_mid and s_large,
-// or, these being one stream, siblings of the large-element kernel before them (k_bins_f32.cu /
-// k_bins_f64.cu).
+// The tile classes of up to 256, 257..512 and 513..1024 particles: branches on s_small, s_mid and
+// s_large, or, these being one stream, one after another on it (k_bins_f32.cu / k_bins_f64.cu).
 template <typename T>
 void launch_stats_tiles(const StatsArgs<T>& a, int num_sms, cudaStream_t s_small, cudaStream_t s_mid,
                         cudaStream_t s_large);
