@@ -266,13 +266,19 @@ int ensure_particles(Ctx& c, int64_t np) {
   return PDFX_OK;
 }
 
-// Counts per element at zero before an advance or a count: the statistics pass before left
-// them so (its node average clears them), unless there was none or it was cut short.
+// Whether the stream records instead of running.  (The legacy stream cannot be asked while another
+// stream of the process is captured in global mode: what is launched on it then fails by itself.)
+bool is_capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) == cudaSuccess) return st != cudaStreamCaptureStatusNone;
+  cudaGetLastError();
+  return false;
+}
+
+// Counts per element and the brute-force list's length at zero before a pass.
 int clear_counts(Ctx& c, cudaStream_t s) {
-  const bool clear = c.counts_clear;
-  c.counts_clear = false;
-  if (clear) return PDFX_OK;
-  PDFX_CUDA(cudaMemsetAsync(c.err + 1, 0, sizeof(int), s));   // the brute-force list's length
+  if (!c.counts.begin(s != c.gstream && is_capturing(s))) return PDFX_OK;
+  PDFX_CUDA(cudaMemsetAsync(c.err + 1, 0, sizeof(int), s));
   return cerr(cudaMemsetAsync(c.plan.cnt, 0, sizeof(int32_t) * c.ne, s));
 }
 
@@ -356,7 +362,7 @@ int run_statistics(Ctx& c, bool counts_ready, bool allow_moves, bool force_resor
     c.launches++;
   }
   const int rc = cerr(cudaGetLastError());
-  c.counts_clear = rc == PDFX_OK;
+  c.counts.end(rc == PDFX_OK);
   return rc;
 }
 
@@ -855,7 +861,7 @@ int set_grid(Ctx& c, int32_t nn, const double* xy, int32_t ne, const int32_t* tr
   c.h_area2 = g.area2;
   c.fem_ready = false;   // the Eulerian calls rebuild their FEM data for this grid
   c.corr_pending = false;
-  c.counts_clear = false;
+  c.counts = CountsState{};
   c.have_grid = true;
   c.have_fields = false;
   return PDFX_OK;
@@ -879,13 +885,16 @@ int capture_cycle(Ctx& c, double dt, int nsteps) {
   const int64_t done0 = c.steps_done, launches0 = c.launches;
   const int cur0 = c.cur, since0 = c.steps_since_sort;
   const bool prof = c.profiling;
+  const CountsState counts0 = c.counts;
   c.profiling = false;
   PDFX_CUDA(cudaStreamBeginCapture(c.gstream, cudaStreamCaptureModeThreadLocal));
+  c.counts.zero = true;   // as the graph's launch leaves them
   int rc = PDFX_OK;
   for (int k = 0; k < nsteps && rc == PDFX_OK; ++k) rc = do_step<T>(c, dt, c.gstream);
   cudaGraph_t g = nullptr;
   const cudaError_t ec = cudaStreamEndCapture(c.gstream, &g);
   c.profiling = prof;
+  c.counts = counts0;
   const int64_t launches1 = c.launches;
   c.step = step0;
   c.steps_done = done0;
@@ -920,7 +929,9 @@ int do_step_many(Ctx& c, double dt, int32_t nsteps, int use_graph, cudaStream_t 
       if (!c.gexec || c.g_dt != dt || c.g_steps != cycle || c.g_buf != c.pbuf[0] || c.g_np != c.np)
         PDFX_TRY(capture_cycle<T>(c, dt, cycle));
       while (left >= cycle) {
+        PDFX_TRY(clear_counts(c, s));
         PDFX_CUDA(cudaGraphLaunch(c.gexec, s));
+        c.counts.end(true);
         c.step += static_cast<uint32_t>(cycle);
         c.steps_done += cycle;
         c.launches += c.g_launches;

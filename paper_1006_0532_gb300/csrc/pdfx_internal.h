@@ -7,6 +7,7 @@
 #include <cuda_runtime.h>
 
 #include "../../include/pdfx.h"
+#include "counts_state.h"
 #include "eulerian_ops.h"
 #include "once.h"
 #include "pdfx_device.cuh"
@@ -269,7 +270,7 @@ struct Ctx {
   int32_t* ne_list = nullptr;   // [3 ne]
   std::vector<int32_t> h_ne_off, h_ne_list;
   bool have_grid = false;
-  bool counts_clear = false;    // plan.cnt is zero on the stream: the last statistics pass cleared it
+  CountsState counts;           // plan.cnt and the brute-force list's length (err[1])
   // fields
   void* fields = nullptr;       // T[nn][32]
   double* fields64 = nullptr;   // staging for the FP32 conversion
