@@ -366,7 +366,7 @@ __device__ __forceinline__ void update_f64(const Model<double>& M, const Step64&
     const double ddx = rel_x(P, M.src_x, M.src_xl, M.period_x), ddy = rel_y(P, M.src_y, M.src_yl);
     const double Uc2 = q[0] * q[0] + q[1] * q[1] + q[2] * q[2];
     if (m64::bits(Uc2) > 0) {
-      const double a1 = M.cs_r2 * m64::rcbrt(eps) + M.Ct * m64::root((ddx * ddx + ddy * ddy) * m64::rcp(Uc2));
+      const double a1 = M.cs_r2 * m64::rcbrt(eps) + M.Ct * m64::root(m64::quotient(ddx * ddx + ddy * ddy, Uc2));
       if (less(a1, tm)) tm = a1;
     }
     itm = m64::rcp(tm);
