@@ -297,12 +297,16 @@ int  pdfx_step_many(void *ctx, double dt, int32_t nsteps, int use_graph, void *s
 int  pdfx_autotune(void *ctx, double dt, int32_t *adv_block, int32_t *sort_every, void *stream);
 
 /* The launch shapes in use (host outputs, any may be NULL): the advance block size, the
- * re-order period and the binning's size-class split. */
+ * re-order period and the binning's size-class split.  Until a block size is chosen
+ * (pdfx_autotune, pdfx_set_launch_shapes) it is 256, or 128 with fewer particles than eight
+ * waves of blocks. */
 int  pdfx_get_launch_shapes(const void *ctx, int32_t *adv_block, int32_t *sort_every, int32_t *tile_split);
 
 /* Sets the launch shapes (a negative value keeps the current one): the advance block size
  * (128 or 256), the re-order period (0 = never) and the binning's size-class split (0 to
- * 256 particles).  None of them changes a result.  PDFX_ERR_ARG for any other value. */
+ * 256 particles; without effect on the hierarchical bins of a grid of up to four elements per
+ * multiprocessor, which take one launch).  None of them changes a result.  PDFX_ERR_ARG for
+ * any other value. */
 int  pdfx_set_launch_shapes(void *ctx, int32_t adv_block, int32_t sort_every, int32_t tile_split);
 
 /* The form of the conjugate-gradient solves' launch to start from: 0 (default) thread-block

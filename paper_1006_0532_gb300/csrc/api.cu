@@ -409,7 +409,7 @@ int do_step(Ctx& c, double dt, cudaStream_t s, bool coupled = false) {
     a.k1 = key1(c.prm);
     a.inst = c.K > 1 ? static_cast<const InstDev<T>*>(c.inst) : nullptr;
     a.einst = c.K > 1 ? c.einst : nullptr;
-    launch_advance<T>(a, c.num_sms, c.adv_block, s);
+    launch_advance<T>(a, c.num_sms, advance_block(c.adv_block, c.np, c.num_sms), s);
     c.launches += 2;   // the advance and the brute-force search
     c.corr_pending = false;
   }
@@ -1628,7 +1628,7 @@ int pdfx_autotune(void* ctx, double dt, int32_t* adv_block, int32_t* sort_every,
 int pdfx_get_launch_shapes(const void* ctx, int32_t* adv_block, int32_t* sort_every, int32_t* tile_split) {
   const Ctx* c = static_cast<const Ctx*>(ctx);
   if (!c) return PDFX_ERR_ARG;
-  if (adv_block) *adv_block = c->adv_block;
+  if (adv_block) *adv_block = advance_block(c->adv_block, c->np, c->num_sms);
   if (sort_every) *sort_every = c->prm.sort_every;
   if (tile_split) *tile_split = c->tile_split;
   return PDFX_OK;

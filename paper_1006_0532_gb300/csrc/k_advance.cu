@@ -914,10 +914,6 @@ inline unsigned blocks_for(int64_t n, int threads) {
 template <typename T>
 void launch_advance(const AdvanceArgs<T>& a, int num_sms, int block, cudaStream_t s) {
   if (a.np <= 0) return;
-  // fewer blocks than eight waves: the smaller block size whatever was chosen, so that the
-  // last wave is fuller and few particles spread over more schedulers (an FP64 step of 211,600
-  // particles 245 -> 228 us, of 2,560 98 -> 87)
-  if (a.np < static_cast<int64_t>(8) * 1024 * num_sms) block = block < 128 ? block : 128;
   const unsigned bgrid = static_cast<unsigned>(num_sms > 0 ? num_sms : 1);
   const unsigned grid = blocks_for(a.np, block);
   // FP32 advance_kernel: 16 waves of resident blocks, each block over a run of consecutive

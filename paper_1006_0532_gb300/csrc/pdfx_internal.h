@@ -293,7 +293,7 @@ struct Ctx {
   int64_t g_np = -1;
   int64_t g_launches = 0;
   // launch shapes (pdfx_autotune)
-  int adv_block = 256;
+  int adv_block = 0;            // 0: none chosen (advance_block)
   int tile_split = kTileSplit;  // the binning's size-class split (Plan::tile_split)
   int solve_form = kSolveCluster;   // the first form of the solves' launch to try
   // instances of a batch (K = 1: the whole grid)
@@ -392,6 +392,13 @@ void launch_chained(void (*kernel)(P...), unsigned grid, unsigned block, size_t 
 // Kernel launchers (defined in the .cu files).
 template <typename T>
 void launch_advance(const AdvanceArgs<T>& a, int num_sms, int block, cudaStream_t s);   // block <= 256
+// The advance's block size: the caller's or the tuning's (chosen), else 256, or 128 for fewer
+// particles than eight waves of blocks, whose last wave is then fuller and whose particles spread
+// over more schedulers (an FP64 step of 211,600 particles 245 -> 228 us, of 2,560 98 -> 87).
+inline int advance_block(int chosen, int64_t np, int num_sms) {
+  if (chosen > 0) return chosen;
+  return np > 0 && np < static_cast<int64_t>(8) * 1024 * num_sms ? 128 : 256;
+}
 template <typename T>
 void launch_init(Particles<T> p, int32_t ne, int32_t ppe, const ElemGeo<T>* geo,
                  const ElemTopo* topo, const T* fields, Model<T> m, uint32_t k0, uint32_t k1,
