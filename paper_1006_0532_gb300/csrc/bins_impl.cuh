@@ -1707,18 +1707,8 @@ __device__ void element_warp_tile(const StatsArgs<T>& a, WarpTile<T, CAP>& t, in
   }
 }
 
-// On the stream of the kernel before it, or in a branch of its own (an ordinary launch).
-template <typename T>
-void launch_class(void (*kernel)(const StatsArgs<T>), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
-                  const StatsArgs<T>& a, bool branch) {
-  if (branch) kernel<<<grid, block, smem, s>>>(a);
-  else launch_chained(kernel, grid, block, smem, s, a);
-}
-
 template <typename T, int CAP, int WARPS, int CLS>
 __global__ void __launch_bounds__(32 * WARPS) warp_tile_kernel(const StatsArgs<T> a) {
-  chain_wait();
-  chain_go();
   extern __shared__ __align__(16) unsigned char warp_smem[];
   const int warp = threadIdx.x >> 5;
   const int b = static_cast<int>(blockIdx.x) * WARPS + warp;
@@ -1732,9 +1722,9 @@ __global__ void __launch_bounds__(32 * WARPS) warp_tile_kernel(const StatsArgs<T
 template <typename T, int CAP, int WARPS>
 constexpr int warp_tile_smem() { return static_cast<int>(sizeof(WarpTile<T, CAP>)) * WARPS; }
 template <typename T, int CAP, int WARPS, int CLS>
-void launch_warp_tile(const StatsArgs<T>& a, bool branch, cudaStream_t s) {
-  launch_class(warp_tile_kernel<T, CAP, WARPS, CLS>, static_cast<unsigned>((a.ne + WARPS - 1) / WARPS), 32 * WARPS,
-               warp_tile_smem<T, CAP, WARPS>(), s, a, branch);
+void launch_warp_tile(const StatsArgs<T>& a, cudaStream_t s) {
+  warp_tile_kernel<T, CAP, WARPS, CLS>
+      <<<static_cast<unsigned>((a.ne + WARPS - 1) / WARPS), 32 * WARPS, warp_tile_smem<T, CAP, WARPS>(), s>>>(a);
 }
 
 // Residency: the FP32 bucket-rank tiles fit 10 blocks of 128 threads up to 512 particles
@@ -1743,8 +1733,6 @@ void launch_warp_tile(const StatsArgs<T>& a, bool branch, cudaStream_t s) {
 template <typename T, int CAP, int THREADS, int CLS>
 __global__ void __launch_bounds__(THREADS, (sizeof(T) == 4 ? (THREADS == 192 ? 1344 : 1280) : 1024) / THREADS)
     rank_tile_kernel(const StatsArgs<T> a) {
-  chain_wait();
-  chain_go();
   extern __shared__ __align__(16) unsigned char rank_smem[];
   RankTile<T, CAP, THREADS>& t = *reinterpret_cast<RankTile<T, CAP, THREADS>*>(rank_smem);
   int moves = 0;
@@ -1760,8 +1748,6 @@ __global__ void __launch_bounds__(THREADS, (sizeof(T) == 4 ? (THREADS == 192 ? 1
 template <typename T, int CAP, int THREADS, int CLS>
 __global__ void __launch_bounds__(THREADS, (sizeof(T) == 4 ? 1024 : 768) / THREADS)
     rank_list_kernel(const StatsArgs<T> a) {
-  chain_wait();
-  chain_go();
   static_assert(CLS != 0, "the class of the step counter takes a block per entry");
   extern __shared__ __align__(16) unsigned char rank_smem[];
   RankTile<T, CAP, THREADS>& t = *reinterpret_cast<RankTile<T, CAP, THREADS>*>(rank_smem);
@@ -1779,11 +1765,10 @@ __global__ void __launch_bounds__(THREADS, (sizeof(T) == 4 ? 1024 : 768) / THREA
 }
 // few: 0, or the blocks of the list kernel.
 template <typename T, int CAP, int THREADS, int CLS>
-void launch_rank_tile(const StatsArgs<T>& a, int few, bool branch, cudaStream_t s) {
+void launch_rank_tile(const StatsArgs<T>& a, int few, cudaStream_t s) {
   constexpr int smem = static_cast<int>(sizeof(RankTile<T, CAP, THREADS>));
-  const bool list = few > 0 && few < a.ne;
-  launch_class(list ? rank_list_kernel<T, CAP, THREADS, CLS> : rank_tile_kernel<T, CAP, THREADS, CLS>,
-               static_cast<unsigned>(list ? few : a.ne), THREADS, smem, s, a, branch);
+  if (few > 0 && few < a.ne) rank_list_kernel<T, CAP, THREADS, CLS><<<static_cast<unsigned>(few), THREADS, smem, s>>>(a);
+  else rank_tile_kernel<T, CAP, THREADS, CLS><<<static_cast<unsigned>(a.ne), THREADS, smem, s>>>(a);
 }
 
 // The plan's large-element lists (every instance's), entries of up to kTileBig particles, on
@@ -1791,8 +1776,6 @@ void launch_rank_tile(const StatsArgs<T>& a, int few, bool branch, cudaStream_t 
 // stats_big_kernel takes the larger ones.
 template <typename T>
 __global__ void __launch_bounds__(256, (sizeof(T) == 4 ? 1280 : 1024) / 256) rank_big_kernel(const StatsArgs<T> a) {
-  chain_wait();
-  chain_go();
   extern __shared__ __align__(16) unsigned char rank_smem[];
   RankTile<T, kTileBig, 256>& t = *reinterpret_cast<RankTile<T, kTileBig, 256>*>(rank_smem);
   bool used = false;
@@ -1836,8 +1819,6 @@ template <typename T> OncePerDevice rank_configured;
 template <typename T, int CAP, int THREADS, int CLS>
 __global__ void __launch_bounds__(THREADS, (sizeof(T) == 4 ? 1536 : 1024) / THREADS)
     stats_tile_kernel(const StatsArgs<T> a) {
-  chain_wait();
-  chain_go();
   __shared__ Tile<T, CAP> t;
   int moves = 0;
   const int e = tile_element<CLS>(a, blockIdx.x, moves);
@@ -1886,29 +1867,28 @@ void launch_stats_tiles_impl(const StatsArgs<T>& a, int num_sms, cudaStream_t s_
   // class (groups of at most 32 positions are sorted by one warp in registers; the largest
   // class in a tile of 1,024).
   const unsigned grid = static_cast<unsigned>(a.ne);
-  const bool branch = s_small != s_mid;
   if (a.cond_mode == 1) {
-    launch_class(stats_tile_kernel<T, 1024, 256, 1>, grid, 256, 0, s_large, a, branch);
-    launch_class(stats_tile_kernel<T, 512, 128, 2>, grid, 128, 0, s_mid, a, branch);
-    launch_class(stats_tile_kernel<T, 256, 128, 0>, grid, 128, 0, s_small, a, branch);
+    stats_tile_kernel<T, 1024, 256, 1><<<grid, 256, 0, s_large>>>(a);
+    stats_tile_kernel<T, 512, 128, 2><<<grid, 128, 0, s_mid>>>(a);
+    stats_tile_kernel<T, 256, 128, 0><<<grid, 128, 0, s_small>>>(a);
   } else {
     configure_tiles<T>();
     // the classes above the mean count by a factor of two and more hold few elements: over
     // their lists where blocks that return would take 10 us and more (0.5 ns each)
     const int64_t mean = a.np / a.ne;
     const int few = a.ne >= 20000 ? 8 * (num_sms > 0 ? num_sms : 1) : 0;
-    launch_rank_tile<T, 768, 192, 1>(a, mean <= 256 ? few : 0, branch, s_large);
+    launch_rank_tile<T, 768, 192, 1>(a, mean <= 256 ? few : 0, s_large);
     // 769..1024 from the large-element list: 4 blocks per SM
-    launch_class(rank_big_kernel<T>, 4 * (num_sms > 0 ? num_sms : 1), 256, sizeof(RankTile<T, kTileBig, 256>), s_large, a,
-                 branch);
-    launch_warp_tile<T, 256, 4, 0>(a, branch, s_small);
+    rank_big_kernel<T><<<static_cast<unsigned>(4 * (num_sms > 0 ? num_sms : 1)), 256, sizeof(RankTile<T, kTileBig, 256>),
+                         s_large>>>(a);
+    launch_warp_tile<T, 256, 4, 0>(a, s_small);
     // 257..512: a block per element with bucket levels in the FP32 form; where the moment sums
     // are FP64 a warp per element, whose register sort leaves the FP64 pipe the shorter wait
     // (8,100 elements of 300 and 500 particles: FP64 form 350 and 530 us -> 292 and 408, FP64
     // accumulation 326 and 464 -> 244 and 363; FP32 form 216 -> 359 us for 12,100 of 350, its
     // 15 resident warps too few)
-    if (mean > 128 && (sizeof(T) == 8 || a.acc64)) launch_warp_tile<T, 512, 2, 2>(a, branch, s_mid);
-    else launch_rank_tile<T, 512, 128, 2>(a, mean <= 128 ? few : 0, branch, s_mid);
+    if (mean > 128 && (sizeof(T) == 8 || a.acc64)) launch_warp_tile<T, 512, 2, 2>(a, s_mid);
+    else launch_rank_tile<T, 512, 128, 2>(a, mean <= 128 ? few : 0, s_mid);
   }
 }
 
