@@ -46,19 +46,19 @@ SINGLE_POSITION_STEP_BYTES = 98
 # measured, so after any change of the code the bench reports traffic as null until the
 # next capture.
 NCU_RECORDS = {
-    # the benchmark's grid family at 23,908 elements, 11.95M particles (DRAM) and 12,152
-    # elements, 6.08M particles (limiters; FP64 form 1.22M), one GB300
-    "0826dbb91f2d07780009902878957367a0de916e9e0d4930764a3aea45b27082": {
-        "traffic": {"advance": (555.000832e6 + 418.712576e6) / 11.954e6,
-                    "statistics_binning": (86.046464e6 + 0.105216e6 + 0.067328e6 + 0.06656e6 + 330.742016e6
-                                           + 19.325184e6 + 0.067072e6) / 11.954e6},
-        "limiter": {"advance": "instruction issue and latency: 67% issue-active at 48% warps active "
+    # the benchmark's grid and 25.0M particles (DRAM), the same family at 12,152 elements, 6.08M
+    # particles (limiters; FP64 form 1.22M), one GB300
+    "ae1cbf1dc88090f2fe4f39c765dc80f1688abee880a59297d601def1b8a91ec0": {
+        "traffic": {"advance": (1161.894400e6 + 943.964928e6) / 25.0e6,
+                    "statistics_binning": (421.674496e6 + 21.236992e6 + 683.644928e6 + 42.826752e6 + 0.066304e6
+                                           + 0.07296e6 + 0.066816e6) / 25.0e6},
+        "limiter": {"advance": "instruction issue and latency: 65% issue-active at 48% warps active "
                                "(64 registers cap 4 blocks of 256), long-scoreboard stalls first; "
                                "DRAM 23% of peak",
                     "statistics_binning": "instruction issue and shared-memory latency: 67% "
                                           "issue-active (<= 512 class), short-scoreboard stalls "
                                           "first; DRAM 10% of peak"},
-        "f64_advance_fp64_inst_per_particle": (222434799 + 75662106 + 138463756) / 1.2152e6,
+        "f64_advance_fp64_inst_per_particle": (250386490 + 75663837 + 133604547) / 1.2152e6,
     },
 }
 STAGES = ["advance", "plan", "lists", "redistribute", "statistics_binning", "node_average"]

@@ -1364,8 +1364,9 @@ __device__ void element_rank_tile(const StatsArgs<T>& a, RankTile<T, CAP, THREAD
 // Bound by instruction issue (75% active).  A block of 128 threads per element with bucket
 // levels, as the larger classes have, took 7,800 warp instructions for an element of 100
 // particles, most of them barriers', tables' and partly filled warps'; this takes about a
-// third.  The statistics stage of 200,000 such elements: 1,971 -> 691 us (with the classes
-// above launched over their lists), of 50,000 in FP64 1,183 -> 631 us.
+// third.  The statistics stage, mean of 32 steps: 200,000 such elements (the street canyon)
+// 1,964 -> 765 us (with the classes above launched over their lists), of 50,000 in FP64 1,133 ->
+// 674 us.
 // ---------------------------------------------------------------------------------------
 template <int CAP> struct WarpIndex { using type = uint16_t; };
 template <> struct WarpIndex<256> { using type = uint8_t; };

@@ -312,10 +312,11 @@ static_assert(kDiagHopHist0 < 32, "an event's bit is its diagnostic's slot");
 // same equations as the FP32 form's below, arranged for the fewest FP64 operations: at 64
 // cycles of a scheduler's FP64 pipe each they are the kernel's time.  C0 enters only as
 // C0 eps = -2/3 wp_ij <u_i u_j> / k; time-step factors are formed once; comparisons are on
-// the bits; the elementary functions are math64.h's.  The kernel takes 396 FP64 warp
-// instructions per 32 particles, its pipe 88% busy: 3.6 ms for 5.0M particles on the
-// 50,000-triangle channel, against 6.7 ms with the library's functions, divisions, edge
-// vectors formed per particle and comparisons in FP64.
+// the bits; the elementary functions are math64.h's.  The kernel takes 415 FP64 warp
+// instructions per 32 particles (378 additions, products and fused products a particle, and a
+// few conversions), its pipe 88% busy: 3.8 ms for 5.0M particles on the 50,000-triangle channel,
+// against 6.7 ms with the library's functions, divisions, edge vectors formed per particle and
+// comparisons in FP64.
 //
 // A coupled step does not take it (PLAIN): its pressure solve stops at the caller's tolerance
 // after some thousand conjugate-gradient iterations, which carry a change of the load's last
