@@ -23,7 +23,7 @@
  *  - Device work is enqueued on the caller's CUDA stream (a cudaStream_t passed as void*,
  *    NULL = the legacy default stream) and is asynchronous unless a call says otherwise.
  *    The statistics of a step fork onto two streams of the context's own and join back
- *    (events) on all but the smallest grids, so that the caller's stream sees every call's
+ *    (events) on all but small and medium grids, so that the caller's stream sees every call's
  *    work in order, and a stream capture of a call records the branches as parallel nodes.
  *    The other kernels of a step are launched with programmatic stream serialisation: each is
  *    set up while the one before it runs and waits for it before it touches memory.

@@ -1812,6 +1812,43 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 ? 1280 : 1024) / 256) sma
   if (N <= kTileBig) element_rank_tile<T, kTileBig, 256>(a, t, e, N, moves);
 }
 
+// The classes of a medium grid in one launch, a block's place in the plan's lists choosing its
+// part, the larger elements first: the large-element list and the two upper classes a block per
+// element on the bucket-rank tile of kTileBig, then the class up to the split a warp per element
+// (61 KB of shared memory, 3 blocks per SM).  The last wave of one class overlaps the next one's
+// first blocks without a fork and a join (medium_grid states what it measured).
+constexpr int kMediumWarps = 8;
+template <typename T>
+__global__ void __launch_bounds__(32 * kMediumWarps, 3) medium_grid_kernel(const StatsArgs<T> a) {
+  chain_wait();
+  chain_go();
+  extern __shared__ __align__(16) unsigned char medium_smem[];
+  const int32_t* sc = a.scal;
+  const int nbig = sc[3], n1 = sc[7], n2 = sc[8], moves = sc[0] > 0;
+  const int b = blockIdx.x;
+  if (b == 0 && threadIdx.x == 0 && a.step_inc) atomicAdd(a.step_inc, 1u);
+  if (b < nbig + n1 + n2) {
+    const int e = b < nbig ? a.big_list[b] : b < nbig + n1 ? a.tiles[a.ne - 1 - (b - nbig)] : a.tiles_mid[b - nbig - n1];
+    const int N = moves ? a.fin[e] : a.cnt[e];
+    if (N <= kTileBig)
+      element_rank_tile<T, kTileBig, 32 * kMediumWarps>(
+          a, *reinterpret_cast<RankTile<T, kTileBig, 32 * kMediumWarps>*>(medium_smem), e, N, moves);
+    return;
+  }
+  const int warp = threadIdx.x >> 5;
+  const int k = (b - nbig - n1 - n2) * kMediumWarps + warp;
+  if (k >= sc[6]) return;
+  const int e = a.tiles[k];
+  const int N = moves ? a.fin[e] : a.cnt[e];
+  element_warp_tile<T, kTileSplit>(a, reinterpret_cast<WarpTile<T, kTileSplit>*>(medium_smem)[warp], e, min(N, kTileSplit), moves);
+}
+template <typename T>
+constexpr size_t medium_smem_bytes() {
+  return sizeof(RankTile<T, kTileBig, 32 * kMediumWarps>) > sizeof(WarpTile<T, kTileSplit>) * kMediumWarps
+             ? sizeof(RankTile<T, kTileBig, 32 * kMediumWarps>)
+             : sizeof(WarpTile<T, kTileSplit>) * kMediumWarps;
+}
+
 template <typename T> OncePerDevice rank_configured;
 
 // One block per entry of one size class of the plan's tile lists (tile_element); the grid
@@ -1841,6 +1878,7 @@ void configure_tiles() {
     };
     allow(reinterpret_cast<const void*>(small_grid_kernel<T>), big);
     allow(reinterpret_cast<const void*>(rank_big_kernel<T>), big);
+    if constexpr (sizeof(T) == 4) allow(reinterpret_cast<const void*>(medium_grid_kernel<T>), medium_smem_bytes<T>());
     allow(reinterpret_cast<const void*>(rank_tile_kernel<T, 768, 192, 1>), sizeof(RankTile<T, 768, 192>));
     allow(reinterpret_cast<const void*>(rank_list_kernel<T, 768, 192, 1>), sizeof(RankTile<T, 768, 192>));
     allow(reinterpret_cast<const void*>(rank_tile_kernel<T, 512, 128, 2>), sizeof(RankTile<T, 512, 128>));
@@ -1852,8 +1890,10 @@ void configure_tiles() {
 }
 
 template <typename T>
-void launch_stats_small_impl(const StatsArgs<T>& a, cudaStream_t s) {
+void launch_stats_small_impl(const StatsArgs<T>& a, bool medium, cudaStream_t s) {
   configure_tiles<T>();
+  if constexpr (sizeof(T) == 4)
+    if (medium) return launch_chained(medium_grid_kernel<T>, a.ne, 32 * kMediumWarps, medium_smem_bytes<T>(), s, a);
   launch_chained(small_grid_kernel<T>, a.ne, 256, sizeof(RankTile<T, kTileBig, 256>), s, a);
 }
 

@@ -10,8 +10,8 @@ void launch_stats_tiles<float>(const StatsArgs<float>& a, int num_sms, cudaStrea
 }
 
 template <>
-void launch_stats_small<float>(const StatsArgs<float>& a, cudaStream_t s) {
-  launch_stats_small_impl<float>(a, s);
+void launch_stats_small<float>(const StatsArgs<float>& a, bool medium, cudaStream_t s) {
+  launch_stats_small_impl<float>(a, medium, s);
 }
 
 }  // namespace pdfx

@@ -10,8 +10,8 @@ void launch_stats_tiles<double>(const StatsArgs<double>& a, int num_sms, cudaStr
 }
 
 template <>
-void launch_stats_small<double>(const StatsArgs<double>& a, cudaStream_t s) {
-  launch_stats_small_impl<double>(a, s);
+void launch_stats_small<double>(const StatsArgs<double>& a, bool medium, cudaStream_t s) {
+  launch_stats_small_impl<double>(a, medium, s);
 }
 
 }  // namespace pdfx

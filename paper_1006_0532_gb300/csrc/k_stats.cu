@@ -975,6 +975,19 @@ void launch_redistribute(Particles<T> p, Plan& pl, int K, const InstDev<T>* inst
   launch_chained(commit_moves_kernel<T>, grid, 256, 0, s, p, pl, K, np, ne, diag, err);
 }
 
+// A grid of some thousand small elements takes its classes in one launch with the step's other
+// kernels' early set-up, where the branches' fork and join cost more than a class's own tile and
+// block size give.  FP32 sums only: with FP64 sums the tiles take too long for it to matter.  us per
+// eager step, branches / one launch: 924 elements of 100 particles 45 / 40, 1,512: 48 / 43, 2,520:
+// 59 / 50, 5,100: 86 / 75; of 200 53 / 50, 62 / 54, 76 / 76, 116 / 113; of 220 65 / 64 (1,512), 78 / 79,
+// 123 / 130; of 300 57 / 59, 69 / 78, 93 / 112, 170 / 208.  A redistributing step of 1,536 elements
+// of 200: 169 / 150.
+constexpr int kMediumElements = 6144, kMediumMean = 208;
+template <typename T>
+bool medium_grid(const StatsArgs<T>& a) {
+  return sizeof(T) == 4 && !a.acc64 && !a.einst && a.ne < kMediumElements && a.np <= static_cast<int64_t>(kMediumMean) * a.ne;
+}
+
 // Returns the kernels launched.
 template <typename T>
 int launch_stats(const StatsArgs<T>& a, int num_sms, cudaStream_t s, const SideStreams* side) {
@@ -987,10 +1000,12 @@ int launch_stats(const StatsArgs<T>& a, int num_sms, cudaStream_t s, const SideS
   // particles, FP64: 72 us a step against 74).
   const unsigned nbig = num_sms > 0 ? num_sms : 1;
   const unsigned tbig = a.ne > 0 && a.np / a.ne >= 256 ? kStatsThreads : kStatsThreads / 2;
-  // a small grid: one launch for every element up to kTileBig, no branches
-  if (a.cond_mode != 1 && small_grid(a.ne, num_sms)) {
+  // a small grid, or a medium one: one launch for every element up to kTileBig, no branches
+  const bool small = a.cond_mode != 1 && small_grid(a.ne, num_sms);
+  const bool medium = a.cond_mode != 1 && !small && medium_grid<T>(a);
+  if (small || medium) {
     launch_chained(stats_big_kernel<T>, nbig, tbig, big, s, a);
-    launch_stats_small<T>(a, s);
+    launch_stats_small<T>(a, medium, s);
     return 2;
   }
   // The tile classes and the large-element kernels take disjoint elements and write disjoint

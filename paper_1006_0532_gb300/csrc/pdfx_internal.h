@@ -420,9 +420,10 @@ void launch_redistribute(Particles<T> p, Plan& pl, int K, const InstDev<T>* inst
                          int num_sms, unsigned long long* diag, int* err, cudaStream_t s);
 template <typename T>
 int launch_stats(const StatsArgs<T>& a, int num_sms, cudaStream_t s, const SideStreams* side);   // kernels launched
-// The hierarchical bins of a small grid in one launch (elements of up to kTileBig particles).
+// The hierarchical bins of a small or (FP32 sums) a medium grid in one launch (elements of up to
+// kTileBig particles).
 template <typename T>
-void launch_stats_small(const StatsArgs<T>& a, cudaStream_t s);   // after the large-element kernel
+void launch_stats_small(const StatsArgs<T>& a, bool medium, cudaStream_t s);   // after the large-element kernel
 // A grid of up to four elements per multiprocessor (us per step, classes / one launch: 64
 // elements of 100 particles FP32 61.0 / 55.6, FP64 85.3 / 79.9; 400: 63.5 / 59.6, 113.7 /
 // 112.4; 900: 66.2 / 70.4, 170.0 / 166.7; 1,600: 73.5 / 83.9, 211 / 238).
