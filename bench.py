@@ -48,10 +48,10 @@ SINGLE_POSITION_STEP_BYTES = 98
 NCU_RECORDS = {
     # the benchmark's grid and 25.0M particles (DRAM), the same family at 12,152 elements, 6.08M
     # particles (limiters; FP64 form 1.22M), one GB300
-    "ae1cbf1dc88090f2fe4f39c765dc80f1688abee880a59297d601def1b8a91ec0": {
-        "traffic": {"advance": (1161.894400e6 + 943.964928e6) / 25.0e6,
-                    "statistics_binning": (421.674496e6 + 21.236992e6 + 683.644928e6 + 42.826752e6 + 0.066304e6
-                                           + 0.07296e6 + 0.066816e6) / 25.0e6},
+    "a610e667265cd613ff161ecee1e1f376e53258064c1ae8857bd680e3921fc466": {
+        "traffic": {"advance": (1161.966848e6 + 943.855616e6) / 25.0e6,
+                    "statistics_binning": (421.678080e6 + 21.252096e6 + 683.652864e6 + 43.142656e6 + 0.066304e6
+                                           + 0.072704e6 + 0.067328e6) / 25.0e6},
         "limiter": {"advance": "instruction issue and latency: 65% issue-active at 48% warps active "
                                "(64 registers cap 4 blocks of 256), long-scoreboard stalls first; "
                                "DRAM 23% of peak",

@@ -1,9 +1,10 @@
 // Per-element statistics and conditional means for elements of up to 768 particles from the
-// plan's tile lists (three size classes, launched as parallel stream branches), and of
-// 769..1024 from the plan's large-element list; larger elements go through the block kernel
-// in k_stats.cu.  The chunk-sort tile below serves every class of Fox's projection; for the
-// hierarchical bins the class up to the split takes the warp tile at the end, the others the
-// bucket-rank tile (a block per element) or, for FP64 sums, the warp tile.
+// plan's tile lists (three size classes, launched as parallel stream branches, on small and
+// medium grids as one launch), and of 769..1024 from the plan's large-element list; larger
+// elements go through the block kernel in k_stats.cu.  The chunk-sort tile below serves every
+// class of Fox's projection; for the hierarchical bins the class up to the split takes the warp
+// tile at the end, the others the bucket-rank tile (a block per element) or, for FP64 sums, the
+// warp tile.
 //
 // Sect. 3.5 / Appendix A: the element's particles are sorted by (u, id); the level-1 groups
 // (positions with equal floor(g1 p / N)) are sorted by (v, id), the level-2 groups by
