@@ -8,8 +8,8 @@ namespace pdfx {
 // on the host: not before the first pass, and not after one that was cut short.  What a capture
 // records has not run, so it changes nothing of this; and its graph may be replayed after
 // anything, so a captured pass clears for itself.  (The library's own graph of a re-order cycle
-// holds no clears: its launch goes through begin() and end() like a pass, its capture through
-// neither's knowledge.)
+// holds no clears: its launch goes through begin() and end() like a pass, and what its capture does
+// to this state is undone.)
 struct CountsState {
   bool zero = false;
 
